@@ -18,6 +18,8 @@
 //     written to global memory with 16-byte accesses.
 // The CTA is synchronised with two block barriers per row and one mbarrier wait (bounded) for the accumulator;
 // several CTAs share an SM and fill each other's gaps.
+#include <limits.h>
+
 #include <algorithm>
 #include <stdio.h>
 #include <stdlib.h>
@@ -82,8 +84,26 @@ __device__ __forceinline__ uint32_t load_pixel(const uint8_t *x, uint32_t off, u
     return word;
 }
 
-// CPR: 16-byte chunks per output pixel when known at compile time (0: read it from the parameters).
-template <int CPR, bool POOL, bool SIGNED, bool FAST>
+// The one or two K slices of a row pair.  Executed by a whole warp, one lane issues: see mma_commit_elect().
+__device__ __forceinline__ void stem_mma_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, const StemParams &p, uint32_t b_slice,
+                                              uint32_t accumulate) {
+    if (p.slices == 2)
+        asm volatile("{\n\t.reg .pred e, p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\telect.sync _|e, 0xffffffff;\n\t"
+                     "setp.ne.b32 p, %7, 0;\n\tsetp.eq.b32 t, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t"
+                     "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, p;\n\t"
+                     "add.u32 x, %1, 2;\n\tadd.u32 y, %2, %5;\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %4};\n\t"
+                     "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, t;\n\t}" ::"r"(d_tmem),
+                     "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(b_slice), "r"(p.idesc), "r"(accumulate)
+                     : "memory");
+    else
+        asm volatile("{\n\t.reg .pred e, p;\n\t.reg .b64 a, b;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+                     "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t"
+                     "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
+                     "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(p.idesc), "r"(accumulate)
+                     : "memory");
+}
+
+template <bool POOL, bool SIGNED, bool FAST>
 __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemParams p, const int grid_units_total) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t acc_bar[2];
@@ -91,7 +111,7 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
     __shared__ int abort_flag;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cpr = CPR ? CPR : p.cpr;
+    const int cpr = p.cpr;
     const uint32_t c_out = (uint32_t)cpr * 16u;
     const int k_bytes = p.kh2 * p.slices * 32;
     const uint32_t w_bytes = (uint32_t)k_bytes * c_out;
@@ -175,8 +195,7 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
         for (int i = 0; i < 2; ++i)
             if (cell_on[i]) line[threadIdx.x + i * STEM_THREADS] = cell[i];
     };
-    // issue the MMAs of output row oy into accumulator kk & 1 (one thread).  A lone thread pays for every instruction
-    // it executes, so the descriptors are assembled from 32-bit words inside one asm block per row pair.
+    // issue the MMAs of output row oy into accumulator kk & 1 (a whole warp)
     const uint32_t a_lo0 = p.a_desc_lbo_sbo | ((pair_base & 0x3ffffu) >> 4), b_lo0 = p.b_desc_lbo_sbo | ((smem_base & 0x3ffffu) >> 4);
     const uint32_t b_slice = 2u * c_out;                 // 16-byte units between the K slices of the weights
     auto issue_row = [&](int oy, int kk) {
@@ -187,23 +206,10 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
             const int pr = oy - p.top + j;
             if (pr < 0 || pr >= p.hp) continue;          // rows above / below the image contribute nothing
             const uint32_t a_lo = a_lo0 + (uint32_t)(pr & (STEM_PAIR_SLOTS - 1)) * (STEM_SLOT_BYTES / 16);
-            if (p.slices == 2)
-                asm volatile("{\n\t.reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %7, 0;\n\t"
-                             "setp.eq.b32 t, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t"
-                             "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, p;\n\t"
-                             "add.u32 x, %1, 2;\n\tadd.u32 y, %2, %5;\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %4};\n\t"
-                             "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, t;\n\t}" ::"r"(d_tmem),
-                             "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(b_slice), "r"(p.idesc), "r"(accumulate)
-                             : "memory");
-            else
-                asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %6, 0;\n\t"
-                             "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t"
-                             "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
-                             "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(p.idesc), "r"(accumulate)
-                             : "memory");
+            stem_mma_pair(d_tmem, a_lo, b_lo, p, b_slice, accumulate);
             accumulate = 1;
         }
-        mma_commit(smem_u32(&acc_bar[kk & 1]));
+        mma_commit_elect(smem_u32(&acc_bar[kk & 1]));
     };
 
     for (int u = u_begin; u < u_end;) {
@@ -228,11 +234,8 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
         if (warp == STEM_EPI_WARPS) {
-            if (lane == 0) {
-                tc_fence_after();
-                issue_row(oy_first, k);
-            }
-            __syncwarp();
+            tc_fence_after();
+            issue_row(oy_first, k);
         }
 
         for (int oy = oy_first; oy <= oy_last; ++oy, ++k) {
@@ -254,11 +257,10 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
             const bool opens = oy == 0;
             const int py = oy >> 1;
             if (warp == STEM_EPI_WARPS) {
-                if (lane == 0 && oy + 1 <= oy_last) {
+                if (oy + 1 <= oy_last) {
                     tc_fence_after();
                     issue_row(oy + 1, k + 1);
                 }
-                __syncwarp();
             } else {
                 // ---- epilogue of row oy: thread = output pixel, 16 channels per accumulator load
                 // the accumulator is usually a few hundred cycles away: sleep on the barrier (the hardware wakes the
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
                     const uint32_t cur = rows_base + (POOL ? (uint32_t)(py & 1) * row_bytes : 0u) + px_off;
                     const uint32_t nxt = rows_base + (uint32_t)((py + 1) & 1) * row_bytes + px_off;
 #pragma unroll
-                    for (int ci = 0; ci < (CPR ? (CPR + 1) / 2 : 8); ++ci) {
+                    for (int ci = 0; ci < 8; ++ci) {
                         const int ch = ch0 + ci;
                         if (ch >= ch1) break;
                         int v[16];
@@ -358,10 +360,375 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
     }
 }
 
+
+// ----------------------------------------------------------------------------- layers of at most 64 channels
+
+// The same layer with its roles on warps of their own, for up to 64 output channels (the stems of the networks here; wider
+// ones keep the kernel above, whose accumulators fit tensor memory twice).  Three warps pack image lines, one warp issues the
+// MMAs, eight warps convert; every hand-over is an mbarrier, so nobody waits at a block-wide barrier and three different
+// steps are packed, multiplied and converted at once.
+//   * A step is a pair of output rows (2r, 2r + 1).  Their windows overlap, so they are ONE multiplication with 2 c_out columns:
+//     the weights of row 2r + 1 are those of row 2r one row pair further down (zeros where a row does not reach).  For the
+//     7 x 7 stem that is 10 instructions of 128 columns instead of 16 of 64, which are bound by the tensor pipe's 50 cycles
+//     per instruction, and half of the hand-overs.
+//   * The rounding shift and the clip are monotone, so the pooling maximum over the three rows is taken on the 32-bit sums
+//     (one three-operand maximum per value; the odd row that two pooled rows share stays in registers) and only one value
+//     in two is requantised.
+//   * The maximum over three columns works on 16-bit lanes of packed bytes: the high bytes of a lane decide whatever lies
+//     below them, so a word costs two three-operand maxima and three shifts.
+//   * Without a pool a thread stores its pixel's channels straight from registers.
+// Measured (224 x 224 images, batch 256, B200): 7 x 7 to 64 channels with the pool 140 -> 82 us, 3 x 3 to 32 channels without a
+// pool 105 -> 62 us; one image 21 -> 17 us.  The pooling conversion is what bounds the first (its warps wait 10 % of the time;
+// the instruction slots are 55 % used), the packing of the lines the second (a fourth packing warp: no change).
+constexpr int ROWS_EPI_WARPS = 8;
+constexpr int ROWS_PACK_WARPS = 3;
+constexpr int ROWS_MMA_WARP = ROWS_EPI_WARPS + ROWS_PACK_WARPS;
+constexpr int ROWS_THREADS = 32 * (ROWS_MMA_WARP + 1);
+constexpr int ROWS_LINES = 16;                  // ring of packed row pairs
+constexpr int ROWS_AHEAD = 4;                   // steps the packing may run ahead of the MMAs: a window of at most 8 pairs plus
+                                                // three times two more lines fit the ring
+constexpr int ROWS_ACCS = 2;
+constexpr int ROWS_CELLS = (STEM_MAX_CELLS + 32 * ROWS_PACK_WARPS - 1) / (32 * ROWS_PACK_WARPS);       // of a line, per thread
+
+// Bytewise maximum of three words.
+template <bool SIGNED>
+__device__ __forceinline__ uint32_t max3_bytes(uint32_t a, uint32_t b, uint32_t c) {
+    const uint32_t hi = SIGNED ? __vimax3_s16x2(a, b, c) : __vimax3_u16x2(a, b, c);
+    const uint32_t lo = SIGNED ? __vimax3_s16x2(a << 8, b << 8, c << 8) : __vimax3_u16x2(a << 8, b << 8, c << 8);
+    return __byte_perm(hi, lo, 0x3715);
+}
+
+// CH: 16-byte chunks per pixel this instantiation has registers for (2 or 4; p.cpr <= CH).
+template <int CH, bool POOL, bool SIGNED, bool FAST>
+__global__ void __launch_bounds__(ROWS_THREADS, 2) f8_stem_rows_tc_kernel(const StemParams p, const int units_total) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) uint64_t line_bars[ROWS_AHEAD];      // the lines a step adds have been packed
+    __shared__ __align__(8) uint64_t done_bars[ROWS_AHEAD];      // a step's MMAs have completed
+    __shared__ __align__(8) uint64_t free_bars[ROWS_ACCS];       // an accumulator has been read
+    __shared__ uint32_t tmem_base_slot;
+    __shared__ int abort_flag;
+
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
+    const uint32_t c_out = (uint32_t)p.cpr * 16u;
+    const uint32_t w_bytes = (uint32_t)((p.kh2 + 1) * p.slices * 32) * 2u * c_out;
+    const uint32_t row_bytes = 128u * c_out;
+    const uint32_t smem_base = smem_u32(smem);
+    const uint32_t line_base = smem_base + w_bytes;
+    const uint32_t rows_base = line_base + ROWS_LINES * STEM_SLOT_BYTES;       // POOL: two rows of column-wise maxima
+    const uint32_t bias_base = rows_base + (POOL ? 2 * row_bytes : 0u);
+    uint8_t *const line_ptr = smem + w_bytes;
+
+    {
+        uint4 *z = (uint4 *)line_ptr;     // cells past the image are never written again: they stay zero
+        for (int i = threadIdx.x; i < ROWS_LINES * STEM_SLOT_BYTES / 16; i += ROWS_THREADS) z[i] = make_uint4(0, 0, 0, 0);
+        const uint4 *wg = (const uint4 *)p.wk;
+        uint4 *ws = (uint4 *)smem;
+        // [K / 16][2 c_out][16]: columns c_out.. are the same weights one row pair later
+        const int pair_chunks = p.slices * 2, last_chunk = p.kh2 * pair_chunks;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < (int)(w_bytes / 16); i += ROWS_THREADS) {
+            const int kc = i / (2 * (int)c_out), n = i - kc * 2 * (int)c_out;
+            const int src = n < (int)c_out ? kc : kc - pair_chunks;
+            ws[i] = src >= 0 && src < last_chunk ? __ldg(wg + src * (int)c_out + (n < (int)c_out ? n : n - (int)c_out)) : make_uint4(0, 0, 0, 0);
+        }
+        int *bs = (int *)(smem + (bias_base - smem_base));
+        const int rnd = 1 << (p.s - 1);
+        for (int i = threadIdx.x; i < (int)c_out; i += ROWS_THREADS) bs[i] = (p.bias ? __ldg(p.bias + i) : 0) + rnd;
+    }
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        for (int i = 0; i < ROWS_AHEAD; ++i) {
+            mbar_init(smem_u32(&line_bars[i]), ROWS_PACK_WARPS);
+            mbar_init(smem_u32(&done_bars[i]), 1);
+        }
+        for (int i = 0; i < ROWS_ACCS; ++i) mbar_init(smem_u32(&free_bars[i]), ROWS_EPI_WARPS);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == ROWS_MMA_WARP) tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)(ROWS_ACCS * p.acc_cols));
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");     // weights and zeroed lines: read by the tensor core
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = uniform(tmem_base_slot);
+    grid_launch_dependents();
+
+    const WaitCtx wc = make_wait_ctx(&abort_flag, p.status, p.wait_limit);
+    const int tagbits = p.tag << 8;
+    const long long total = units_total;
+    // a unit is a pair of convolution rows (2r, 2r + 1), with a pool the pooled row r; every role walks the same list
+    const int u_begin = (int)(total * blockIdx.x / gridDim.x), u_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    const uint32_t line_bar = smem_u32(line_bars), done_bar = smem_u32(done_bars), free_bar = smem_u32(free_bars);
+    int k = 0;                       // steps so far: barrier k % ROWS_AHEAD, accumulator k % ROWS_ACCS
+    bool ok = true;
+
+    if (warp >= ROWS_EPI_WARPS && warp < ROWS_MMA_WARP) {
+        // ------------------------------------------------------------------ packing
+        const int pt = threadIdx.x - 32 * ROWS_EPI_WARPS;
+        const uint32_t img_row_bytes = (uint32_t)p.w * p.c;
+        const uint32_t last_word = (uint32_t)p.n * p.h * img_row_bytes - 4u;
+        uint32_t cell_off[ROWS_CELLS], cell_mask[ROWS_CELLS];      // byte offset inside an image row; mask of the channel bytes
+        bool cell_on[ROWS_CELLS];
+#pragma unroll
+        for (int i = 0; i < ROWS_CELLS; ++i) {
+            const int col = pt + i * 32 * ROWS_PACK_WARPS, iw = col - p.left;
+            const bool px = col < p.ncell && iw >= 0 && iw < p.w;   // else zero padding
+            cell_on[i] = col < p.ncell;
+            cell_off[i] = px ? (uint32_t)iw * p.c : 0u;
+            cell_mask[i] = px ? 0xffffffffu >> (32 - 8 * p.c) : 0u;
+        }
+        grid_dependency_wait();        // the image may belong to earlier work in the stream
+        // The words of a line's pixels, all requested before the first is used (a load behind a branch of its own, with its
+        // use in the same branch, waits for memory once per cell: 4000 cycles a line instead of 900); combined when the line
+        // is stored.
+        uint32_t raw[2][ROWS_CELLS][2][FAST ? 2 : 1];        // two lines at a time
+        uint32_t row_off[2][2] = {{0u, 0u}, {0u, 0u}}, second_mask[2] = {0u, 0u};
+        auto load_lines = [&](int img, int pr0) {
+#pragma unroll
+            for (int l = 0; l < 2; ++l) {
+                const int pr = min(pr0 + l, p.hp - 1);            // (a line past the image is not stored)
+                row_off[l][0] = ((uint32_t)img * p.h + 2u * pr) * img_row_bytes;
+                second_mask[l] = 2 * pr + 1 < p.h ? 0xffffffffu : 0u;
+                row_off[l][1] = row_off[l][0] + (img_row_bytes & second_mask[l]);
+#pragma unroll
+                for (int i = 0; i < ROWS_CELLS; ++i)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const uint32_t off = row_off[l][e] + cell_off[i];
+                        if (FAST) {      // two aligned words around the pixel, none beyond the tensor's last one
+                            raw[l][i][e][0] = ldg32(p.x + (off & ~3u));
+                            raw[l][i][e][FAST ? 1 : 0] = ldg32(p.x + min((off & ~3u) + 4u, last_word));
+                        } else {
+                            raw[l][i][e][0] = load_pixel<false>(p.x, off, last_word, p.c);
+                        }
+                    }
+            }
+        };
+        auto line_cell = [&](int l, int i) {
+            uint32_t v[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                v[e] = raw[l][i][e][0];
+                if (FAST) v[e] = __funnelshift_r(v[e], raw[l][i][e][FAST ? 1 : 0], ((row_off[l][e] + cell_off[i]) & 3u) * 8u);
+                v[e] &= cell_mask[i];
+            }
+            return make_uint2(v[0], v[1] & second_mask[l]);
+        };
+        int line = 0;                  // lines packed so far: slot line % ROWS_LINES
+        for (int u = u_begin; ok && u < u_end;) {
+            const int img = u / p.rows_per_img, r0 = u - img * p.rows_per_img;
+            const int r1 = min(p.rows_per_img, r0 + (u_end - u));
+            u += r1 - r0;
+            const int first = POOL && r0 > 0 ? r0 - 1 : r0;          // (pool: the row above the first pooled row)
+            int pr = max(0, 2 * first - p.top);                      // next pair to pack
+            load_lines(img, pr);
+            for (int r = first; r < r1; ++r, ++k) {
+                // a new image does not share lines with the steps before it: let those finish, so that the ring holds one
+                // image's window at a time
+                const int need = r == first ? k - 1 : k - ROWS_AHEAD;
+                bool got = true;
+                if (need >= 0) got = mbar_wait(done_bar + 8 * (need % ROWS_AHEAD), (uint32_t)(need / ROWS_AHEAD) & 1u, wc, tagbits | 121);
+                if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+                const int pr_end = min(p.hp, 2 * r + 1 - p.top + p.kh2);
+                while (pr < pr_end) {
+#pragma unroll
+                    for (int l = 0; l < 2; ++l)
+                        if (pr + l < pr_end) {
+                            uint2 *dst = (uint2 *)(line_ptr + ((line + l) & (ROWS_LINES - 1)) * STEM_SLOT_BYTES) + pt;
+#pragma unroll
+                            for (int i = 0; i < ROWS_CELLS; ++i)
+                                if (cell_on[i]) dst[i * 32 * ROWS_PACK_WARPS] = line_cell(l, i);
+                        }
+                    const int n = min(2, pr_end - pr);
+                    line += n;
+                    pr += n;
+                    if (pr < p.hp) load_lines(img, pr);              // in flight until their turn
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(line_bar + 8 * (k % ROWS_AHEAD));
+            }
+        }
+    } else if (warp == ROWS_MMA_WARP) {
+        // ------------------------------------------------------------------ MMA issue: the whole warp runs the loop, one lane issues
+        {
+            const uint32_t a_lo0 = p.a_desc_lbo_sbo | ((line_base & 0x3ffffu) >> 4), b_lo0 = p.b_desc_lbo_sbo | ((smem_base & 0x3ffffu) >> 4);
+            const uint32_t b_slice = 4u * c_out;                 // 16-byte units between the K slices of the weights
+            int line = 0;
+            for (int u = u_begin; ok && u < u_end;) {
+                const int img = u / p.rows_per_img, r0 = u - img * p.rows_per_img;
+                const int r1 = min(p.rows_per_img, r0 + (u_end - u));
+                u += r1 - r0;
+                const int first = POOL && r0 > 0 ? r0 - 1 : r0;
+                const int pr_first = max(0, 2 * first - p.top);
+                const int line_of_pr = line - pr_first;              // ring index of pair 0 of this image (may be negative)
+                for (int r = first; r < r1; ++r, ++k) {
+                    bool got = true;
+                    if (k >= ROWS_ACCS) got = mbar_wait(free_bar + 8 * (k % ROWS_ACCS), (uint32_t)(k / ROWS_ACCS - 1) & 1u, wc, tagbits | 122);
+                    got = got && mbar_wait(line_bar + 8 * (k % ROWS_AHEAD), (uint32_t)(k / ROWS_AHEAD) & 1u, wc, tagbits | 123);
+                    if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t d_tmem = tmem_base + (uint32_t)((k % ROWS_ACCS) * p.acc_cols);
+                    uint32_t accumulate = 0;
+                    uint32_t b_lo = b_lo0;
+                    for (int j = 0; j <= p.kh2; ++j, b_lo += b_slice * p.slices) {
+                        const int pr = 2 * r - p.top + j;
+                        if (pr < 0 || pr >= p.hp) continue;          // rows above / below the image contribute nothing
+                        const uint32_t a_lo = a_lo0 + (uint32_t)((line_of_pr + pr) & (ROWS_LINES - 1)) * (STEM_SLOT_BYTES / 16);
+                        stem_mma_pair(d_tmem, a_lo, b_lo, p, b_slice, accumulate);
+                        accumulate = 1;
+                    }
+                    mma_commit_elect(done_bar + 8 * (k % ROWS_AHEAD));
+                }
+                line = line_of_pr + max(pr_first, min(p.hp, 2 * r1 - 1 - p.top + p.kh2));
+            }
+            if (!ok && k > 0) {
+                // aborting: give the MMAs already issued time to finish before tensor memory is released
+                const unsigned long long t0 = clock64();
+                while (!mbar_try_wait(done_bar + 8 * ((k - 1) % ROWS_AHEAD), (uint32_t)((k - 1) / ROWS_AHEAD) & 1u) &&
+                       (unsigned long long)(clock64() - t0) < DRAIN_LIMIT_CYCLES) {
+                }
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ conversion: thread = output pixel
+        // After a wait that gave up (ok == false) a warp goes through the remaining steps without touching anything, so that the
+        // barrier of the eight warps below stays complete.
+        const int quarter = warp & 3, half = warp >> 2;
+        const int px = quarter * 32 + lane;
+        const uint32_t t_lane = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        const uint32_t rsel[4] = {0, 0, 0, 0};
+        grid_dependency_wait();        // the output may overwrite what earlier work in the stream still reads
+        auto step_ready = [&]() {
+            const uint32_t bar = done_bar + 8 * (k % ROWS_AHEAD), parity = (uint32_t)(k / ROWS_AHEAD) & 1u;
+            // (in line: around a call the registers of the open pooled row would be spilled, and so little L1 is left beside the
+            // shared memory that they come back from L2)
+            const bool got = mbar_try_wait_hint(bar, parity, 4000u) || mbar_wait_poll(bar, parity, wc, tagbits | 120);
+            ok = __all_sync(0xffffffffu, got) && ok;
+            tc_fence_after();
+        };
+        auto step_read = [&]() {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(free_bar + 8 * (k % ROWS_ACCS));
+            ++k;
+        };
+        if (POOL) {
+            constexpr int CI = (CH + 1) / 2;
+            const int ch0 = half * CI;                            // this warp's chunks of the pixel: [ch0, ch0 + CI), those < cpr
+            const uint32_t swz = ((uint32_t)px >> p.swz_shift) & (uint32_t)p.swz_mask;
+            int prev[CI][16];                                     // the row above the pooled row that is open
+            uint32_t buf = 0;
+            for (int u = u_begin; u < u_end;) {
+                const int img = u / p.rows_per_img, r0 = u - img * p.rows_per_img;
+                const int r1 = min(p.rows_per_img, r0 + (u_end - u));
+                u += r1 - r0;
+#pragma unroll
+                for (int ci = 0; ci < CI; ++ci)
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) prev[ci][j] = INT_MIN;
+                if (r0 > 0) {
+                    step_ready();
+                    if (ok) {
+#pragma unroll
+                        for (int ci = 0; ci < CI; ++ci)
+                            if (ch0 + ci < p.cpr) {
+                                tmem_ld16(t_lane + (uint32_t)((k % ROWS_ACCS) * p.acc_cols + (p.cpr + ch0 + ci) * 16), prev[ci]);
+                                tmem_ld_wait16(prev[ci]);
+                            }
+                    }
+                    step_read();
+                }
+                for (int py = r0; py < r1; ++py) {
+                    const bool two = 2 * py + 1 < p.ho;
+                    const uint32_t t_addr = t_lane + (uint32_t)((k % ROWS_ACCS) * p.acc_cols);
+                    step_ready();
+                    const uint32_t dst = rows_base + buf * row_bytes + (uint32_t)px * c_out;
+#pragma unroll
+                    for (int ci = 0; ci < CI; ++ci) {
+                        const int ch = ch0 + ci;
+                        if (ok && ch < p.cpr) {
+                            int a[16], b[16];
+                            tmem_ld16(t_addr + ch * 16, a);
+                            if (two) {
+                                tmem_ld16(t_addr + (p.cpr + ch) * 16, b);
+                            } else {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) b[j] = INT_MIN;
+                            }
+                            tmem_ld_wait16(a);
+                            tmem_ld_wait16(b);
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) {
+                                a[j] = __vimax3_s32(prev[ci][j], a[j], b[j]);
+                                prev[ci][j] = b[j];
+                            }
+                            sts128(dst + (((uint32_t)ch ^ swz) << 4),
+                                   epilogue_fast16<false, SIGNED>(a, bias_base + 64 * ch, make_uint4(0, 0, 0, 0), 1, 0, rsel, p.s));
+                        }
+                    }
+                    step_read();
+                    asm volatile("bar.sync 1, %0;" ::"n"(ROWS_EPI_WARPS * 32) : "memory");
+                    // maximum over three neighbouring columns; the other buffer is free for the next row meanwhile
+                    const uint32_t src = rows_base + buf * row_bytes;
+                    uint8_t *out = p.y + ((size_t)img * p.po + py) * (size_t)p.pwo * c_out;
+                    if (ok)
+                        for (int it = threadIdx.x; it < p.pwo * p.cpr; it += ROWS_EPI_WARPS * 32) {
+                            const int ppx = CH == 4 && p.cpr == 4 ? it >> 2 : it / p.cpr, ch = it - ppx * p.cpr;
+                            uint4 t[3];
+#pragma unroll
+                            for (int d = 0; d < 3; ++d) {
+                                const uint32_t cx = (uint32_t)min(max(2 * ppx + d - 1, 0), p.wo - 1);      // the edge column again
+                                t[d] = lds128(src + cx * c_out + (((uint32_t)ch ^ ((cx >> p.swz_shift) & (uint32_t)p.swz_mask)) << 4));
+                            }
+                            *(uint4 *)(out + (size_t)it * 16) =
+                                make_uint4(max3_bytes<SIGNED>(t[0].x, t[1].x, t[2].x), max3_bytes<SIGNED>(t[0].y, t[1].y, t[2].y),
+                                           max3_bytes<SIGNED>(t[0].z, t[1].z, t[2].z), max3_bytes<SIGNED>(t[0].w, t[1].w, t[2].w));
+                        }
+                    buf ^= 1u;
+                }
+            }
+        } else {
+            for (int u = u_begin; u < u_end;) {
+                const int img = u / p.rows_per_img, r0 = u - img * p.rows_per_img;
+                const int r1 = min(p.rows_per_img, r0 + (u_end - u));
+                u += r1 - r0;
+                for (int r = r0; r < r1; ++r) {
+                    const int oy = 2 * r + half;                  // the warps of a half take one of the two rows
+                    step_ready();
+                    const uint32_t t_addr = t_lane + (uint32_t)((k % ROWS_ACCS) * p.acc_cols) + (uint32_t)half * c_out;
+                    uint8_t *out = p.y + (((size_t)img * p.ho + oy) * (size_t)p.wo + px) * c_out;
+                    if (ok && oy < p.ho) {
+#pragma unroll
+                        for (int ch = 0; ch < CH; ++ch)
+                            if (ch < p.cpr) {
+                                int a[16];
+                                tmem_ld16(t_addr + ch * 16, a);
+                                tmem_ld_wait();
+                                const uint4 o = epilogue_fast16<false, SIGNED>(a, bias_base + 64 * ch, make_uint4(0, 0, 0, 0), 1, 0, rsel, p.s);
+                                if (px < p.wo) *(uint4 *)(out + 16 * ch) = o;
+                            }
+                    }
+                    step_read();
+                }
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == ROWS_MMA_WARP) {
+        tc_fence_after();
+        tmem_dealloc(tmem_base, (uint32_t)(ROWS_ACCS * p.acc_cols));
+    }
+}
+
 }   // namespace
 
 static size_t stem_smem_bytes(int kh2, int slices, int c_out) {
     return (size_t)kh2 * slices * 32 * c_out + STEM_PAIR_SLOTS * STEM_SLOT_BYTES + 2 * 128 * (size_t)c_out + 4 * (size_t)c_out;
+}
+static size_t stem_rows_smem_bytes(int kh2, int slices, int c_out, bool pool) {
+    return (size_t)(kh2 + 1) * slices * 32 * 2 * c_out + ROWS_LINES * STEM_SLOT_BYTES + (pool ? 2 * 128 * (size_t)c_out : 0) + 4 * (size_t)c_out;
 }
 
 bool f8_stem_tc_supported(const F8ConvGeom &g, const F8Requant &q, int kh2, int slices) {
@@ -376,14 +743,22 @@ bool f8_stem_tc_supported(const F8ConvGeom &g, const F8Requant &q, int kh2, int 
 
 namespace {
 typedef void (*StemKernel)(const StemParams, const int);
-template <int CPR, bool POOL, bool SIGNED>
-StemKernel pick_fast(bool fast) {
-    return fast ? f8_stem_tc_kernel<CPR, POOL, SIGNED, true> : f8_stem_tc_kernel<CPR, POOL, SIGNED, false>;
+template <bool POOL, bool SIGNED>
+StemKernel pick_wide(bool fast) {
+    return fast ? f8_stem_tc_kernel<POOL, SIGNED, true> : f8_stem_tc_kernel<POOL, SIGNED, false>;
 }
-template <int CPR>
-StemKernel pick_kernel(bool pool, bool sgn, bool fast) {
-    if (pool) return sgn ? pick_fast<CPR, true, true>(fast) : pick_fast<CPR, true, false>(fast);
-    return sgn ? pick_fast<CPR, false, true>(fast) : pick_fast<CPR, false, false>(fast);
+template <int CH, bool POOL, bool SIGNED>
+StemKernel pick_rows(bool fast) {
+    return fast ? f8_stem_rows_tc_kernel<CH, POOL, SIGNED, true> : f8_stem_rows_tc_kernel<CH, POOL, SIGNED, false>;
+}
+template <int CH>
+StemKernel pick_rows(bool pool, bool sgn, bool fast) {
+    if (pool) return sgn ? pick_rows<CH, true, true>(fast) : pick_rows<CH, true, false>(fast);
+    return sgn ? pick_rows<CH, false, true>(fast) : pick_rows<CH, false, false>(fast);
+}
+StemKernel pick_wide(bool pool, bool sgn, bool fast) {
+    if (pool) return sgn ? pick_wide<true, true>(fast) : pick_wide<true, false>(fast);
+    return sgn ? pick_wide<false, true>(fast) : pick_wide<false, false>(fast);
 }
 }   // namespace
 
@@ -397,20 +772,24 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
     p.kh2 = kh2; p.top = top; p.left = left; p.hp = (g.h + 1) / 2; p.slices = slices;
     p.ncell = std::min(STEM_MAX_CELLS, 2 * (g.wo - 1) + slices * 4);
     p.pool = pool;
+    // up to 64 channels: the kernel with a warp role each (two rows per step, two accumulators of at most 128 columns, two CTAs per SM);
+    // wider layers would leave it one CTA per SM or not fit, and keep the kernel with two accumulators
+    const bool rows = g.c_out <= 64;
+    const int n_cols = rows ? 2 * g.c_out : g.c_out;        // columns of one multiplication
     p.po = (g.ho - 1) / 2 + 1;
     p.pwo = (g.wo - 1) / 2 + 1;
-    p.rows_per_img = pool ? p.po : g.ho;
+    p.rows_per_img = pool ? p.po : (rows ? (g.ho + 1) / 2 : g.ho);
     p.acc_cols = 32;
-    while (p.acc_cols < g.c_out) p.acc_cols *= 2;
+    while (p.acc_cols < n_cols) p.acc_cols *= 2;
     p.cpr = g.c_out / 16;
     const bool pow2 = (p.cpr & (p.cpr - 1)) == 0;
     p.swz_shift = p.cpr == 4 ? 1 : (p.cpr == 2 ? 2 : 0);
     p.swz_mask = (pow2 && p.cpr > 1) ? std::min(p.cpr, 8) - 1 : 0;
-    p.idesc = (2u << 4) | ((g.x_signed ? 1u : 0u) << 7) | (1u << 10) | ((uint32_t)(g.c_out >> 3) << 17) | ((128u >> 4) << 24);
+    p.idesc = (2u << 4) | ((g.x_signed ? 1u : 0u) << 7) | (1u << 10) | ((uint32_t)(n_cols >> 3) << 17) | ((128u >> 4) << 24);
     // K-major operands without swizzle: core matrices of 8 rows x 16 bytes are 128 contiguous bytes; the leading
     // byte offset is the distance between core matrices along K, the stride byte offset the one between 8-row groups.
-    // A (overlapping windows): 16 bytes along K, 128 bytes along M.  B ([K/16][c_out][16]): c_out * 16 along K, 128 along N.
-    const uint32_t a_lbo = 16, a_sbo = 128, b_lbo = (uint32_t)g.c_out * 16, b_sbo = 128;
+    // A (overlapping windows): 16 bytes along K, 128 bytes along M.  B ([K/16][columns][16]): columns * 16 along K, 128 along N.
+    const uint32_t a_lbo = 16, a_sbo = 128, b_lbo = (uint32_t)n_cols * 16, b_sbo = 128;
     p.a_desc_lbo_sbo = (a_lbo >> 4) << 16;
     p.b_desc_lbo_sbo = (b_lbo >> 4) << 16;
     p.a_desc_hi = (a_sbo >> 4) | (1u << 14);     // stride byte offset at bit 32, descriptor version 1 at bit 46, no swizzle
@@ -423,9 +802,9 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
 
     const bool fast = ((uintptr_t)x & 3) == 0 && ((size_t)g.n * g.h * g.w * g.c) % 4 == 0;
     const bool sgn = p.signed_out != 0;
-    StemKernel kernel = p.cpr == 4 ? pick_kernel<4>(pool != 0, sgn, fast)
-                        : (p.cpr == 2 ? pick_kernel<2>(pool != 0, sgn, fast) : pick_kernel<0>(pool != 0, sgn, fast));
-    const size_t smem = stem_smem_bytes(kh2, slices, g.c_out);
+    StemKernel kernel = !rows ? pick_wide(pool != 0, sgn, fast) : (p.cpr > 2 ? pick_rows<4>(pool != 0, sgn, fast) : pick_rows<2>(pool != 0, sgn, fast));
+    const size_t smem = rows ? stem_rows_smem_bytes(kh2, slices, g.c_out, pool != 0) : stem_smem_bytes(kh2, slices, g.c_out);
+    const int threads = rows ? ROWS_THREADS : STEM_THREADS, accs = rows ? ROWS_ACCS : 2;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024));
     // several CTAs are meant to share an SM: ask for the largest shared-memory carve-out (the default preference
     // sizes it for a single CTA of this kernel)
@@ -435,23 +814,24 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // CTAs that fit an SM, from the kernel's own resource use (the runtime's occupancy query answers 1 for this
-    // kernel whatever the carve-out): registers, shared memory, threads, and two accumulators each in tensor memory
+    // kernel whatever the carve-out): registers, shared memory, threads, and their accumulators in tensor memory
     cudaFuncAttributes fa;
     if (cudaFuncGetAttributes(&fa, kernel) == cudaSuccess && fa.numRegs > 0) {
-        const int regs_per_cta = ((fa.numRegs + 7) / 8 * 8) * STEM_THREADS;
+        const int regs_per_cta = ((fa.numRegs + 7) / 8 * 8) * threads;
         const int by_regs = 65536 / regs_per_cta;
         const int by_smem = (int)((227 * 1024) / (smem + fa.sharedSizeBytes + 1024));
-        const int by_threads = 2048 / STEM_THREADS;
+        const int by_threads = 2048 / threads;
         occ = std::min(std::min(by_regs, by_smem), by_threads);
     }
-    occ = std::min(occ, 512 / (2 * p.acc_cols));
+    occ = std::min(occ, 512 / (accs * p.acc_cols));
     occ = std::max(1, std::min(occ, 4));
     const long long units = (long long)g.n * p.rows_per_img;
-    // bands of at least four output rows (each band recomputes one row above it when pooling)
-    long long grid = std::min<long long>((long long)sms * occ, std::max<long long>(1, units / 4));
+    // bands of at least four units (with a pool every band computes one row above it again); when that leaves SMs idle, as many
+    // bands as there are units up to one per SM
+    long long grid = std::min<long long>((long long)sms * occ, std::max<long long>(units / 4, std::min<long long>(units, sms)));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(STEM_THREADS);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];

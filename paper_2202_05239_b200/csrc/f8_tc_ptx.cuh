@@ -32,6 +32,11 @@ __device__ __forceinline__ WaitCtx make_wait_ctx(volatile int *abort_flag, int *
 
 // ----------------------------------------------------------------------------- PTX wrappers
 
+// A value that is the same in all lanes of a (converged) warp, in a form the compiler knows to be so: branches on it do not
+// count as divergent, and what is computed from it may live in uniform registers.
+template <typename T>
+__device__ __forceinline__ T uniform(T v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Programmatic dependent launch.  A grid launched with the programmatic-serialization attribute may start
@@ -76,7 +81,7 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
 }
 
 // Bounded wait.  Returns false when the kernel is aborting (this wait or another one ran out).
-__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const WaitCtx &wc, int code) {
+__device__ __forceinline__ bool mbar_wait_poll(uint32_t bar, uint32_t parity, const WaitCtx &wc, int code) {
     volatile int *abort_flag = wc.abort_flag;
     int *status = wc.status;
     const unsigned long long t0 = clock64();
@@ -116,6 +121,9 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const
             }
         }
     }
+}
+__device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const WaitCtx &wc, int code) {
+    return mbar_wait_poll(bar, parity, wc, code);
 }
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx &wc, int code) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -241,6 +249,15 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
 }
+// The same from a whole warp.  A loop that only one lane runs keeps every address and descriptor word in that lane's
+// registers, and each of them has to be moved to the uniform registers an MMA reads; when the warp runs the loop together and
+// one lane is elected at the instruction itself, the compiler can keep them uniform throughout.  The elected lane is the same
+// every time, so a commit covers the warp's earlier MMAs.
+__device__ __forceinline__ void mma_commit_elect(uint32_t bar) {
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+                 : "memory");
+}
 
 // ----------------------------------------------------------------------------- CTA pairs (tcgen05 cta_group::2)
 // Two CTAs of a cluster work on one 256-row tile: each holds its own 128 rows of A and half of the B tile in its shared
@@ -328,6 +345,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, int (&v)[16]) {
         : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// The same wait, tied to the registers of a load: arithmetic on them that depends on nothing else must not be moved ahead of it.
+__device__ __forceinline__ void tmem_ld_wait16(int (&v)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]),
+                   "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+                 :
+                 : "memory");
+}
 
 // Shared-memory matrix descriptor of a K-major tile whose rows are `kb` bytes long and swizzled with
 // the matching TMA mode: 8-row groups are 8*kb bytes apart (stride byte offset), the leading offset

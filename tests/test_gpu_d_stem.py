@@ -97,3 +97,31 @@ def test_stem_pool_fusion_needs_a_single_consumer(ref):
     assert net.last_launch_count == 3
     assert np.array_equal(out.cpu().numpy().reshape(want[-1].shape), want[-1])
     net.close()
+
+
+# (h, w, c, c_out, k, pad, batch, y_dtype, with_pool): where the kernel for up to 64 channels changes its ways
+ROWS_EDGE_CASES = [
+    (2, 2, 3, 64, 7, 3, 3, synth.U8, True),         # one output row and column per image
+    (6, 8, 3, 64, 7, 3, 900, synth.U8, True),       # three rows per image, several images per CTA: windows never shared
+    (10, 6, 3, 32, 3, 1, 700, synth.U8, False),     # odd row count without a pool, several images per CTA
+    (256, 256, 3, 64, 7, 3, 1, synth.U8, True),     # 128 outputs per row; as many bands as rows
+    (33, 31, 3, 64, 8, 4, 5, synth.S8, True),       # windows of eight taps: five row pairs, six per step
+    (95, 97, 3, 16, 3, 1, 2, synth.U8, True),       # byte count of a row not a multiple of four
+]
+
+
+@pytest.mark.parametrize("case", range(len(ROWS_EDGE_CASES)))
+def test_stem_rows_kernel_edges(ref, case):
+    h, w, c, c_out, k, pad, batch, y_dtype, with_pool = ROWS_EDGE_CASES[case]
+    rng = np.random.default_rng(970 + case)
+    layers = _stem_net(rng, h, w, c, c_out, k, pad, y_dtype, with_pool)
+    x = rng.integers(-128, 128, size=(batch, h, w, c)).astype(np.int8)
+    want = ref.net_forward(layers, x, keep_all=False)[-1]
+    a = api()
+    net = a.Net(layers, batch)
+    before = a.f8_tc_launch_count()
+    out = net.forward(a.to_device(x))
+    torch.cuda.synchronize()
+    a.f8_device_status()
+    assert a.f8_tc_launch_count() - before == 1 and net.last_launch_count == 1
+    assert int((out.cpu().numpy().reshape(want.shape) != want).sum()) == 0
