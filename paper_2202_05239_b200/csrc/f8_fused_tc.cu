@@ -94,7 +94,7 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
     uint8_t *smem_aligned = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     FtControl &ctl = *(FtControl *)smem_aligned;
     uint8_t *smem = smem_aligned + FT_CONTROL_BYTES;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform((int)(threadIdx.x >> 5)), lane = threadIdx.x & 31;
     const int worker = (int)blockIdx.x, n_workers = (int)gridDim.x;
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t full_bar = smem_u32(&ctl.full[0]), empty_bar = smem_u32(&ctl.empty[0]);
@@ -139,7 +139,7 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = ctl.tmem_base_slot;
+    const uint32_t tmem_base = uniform(ctl.tmem_base_slot);
     grid_launch_dependents();
 
     const int n_local = worker < p.m_tiles ? (p.m_tiles - worker + n_workers - 1) / n_workers : 0;
@@ -213,11 +213,11 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
         if (half == 1 && lane == 0) mbar_wait(wres_bar, 0, wc, tagbits | 210);
     } else if (warp == FT_MMA_WARP) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0 && n_local > 0) {
+        if (n_local > 0) {
             const uint32_t desc_lo0 = (uint32_t)p.desc_hi | ((smem_base & 0x3ffffu) >> 4);
             const uint32_t desc_hi32 = (uint32_t)(p.desc_hi >> 32);
             const uint32_t w1_lo = desc_lo0 + (p.w1_off >> 4);
-            bool ok = mbar_wait(wres_bar, 0, wc, tagbits | 211);
+            bool ok = warp_wait(wres_bar, 0, wc, tagbits | 211);
             bool committed_any = false;
             int last_acc = 0;
             uint32_t last_acc_phase = 0;
@@ -225,12 +225,12 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
             const int G = p.group, NG = p.groups;
             for (int l = 0; ok && l < n_local; ++l) {
                 const int acc = l & 1;
-                if (!mbar_wait(tempty1 + 8 * acc, (uint32_t)((l >> 1) & 1) ^ 1u, wc, tagbits | 202)) { ok = false; break; }
+                if (!warp_wait(tempty1 + 8 * acc, (uint32_t)((l >> 1) & 1) ^ 1u, wc, tagbits | 202)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)acc * FT_C;
                 int tap = 0;
                 for (int k = 0; k < NG; ++k) {
-                    if (!mbar_wait(full_bar + 8 * slot, (uint32_t)(use & 1), wc, tagbits | 203)) { ok = false; break; }
+                    if (!warp_wait(full_bar + 8 * slot, (uint32_t)(use & 1), wc, tagbits | 203)) { ok = false; break; }
                     tc_fence_after();
                     uint32_t a_lo = desc_lo0 + (uint32_t)(slot * G) * (FT_A_BYTES >> 4);
                     for (int t = 0; t < G && tap < p.taps; ++t, ++tap, a_lo += FT_A_BYTES >> 4)
@@ -248,7 +248,7 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
                 // the releases of the last stage uses, which nobody else waits for, must land before the CTA goes
                 const int total = n_local * NG;
                 for (int g = max(0, total - p.stages); g < total; ++g)
-                    mbar_wait(empty_bar + 8 * (g % p.stages), (uint32_t)(g / p.stages) & 1u, wc, tagbits | 212);
+                    warp_wait(empty_bar + 8 * (g % p.stages), (uint32_t)(g / p.stages) & 1u, wc, tagbits | 212);
             } else if (committed_any) {
                 // let the tensor pipe finish what was issued before tensor memory is released
                 const unsigned long long t0 = clock64();
@@ -261,22 +261,22 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
         // GEMM 2 of local tile i: the staged tile times the pointwise weights, as soon as the first layer's epilogue has
         // written the tile and the second layer's epilogue has read the previous result out of the accumulator.  A thread
         // of its own, so that these waits do not sit between the first issuer's instructions.
-        if (lane == 0 && n_local > 0) {
+        if (n_local > 0) {
             const uint32_t desc_lo0 = (uint32_t)p.desc_hi | ((smem_base & 0x3ffffu) >> 4);
             const uint32_t desc_hi32 = (uint32_t)(p.desc_hi >> 32);
             const uint32_t w2_lo = desc_lo0 + (p.w2_off >> 4), t_lo = desc_lo0 + (p.t_off >> 4);
-            bool ok = mbar_wait(wres_bar, 0, wc, tagbits | 214);
+            bool ok = warp_wait(wres_bar, 0, wc, tagbits | 214);
             int i = 0;
             for (; ok && i < n_local; ++i) {
-                if (!mbar_wait(tmid_full, (uint32_t)(i & 1), wc, tagbits | 205)) { ok = false; break; }
-                if (!mbar_wait(tempty2, (uint32_t)(i & 1) ^ 1u, wc, tagbits | 206)) { ok = false; break; }
+                if (!warp_wait(tmid_full, (uint32_t)(i & 1), wc, tagbits | 205)) { ok = false; break; }
+                if (!warp_wait(tempty2, (uint32_t)(i & 1) ^ 1u, wc, tagbits | 206)) { ok = false; break; }
                 tc_fence_after();
                 mma_i8_sub<2>(tmem_base + FT_ACC2_COL, t_lo, w2_lo, desc_hi32, p.idesc2, 0u);
                 mma_commit(tmid_free);
                 mma_commit(tfull2);
             }
             // the last release of the staged tile has no other waiter
-            if (ok) mbar_wait(tmid_free, (uint32_t)((n_local - 1) & 1), wc, tagbits | 213);
+            if (ok) warp_wait(tmid_free, (uint32_t)((n_local - 1) & 1), wc, tagbits | 213);
         }
     } else if (warp == FT_MOVER_WARP) {
         // ------------------------------------------------------------------ output mover

@@ -5,7 +5,7 @@
 //     activation tensor by TMA in im2col mode (zero fill outside the image and past the last pixel);
 //     B tiles (BN output channels x KB) come from the OHWI weight tensor by tiled TMA.  Both land in
 //     shared memory in the swizzled K-major layout tcgen05.mma reads.
-//   * One thread issues tcgen05.mma.kind::i8 (u8|s8 x s8 -> s32); the 128 x BN int32 accumulator lives
+//   * One warp (one elected lane) issues tcgen05.mma.kind::i8 (u8|s8 x s8 -> s32); the 128 x BN int32 accumulator lives
 //     in tensor memory, double buffered so the epilogue of tile i overlaps the main loop of tile i+1.
 //   * Sixteen epilogue warps read the accumulator with tcgen05.ld (one output pixel per thread, 16
 //     consecutive channels per load), add the bias, align and add the residual, apply the rounding
@@ -268,7 +268,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     uint32_t &tmem_base_slot = ctl.tmem_base_slot;
     int &abort_flag = ctl.abort_flag;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = uniform((int)(threadIdx.x >> 5));
     const int lane = threadIdx.x & 31;
     // persistent workers: CTAs, or CTA pairs (rank 0 = the even CTA, which owns the stage barriers and issues the MMAs)
     const uint32_t cta_rank = PAIR ? cluster_cta_rank() : 0u;
@@ -326,7 +326,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     __syncthreads();
     if (PAIR) cluster_sync_all();      // the partner's barriers exist before anything is sent to them
     tc_fence_after();
-    const uint32_t tmem_base = tmem_base_slot;
+    const uint32_t tmem_base = uniform(tmem_base_slot);
     // the next grid in the stream may be scheduled from here on: its CTAs take over an SM when this grid's
     // CTA there has exited, and run their prologue while the rest of this grid finishes
     grid_launch_dependents();
@@ -584,7 +584,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 for (int g = max(0, total_uses - p.stages); g < total_uses; ++g)
                     mbar_wait(empty_bar + 8 * (g % p.stages), (uint32_t)(g / p.stages) & 1u, wc, tagbits | 113);
             }
-        } else if (lane == 0 && (q_issuer == 0 || p.dual_issue)) {
+        } else if (q_issuer == 0 || p.dual_issue) {
             int stage = 0;
             uint32_t phase = 0;
             int local = 0;
@@ -599,7 +599,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             const uint32_t stage16 = p.stage_bytes >> 4, sub16 = p.sub_bytes >> 4, a16 = p.a_bytes >> 4;
             const uint32_t b16 = p.b_bytes >> 4, bres_lo = desc_lo0 + (p.bres_off >> 4);
             const uint32_t b_step = p.b_res ? b16 : sub16;
-            if (p.b_res && !mbar_wait(bres_bar, 0, wc, tagbits | 111)) ok = false;
+            if (p.b_res && !warp_wait(bres_bar, 0, wc, tagbits | 111)) ok = false;
             const int mmas = p.kb >> 5;      // 1, 2 or 4 instructions per stage
             for (int tile = worker; ok && tile < total_tiles; tile += n_workers, ++local) {
                 const int acc = local & 1;
@@ -611,7 +611,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                     continue;
                 }
                 const uint32_t acc_phase = (local >> 1) & 1;
-                if (!mbar_wait(tempty_bar + 8 * acc, acc_phase ^ 1, wc, tagbits | 102)) { ok = false; break; }
+                if (!warp_wait(tempty_bar + 8 * acc, acc_phase ^ 1, wc, tagbits | 102)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + acc * 256;   // two 256-column accumulators
                 uint32_t b_tile_lo = 0;
@@ -622,7 +622,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 if (SUP) {
                     // one stage use: the activation tiles of up to p.sup M tiles, each accumulated (a single k-iteration) into
                     // its own column range of this accumulator
-                    if (!mbar_wait(full_bar + 8 * stage, phase, wc, tagbits | 103)) { ok = false; break; }
+                    if (!warp_wait(full_bar + 8 * stage, phase, wc, tagbits | 103)) { ok = false; break; }
                     tc_fence_after();
                     const int subs = min(p.sup, p.m_tiles - tile * p.sup);
                     uint32_t a_lo = stage_lo;
@@ -639,7 +639,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                     // one stage use per channel chunk; the nine taps read the same tile at shifted row offsets
                     const uint32_t kb16 = (uint32_t)p.kb >> 4;
                     for (int cc = 0; cc < p.c_chunks; ++cc) {
-                        if (!mbar_wait(full_bar + 8 * stage, phase, wc, tagbits | 103)) { ok = false; break; }
+                        if (!warp_wait(full_bar + 8 * stage, phase, wc, tagbits | 103)) { ok = false; break; }
                         tc_fence_after();
                         uint32_t first = cc != 0 ? 1u : 0u;
                         uint32_t b_lo = b_tile_lo + (uint32_t)cc * b16;
@@ -660,7 +660,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                     }
                 } else
                 for (int kc = 0; kc < k_iters; kc += p.group) {
-                    if (!mbar_wait(full_bar + 8 * stage, phase, wc, tagbits | 103)) { ok = false; break; }
+                    if (!warp_wait(full_bar + 8 * stage, phase, wc, tagbits | 103)) { ok = false; break; }
                     tc_fence_after();
                     const int subs = min(p.group, k_iters - kc);
                     const uint32_t first = kc != 0 ? 1u : 0u;      // the tile's first MMA overwrites the accumulator
@@ -697,7 +697,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 for (int g = max(0, total_uses - p.stages); g < total_uses; ++g) {
                     const int t_of_g = g / uses_tile;
                     if (p.dual_issue && (t_of_g & 1) != q_issuer) continue;
-                    mbar_wait(empty_bar + 8 * (g % p.stages), (uint32_t)(g / p.stages) & 1u, wc, tagbits | 112);
+                    warp_wait(empty_bar + 8 * (g % p.stages), (uint32_t)(g / p.stages) & 1u, wc, tagbits | 112);
                 }
             }
             if (!ok && committed_any) {
@@ -970,7 +970,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) f8_mma_probe_kernel(int iters,
         const uint32_t idesc = (2u << 4) | (0u << 7) | (1u << 10) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
         for (int i = 0; i < iters; ++i)
             mma_i8(tmem_base + (i & 1) * 256, a_desc + 2 * (i & 3), b_desc + 2 * (i & 3), idesc, i > 1 ? 1u : 0u);
-        mma_commit(smem_u32(&bar));
+        mma_commit_thread(smem_u32(&bar));
         mbar_wait(smem_u32(&bar), 0, make_wait_ctx(&abort_flag, status, 0), 105);
     }
     tc_fence_before();

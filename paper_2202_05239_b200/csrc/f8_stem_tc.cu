@@ -84,11 +84,11 @@ __device__ __forceinline__ uint32_t load_pixel(const uint8_t *x, uint32_t off, u
     return word;
 }
 
-// The one or two K slices of a row pair.  Executed by a whole warp, one lane issues: see mma_commit_elect().
+// The one or two K slices of a row pair.  Executed by a whole warp, one lane issues: see mma_commit().
 __device__ __forceinline__ void stem_mma_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, const StemParams &p, uint32_t b_slice,
                                               uint32_t accumulate) {
     if (p.slices == 2)
-        asm volatile("{\n\t.reg .pred e, p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\telect.sync _|e, 0xffffffff;\n\t"
+        asm volatile("{\n\t" F8_ELECT ".reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\t"
                      "setp.ne.b32 p, %7, 0;\n\tsetp.eq.b32 t, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t"
                      "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, p;\n\t"
                      "add.u32 x, %1, 2;\n\tadd.u32 y, %2, %5;\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %4};\n\t"
@@ -96,7 +96,7 @@ __device__ __forceinline__ void stem_mma_pair(uint32_t d_tmem, uint32_t a_lo, ui
                      "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(b_slice), "r"(p.idesc), "r"(accumulate)
                      : "memory");
     else
-        asm volatile("{\n\t.reg .pred e, p;\n\t.reg .b64 a, b;\n\telect.sync _|e, 0xffffffff;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+        asm volatile("{\n\t" F8_ELECT ".reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %6, 0;\n\t"
                      "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t"
                      "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
                      "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(p.idesc), "r"(accumulate)
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
             stem_mma_pair(d_tmem, a_lo, b_lo, p, b_slice, accumulate);
             accumulate = 1;
         }
-        mma_commit_elect(smem_u32(&acc_bar[kk & 1]));
+        mma_commit(smem_u32(&acc_bar[kk & 1]));
     };
 
     for (int u = u_begin; u < u_end;) {
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) f8_stem_rows_tc_kernel(const 
                         stem_mma_pair(d_tmem, a_lo, b_lo, p, b_slice, accumulate);
                         accumulate = 1;
                     }
-                    mma_commit_elect(done_bar + 8 * (k % ROWS_AHEAD));
+                    mma_commit(done_bar + 8 * (k % ROWS_AHEAD));
                 }
                 line = line_of_pr + max(pr_first, min(p.hp, 2 * r1 - 1 - p.top + p.kh2));
             }

@@ -131,6 +131,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
     return mbar_wait_slow(bar, parity, wc, code);
 }
 
+// A whole warp waits; the answer is uniform.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const WaitCtx &wc, int code) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, wc, code));
+}
+
 __device__ __forceinline__ void tma_load_im2col(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c, int w,
                                                 int h, int n, uint16_t off_w, uint16_t off_h) {
     asm volatile(
@@ -203,29 +208,34 @@ __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_
         : "memory");
 }
 
-// The K = 32 slices of one sub-chunk (kb / 32 of them), issued from one asm block.  A lone thread pays a few
-// cycles for every instruction it executes, and the tensor pipe is only kept busy when an MMA costs the
-// issuing thread no more than a handful of them: the shared-memory descriptors of the slices differ only
-// in their low words (start address, 16-byte units), so those are advanced with 32-bit adds inside the
-// block and the constant high word (SBO, version, swizzle mode) is attached by a register-pair move.
-#define F8_MMA_I8 "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, "
+// The MMA-issuing warps run their loops as a whole and one lane is elected at the instruction itself (always the same one, so
+// a commit covers the warp's earlier MMAs).  In a loop that a single lane runs, the compiler has to keep every address and
+// descriptor word in that lane's registers and move each of them to the uniform registers the instruction reads; a
+// convergent loop over values known to be uniform (uniform(), votes on the waits) lives there throughout.  Measured on the
+// first-layer kernel: 195 -> 130 cycles per instruction of 64 columns with the epilogue warps at work.
+//
+// The K = 32 slices of one sub-chunk (kb / 32 of them), issued from one asm block: the shared-memory descriptors of the slices
+// differ only in their low words (start address, 16-byte units), so those are advanced with 32-bit adds inside the block and
+// the constant high word (SBO, version, swizzle mode) is attached by a register-pair move.
+#define F8_ELECT ".reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+#define F8_MMA_I8 "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, "
 #define F8_MMA_NEXT(off) \
     "add.u32 x, %1, " #off ";\n\tadd.u32 y, %2, " #off ";\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %3};\n\t" F8_MMA_I8 "t;\n\t"
 template <int MMAS>
 __device__ __forceinline__ void mma_i8_sub(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi,
                                            uint32_t idesc, uint32_t accumulate) {
     if (MMAS == 1)
-        asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        asm volatile("{\n\t" F8_ELECT ".reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %5, 0;\n\t"
                      "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t" F8_MMA_I8 "p;\n\t}" ::"r"(d_tmem),
                      "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
                      : "memory");
     else if (MMAS == 2)
-        asm volatile("{\n\t.reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        asm volatile("{\n\t" F8_ELECT ".reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\t"
                      "setp.eq.b32 t, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t" F8_MMA_I8 "p;\n\t"
                      F8_MMA_NEXT(2) "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"(accumulate)
                      : "memory");
     else
-        asm volatile("{\n\t.reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+        asm volatile("{\n\t" F8_ELECT ".reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\t"
                      "setp.eq.b32 t, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t" F8_MMA_I8 "p;\n\t"
                      F8_MMA_NEXT(2) F8_MMA_NEXT(4) F8_MMA_NEXT(6) "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi),
                      "r"(idesc), "r"(accumulate)
@@ -244,18 +254,14 @@ __device__ __forceinline__ void mma_i8_stage(uint32_t d_tmem, uint32_t a_lo, uin
         mma_i8_sub<MMAS>(d_tmem, a_lo, b_lo, desc_hi, idesc, 1u);
     }
 }
-// mbarrier arrives once every tcgen05.mma issued so far by this thread has completed.
+// mbarrier arrives once every tcgen05.mma issued so far by this warp has completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
+    asm volatile("{\n\t" F8_ELECT "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
                  : "memory");
 }
-// The same from a whole warp.  A loop that only one lane runs keeps every address and descriptor word in that lane's
-// registers, and each of them has to be moved to the uniform registers an MMA reads; when the warp runs the loop together and
-// one lane is elected at the instruction itself, the compiler can keep them uniform throughout.  The elected lane is the same
-// every time, so a commit covers the warp's earlier MMAs.
-__device__ __forceinline__ void mma_commit_elect(uint32_t bar) {
-    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
-                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+// The same for a single thread that issued its MMAs by itself (mma_i8).
+__device__ __forceinline__ void mma_commit_thread(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
 }
 
@@ -313,21 +319,22 @@ __device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t cols
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t cols) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
-// arrives on the barrier at this offset in both CTAs of the pair once every MMA issued so far by this thread has completed
+// arrives on the barrier at this offset in both CTAs of the pair once every MMA issued so far by this warp has completed
 __device__ __forceinline__ void mma_commit_pair(uint32_t bar) {
     const uint16_t both = 3;
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+    asm volatile("{\n\t" F8_ELECT
+                 "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}" ::"r"(bar),
                  "h"(both)
                  : "memory");
 }
 // The K = 32 slices of one 128-byte sub-chunk (four of them) as 256-row instructions of the pair, from one asm block.
-#define F8_MMA_I8_PAIR "tcgen05.mma.cta_group::2.kind::i8 [%0], a, b, %4, {%6, %6, %6, %6, %6, %6, %6, %6}, "
+#define F8_MMA_I8_PAIR "@e tcgen05.mma.cta_group::2.kind::i8 [%0], a, b, %4, {%6, %6, %6, %6, %6, %6, %6, %6}, "
 #define F8_MMA_NEXT_PAIR(off) \
     "add.u32 x, %1, " #off ";\n\tadd.u32 y, %2, " #off ";\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %3};\n\t" F8_MMA_I8_PAIR "t;\n\t"
 __device__ __forceinline__ void mma_i8_sub_pair4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
                                                  uint32_t accumulate) {
     const uint32_t zero = 0;      // no output lane is disabled
-    asm volatile("{\n\t.reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+    asm volatile("{\n\t" F8_ELECT ".reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\tsetp.ne.b32 p, %5, 0;\n\t"
                  "setp.eq.b32 t, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t" F8_MMA_I8_PAIR "p;\n\t"
                  F8_MMA_NEXT_PAIR(2) F8_MMA_NEXT_PAIR(4) F8_MMA_NEXT_PAIR(6) "}" ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi),
                  "r"(idesc), "r"(accumulate), "r"(zero)
