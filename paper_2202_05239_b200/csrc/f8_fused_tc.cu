@@ -115,7 +115,7 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
     if (threadIdx.x == 0) {
         ctl.abort_flag = 0;
         for (int s = 0; s < p.stages; ++s) {
-            mbar_init(full_bar + 8 * s, p.group);  // every lane that requests a tap of the group announces its bytes
+            mbar_init(full_bar + 8 * s, 1);        // the warp that requests the group announces its bytes
             mbar_init(empty_bar + 8 * s, 1);       // commit of the MMAs that read the stage
         }
         mbar_init(wres_bar, 1);
@@ -150,59 +150,50 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
         // ------------------------------------------------------------------ TMA producers
         // A stage holds a group of G consecutive taps of one tile (one barrier pair per group: every wait, fence and commit
         // costs the lone MMA-issuing thread a few hundred cycles, as much as several MMAs).  Group k of local tile l is
-        // use u = l * groups + k of the ring: stage u mod S, use u div S.  Warp h requests the uses of parity h, every
-        // tap in a lane of its own (loads issued by different threads overlap).  S is even, so a stage is always
-        // refilled by the same warp: the wait for its previous refill comes earlier in that warp's program order, and
-        // a parity wait (which can only tell a phase from its neighbour) cannot take an older release for the last one.
+        // use u = l * groups + k of the ring: stage u mod S, use u div S.  Warp h requests the uses of parity h.  S is even, so a
+        // stage is always refilled by the same warp: the wait for its previous refill comes earlier in that warp's program
+        // order, and a parity wait (which can only tell a phase from its neighbour) cannot take an older release for the last one.
         const int half = warp == FT_A2_WARP ? 1 : 0;
         if (half == 1) {
             // the weights of both layers, once per CTA: nothing the previous grid writes
-            const int n_loads = p.taps + 1;
-            if (lane == 0) mbar_expect_tx(wres_bar, (uint32_t)p.taps * FT_W1_BYTES + FT_W2_BYTES);
-            __syncwarp();
-            if (lane < p.taps) tma_load_3d(smem_base + p.w1_off + (uint32_t)lane * FT_W1_BYTES, &map_w1, wres_bar, 0, lane, 0);
-            else if (lane == n_loads - 1) tma_load_3d(smem_base + p.w2_off, &map_w2, wres_bar, 0, 0, 0);
+            warp_expect_tx(wres_bar, (uint32_t)p.taps * FT_W1_BYTES + FT_W2_BYTES);
+            for (int t = 0; t < p.taps; ++t) tma_load_3d(smem_base + p.w1_off + (uint32_t)t * FT_W1_BYTES, &map_w1, wres_bar, 0, t, 0, lane == t);
+            tma_load_3d(smem_base + p.w2_off, &map_w2, wres_bar, 0, 0, 0, lane == p.taps);
         }
         grid_dependency_wait();
-        const int G = p.group, NG = p.groups, S = p.stages, per_round = S >> 1;
-        const int gi = lane / G, ti = lane - gi * G;       // this lane's group among the warp's groups of a tile, tap in the group
+        const int G = p.group, NG = p.groups;
         bool ok = true, have_last = false;
-        int last_slot = 0;
-        uint32_t last_par = 0;
-        for (int l = 0; l < n_local; ++l) {
+        int last_slot = 0, slot = 0, u = 0;
+        uint32_t last_par = 0, par = 0;
+        for (int l = 0; ok && l < n_local; ++l) {
             const int m0 = (worker + l * n_workers) * FT_TILE_M;
             const int t1 = ft_div(m0, p.div_wo);
             const int ow = m0 - t1 * p.wo;
             const int img = ft_div(t1, p.div_ho);
             const int oh = t1 - img * p.ho;
-            const int u0 = l * NG;
-            const int k0 = (half - u0) & 1;                          // this warp's first group of the tile
-            const int n_mine = k0 < NG ? (NG - k0 + 1) >> 1 : 0;     // groups k0, k0 + 2, ...
-            const int k = k0 + 2 * gi, u = u0 + k, tap = k * G + ti;
-            const int slot = u % S, use = u / S;
-            const int r = tap / p.kw, sx = tap - r * p.kw;
-            // at most S / 2 of the warp's groups at a time: they lie in different stages, and a stage a later round needs
-            // is freed by loads that were requested in an earlier one
-            for (int r0 = 0; ok && r0 < n_mine; r0 += per_round) {
-                const bool act = gi < n_mine && gi >= r0 && gi < r0 + per_round;
-                bool got = true;
-                if (act) got = mbar_wait(empty_bar + 8 * slot, (uint32_t)(use & 1) ^ 1u, wc, tagbits | 201);
-                if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
-                if (act) {
+            const int base_w = ow * p.stride - p.pad, base_h = oh * p.stride - p.pad;
+            int tap = 0, r = 0, sx = 0;
+            for (int k = 0; k < NG; ++k, ++u) {
+                const int n = min(G, p.taps - tap);
+                if ((u & 1) != half) {
+                    for (int t = 0; t < n; ++t)
+                        if (++sx == p.kw) { sx = 0; ++r; }
+                } else {
+                    if (!warp_wait(empty_bar + 8 * slot, par ^ 1u, wc, tagbits | 201)) { ok = false; break; }
                     const uint32_t fb = full_bar + 8 * slot;
-                    if (tap < p.taps) {
-                        mbar_expect_tx(fb, FT_A_BYTES);
-                        tma_load_im2col(smem_base + (uint32_t)(slot * G + ti) * FT_A_BYTES, &map_a, fb, 0, ow * p.stride - p.pad,
-                                        oh * p.stride - p.pad, img, (uint16_t)sx, (uint16_t)r);
-                        have_last = true;
-                        last_slot = slot;
-                        last_par = (uint32_t)(use & 1);
-                    } else {
-                        mbar_arrive(fb);        // a tap the last group does not have
+                    warp_expect_tx(fb, (uint32_t)n * FT_A_BYTES);
+                    uint32_t dst = smem_base + (uint32_t)(slot * G) * FT_A_BYTES;
+                    for (int t = 0; t < n; ++t, dst += FT_A_BYTES) {
+                        tma_load_im2col(dst, &map_a, fb, 0, base_w, base_h, img, (uint16_t)sx, (uint16_t)r, lane == ((slot * G + t) & 31));
+                        if (++sx == p.kw) { sx = 0; ++r; }
                     }
+                    have_last = true;
+                    last_slot = slot;
+                    last_par = par;
                 }
+                tap += n;
+                if (++slot == p.stages) { slot = 0; par ^= 1u; }
             }
-            if (!ok) break;
         }
         if (!ok && have_last) {
             const unsigned long long t0 = clock64();
@@ -280,38 +271,38 @@ f8_conv_pw_fused_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __gr
         }
     } else if (warp == FT_MOVER_WARP) {
         // ------------------------------------------------------------------ output mover
-        if (lane == 0) {
+        {
             grid_dependency_wait();
             int b = 0;
             uint32_t bphase = 0;
             for (int l = 0; l < n_local; ++l) {
                 const int m0 = (worker + l * n_workers) * FT_TILE_M;
-                if (!mbar_wait(out_full + 8 * b, bphase, wc, tagbits | 208)) break;
+                if (!warp_wait(out_full + 8 * b, bphase, wc, tagbits | 208)) break;
                 const uint32_t src = smem_base + p.out_off + (uint32_t)b * FT_OUT_BYTES;
                 tma_store_2d(&map_y, src, 0, m0);
                 tma_store_2d(&map_y, src + FT_TILE_M * 128, 128, m0);
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                mbar_arrive(out_free + 8 * b);
+                tma_store_commit();
+                tma_store_wait_read();
+                warp_arrive(out_free + 8 * b);
                 if (++b == p.out_bufs) { b = 0; bphase ^= 1; }
             }
-            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+            tma_store_wait();
         }
     } else if (warp == FT_FETCH_WARP) {
         // ------------------------------------------------------------------ shortcut fetcher
-        if (RES && lane == 0) {
+        if (RES) {
             grid_dependency_wait();
             int rb = 0, l = 0;
             uint32_t rphase = 0;
             bool ok = true;
             for (; l < n_local; ++l) {
                 const int m0 = (worker + l * n_workers) * FT_TILE_M;
-                if (!mbar_wait(out_free + 8 * rb, rphase ^ 1u, wc, tagbits | 207)) { ok = false; break; }
+                if (!warp_wait(out_free + 8 * rb, rphase ^ 1u, wc, tagbits | 207)) { ok = false; break; }
                 const uint32_t fb = res_full + 8 * rb;
                 const uint32_t dst = smem_base + p.out_off + (uint32_t)rb * FT_OUT_BYTES;
-                mbar_expect_tx(fb, FT_OUT_BYTES);
-                tma_load_2d(dst, &map_r, fb, 0, m0);
-                tma_load_2d(dst + FT_TILE_M * 128, &map_r, fb, 128, m0);
+                warp_expect_tx(fb, FT_OUT_BYTES);
+                tma_load_2d(dst, &map_r, fb, 0, m0, lane == 0);
+                tma_load_2d(dst + FT_TILE_M * 128, &map_r, fb, 128, m0, lane == 1);
                 if (++rb == p.out_bufs) { rb = 0; rphase ^= 1; }
             }
             if (!ok) {

@@ -132,9 +132,9 @@ struct TcParams {
     uint32_t swz_mask;        // 7, 3, 1 or 0: address bits 7.. XORed into the 16-byte chunk index
     uint32_t out_bytes;       // TILE_M * bn
     int out_bufs;             // staged output tiles in the ring (2..MAX_OUT_BUFS)
+    uint32_t ktab_off;        // table of k-iteration coordinates (8 bytes each)
     uint32_t out_off, bias_off;   // byte offsets behind the stages: two output tiles, two residual
                                            // tiles, int32 bias' of all padded columns
-    uint32_t ktab_off;        // table of k-iteration coordinates (8 bytes each)
     F8Requant q;
     F8Sibling sib;            // second consumer of the same sums (generic epilogue only)
     int vec_bytes2;           // widest aligned store of the second output's rows
@@ -271,7 +271,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     const int warp = uniform((int)(threadIdx.x >> 5));
     const int lane = threadIdx.x & 31;
     // persistent workers: CTAs, or CTA pairs (rank 0 = the even CTA, which owns the stage barriers and issues the MMAs)
-    const uint32_t cta_rank = PAIR ? cluster_cta_rank() : 0u;
+    const uint32_t cta_rank = PAIR ? uniform(cluster_cta_rank()) : 0u;
     const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
     const int n_workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     const uint32_t full_bar = smem_u32(&bars[0]);
@@ -345,6 +345,9 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         // There is no per-k-iteration loop (a single warp spends a few hundred cycles of loop overhead per
         // iteration, which used to bound layers with many short k-iterations), and consecutive loads sit in
         // different per-thread TMA queues, so they overlap.
+        // (One lane per load, each with its own coordinates, beats a convergent loop over the loads with uniform operands here:
+        // such a loop waits for a load to be accepted before it reuses the registers -- 3x3 64 -> 64 at 56 x 56, batch 64, 20.5
+        // against 28.7 us.  With one load per stage use, below, and in the stores the convergent form wins.)
         const uint2 *ktab = (const uint2 *)(smem + p.ktab_off);
         const int opnd = (warp == A_PROD_WARP || warp == A2_PROD_WARP) ? 0 : 1;
         const int half = (warp == A2_PROD_WARP || warp == B2_PROD_WARP) ? 1 : 0;      // which uses this warp takes (p.alt)
@@ -353,20 +356,17 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             // Resident weights: when all B tiles fit beside the pipeline, they are loaded once and every tile
             // of this CTA reuses them; the stages then carry activations only (the weight re-reads are what
             // saturates the L2 -> SM path of layers with few output channels).
-            const int n_loads = p.n_tiles * k_iters;
-            if (lane == 0) mbar_expect_tx(bres_bar, (uint32_t)n_loads * p.tx_b);
-            __syncwarp();
-            for (int i = lane; i < n_loads; i += 32) {
-                const int n_t = i / k_iters, k = i - n_t * k_iters;
-                const uint2 e = ktab[k];
-                tma_load_3d(smem_base + p.bres_off + (uint32_t)i * p.b_bytes, &map_b, bres_bar, (int)e.x, (int)(e.y >> 16),
-                            n_t * p.bn);
-            }
+            warp_expect_tx(bres_bar, (uint32_t)(p.n_tiles * k_iters) * p.tx_b);
+            uint32_t dst = smem_base + p.bres_off;
+            int turn = 0;
+            for (int n_t = 0; n_t < p.n_tiles; ++n_t)
+                for (int tap = 0; tap < p.kh * p.kw; ++tap)
+                    for (int cc = 0; cc < p.c_chunks; ++cc, ++turn, dst += p.b_bytes)
+                        tma_load_3d(dst, &map_b, bres_bar, cc * p.kb, tap, n_t * p.bn, lane == (turn & 31));
         }
         {
         // With resident weights the weight warp has nothing left to request: it takes the odd sub-chunks of
-        // the activation loads off the activation warp (issuing a TMA instruction holds a warp for a few
-        // hundred cycles per participating lane, which otherwise bounds layers with short tiles).
+        // the activation loads off the activation warp.
         const bool a_helper = opnd == 1 && p.b_res;
         const int j_mask = p.b_res ? 1 : 0, j_want = a_helper ? 1 : 0;     // which sub-chunks this warp requests
         if (opnd == 0 || a_helper) grid_dependency_wait();      // activations come from the previous grid; weights do not
@@ -374,27 +374,22 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         uint32_t phase = 0;
         bool have_last = false;
         int last_stage = 0;
-        uint32_t last_phase = 0;            // stage / phase of this lane's most recent load (for the drain on abort)
+        uint32_t last_phase = 0;            // stage / phase of this warp's most recent load (for the drain on abort)
         bool ok = true;
         if (p.win) {
-            // one load per (tile, channel chunk): the padded rows of the band, requested by the lane that owns the stage
+            // one load per (tile, channel chunk): the padded rows of the band
             for (int tile = worker; ok && opnd == 0 && tile < total_tiles; tile += n_workers) {
                 const int m_t = fast_div(tile, p.div_n_tiles);
                 const int img = fast_div(m_t, p.div_bands);
                 const int y0 = (m_t - img * p.win_bands) * p.win_r;
                 for (int cc = 0; cc < p.c_chunks; ++cc) {
-                    if (!__all_sync(0xffffffffu, mbar_wait(empty_bar + 8 * stage, phase ^ 1, wc, tagbits | 101))) {
-                        ok = false;
-                        break;
-                    }
-                    if (lane == (stage & 31)) {
-                        const uint32_t fb = full_bar + 8 * stage;
-                        mbar_expect_tx(fb, p.tx_win);
-                        tma_load_4d(smem_base + stage * p.stage_bytes, &map_a, fb, cc * p.kb, -1, y0 - 1, img);
-                        have_last = true;
-                        last_stage = stage;
-                        last_phase = phase;
-                    }
+                    if (!warp_wait(empty_bar + 8 * stage, phase ^ 1, wc, tagbits | 101)) { ok = false; break; }
+                    const uint32_t fb = full_bar + 8 * stage;
+                    warp_expect_tx(fb, p.tx_win);
+                    tma_load_4d(smem_base + stage * p.stage_bytes, &map_a, fb, cc * p.kb, -1, y0 - 1, img, lane == (stage & 31));
+                    have_last = true;
+                    last_stage = stage;
+                    last_phase = phase;
                     if (++stage == p.stages) { stage = 0; phase ^= 1; }
                 }
             }
@@ -402,31 +397,25 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             // one stage use per group of M tiles: sub-chunk j is the activation tile of M tile first + j (a single k-iteration
             // per tile; the weights are resident, so the two producer warps share the sub-chunks as usual)
             for (int tile = worker; ok && tile < total_tiles; tile += n_workers) {
-                if (!__all_sync(0xffffffffu, mbar_wait(empty_bar + 8 * stage, phase ^ 1, wc, tagbits | 101))) {
-                    ok = false;
-                    break;
-                }
+                if (!warp_wait(empty_bar + 8 * stage, phase ^ 1, wc, tagbits | 101)) { ok = false; break; }
                 const int first_m = tile * p.sup;
                 const int subs = min(p.sup, p.m_tiles - first_m);
                 const uint32_t fb = full_bar + 8 * stage;
-                if (lane == 0) {
-                    const uint32_t bytes = (uint32_t)(opnd == 0 ? (subs + 1) >> 1 : subs >> 1) * p.tx_a;
-                    if (bytes) mbar_expect_tx(fb, bytes);
-                    else mbar_arrive(fb);
-                }
-                __syncwarp();
-                const int j = (lane - stage * p.sup) & 31;
-                if (j < subs && (j & 1) == opnd) {
+                const uint32_t bytes = (uint32_t)(opnd == 0 ? (subs + 1) >> 1 : subs >> 1) * p.tx_a;
+                if (bytes) warp_expect_tx(fb, bytes);
+                else warp_arrive(fb);
+                for (int j = opnd; j < subs; j += 2) {
                     const int m0 = (first_m + j) * TILE_M;
                     const uint32_t dst = smem_base + stage * p.stage_bytes + j * p.a_bytes;
+                    const uint32_t on = lane == ((stage * p.sup + j) & 31);
                     if (p.a_plain) {
-                        tma_load_2d(dst, &map_a, fb, 0, m0);
+                        tma_load_2d(dst, &map_a, fb, 0, m0, on);
                     } else {
                         const int t1 = fast_div(m0, p.div_wo);
                         const int ow = m0 - t1 * p.wo;
                         const int img = fast_div(t1, p.div_ho);
                         const int oh = t1 - img * p.ho;
-                        tma_load_im2col(dst, &map_a, fb, 0, ow * p.stride_w - p.pad_w, oh * p.stride_h - p.pad_h, img, 0, 0);
+                        tma_load_im2col(dst, &map_a, fb, 0, ow * p.stride_w - p.pad_w, oh * p.stride_h - p.pad_h, img, 0, 0, on);
                     }
                     have_last = true;
                     last_stage = stage;
@@ -476,9 +465,9 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                     const uint2 e = ktab[kc + j];       // x: first channel of the chunk, y: tap << 16 | r << 8 | s
                     const uint32_t dst = smem_base + stage * p.stage_bytes + j * p.sub_bytes;
                     if (opnd == 0 || a_helper)
-                        tma_load_4d(dst, &map_a, fb, (int)e.x, base_w + (int)(e.y & 0xff), base_h + (int)((e.y >> 8) & 0xff), img);
+                        tma_load_4d(dst, &map_a, fb, (int)e.x, base_w + (int)(e.y & 0xff), base_h + (int)((e.y >> 8) & 0xff), img, 1u);
                     else
-                        tma_load_3d(dst + p.a_bytes, &map_b, fb, (int)e.x, (int)(e.y >> 16), n_base);
+                        tma_load_3d(dst + p.a_bytes, &map_b, fb, (int)e.x, (int)(e.y >> 16), n_base, 1u);
                     have_last = true;
                     last_stage = stage;
                     last_phase = phase;
@@ -533,20 +522,20 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                     if (PAIR) {
                         // this CTA's 128 rows of activations, its half of the weight tile; completion on the even CTA's barrier
                         if (opnd == 0 && p.a_plain)
-                            tma_load_2d_pair(dst, &map_a, fb, (int)e.x, m0);
+                            tma_load_2d_pair(dst, &map_a, fb, (int)e.x, m0, 1u);
                         else if (opnd == 0)
                             tma_load_im2col_pair(dst, &map_a, fb, (int)e.x, base_w, base_h, img, (uint16_t)(e.y & 0xff),
-                                                 (uint16_t)((e.y >> 8) & 0xff));
+                                                 (uint16_t)((e.y >> 8) & 0xff), 1u);
                         else
                             tma_load_3d_pair(dst + p.a_bytes, &map_b, fb, (int)e.x, (int)(e.y >> 16),
-                                             n_base + (int)cta_rank * (p.bn >> 1));
+                                             n_base + (int)cta_rank * (p.bn >> 1), 1u);
                     } else if ((opnd == 0 || a_helper) && p.a_plain)
-                        tma_load_2d(dst, &map_a, fb, (int)e.x, m0);
+                        tma_load_2d(dst, &map_a, fb, (int)e.x, m0, 1u);
                     else if (opnd == 0 || a_helper)
                         tma_load_im2col(dst, &map_a, fb, (int)e.x, base_w, base_h, img, (uint16_t)(e.y & 0xff),
-                                        (uint16_t)((e.y >> 8) & 0xff));
+                                        (uint16_t)((e.y >> 8) & 0xff), 1u);
                     else
-                        tma_load_3d(dst + p.a_bytes, &map_b, fb, (int)e.x, (int)(e.y >> 16), n_base);
+                        tma_load_3d(dst + p.a_bytes, &map_b, fb, (int)e.x, (int)(e.y >> 16), n_base, 1u);
                     have_last = true;
                     last_stage = stage;
                     last_phase = phase;
@@ -555,9 +544,11 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             }
         }
         if (!ok && have_last) {
-            // Drain: loads of one thread are served in order, so waiting (bounded) for the most recent one
-            // covers everything this lane has in flight before the CTA's shared memory goes away.
+            // Drain: wait about 0.2 ms for the loads of all lanes and (bounded) for the most recent one before the CTA's shared
+            // memory goes away.
             const unsigned long long t0 = clock64();
+            while ((unsigned long long)(clock64() - t0) < 400000ull) {
+            }
             while (!mbar_try_wait(full_bar + 8 * last_stage, last_phase) &&
                    (unsigned long long)(clock64() - t0) < DRAIN_LIMIT_CYCLES) {
             }
@@ -710,7 +701,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         }
     } else if (warp == MOVER_WARP) {
         // ------------------------------------------------------------------ output mover
-        if (STAGED && lane == 0) {
+        if (STAGED) {
             grid_dependency_wait();     // the output may overwrite a tensor the previous grid still reads
             // stores: a tile leaves from its buffer of the ring once all epilogue warps have written it
             int b = 0;
@@ -718,7 +709,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             for (int tile = worker; tile < total_tiles; tile += n_workers) {
                 const int m_q = fast_div(tile, p.div_n_tiles), n_t = tile - m_q * p.n_tiles;
             const int m_t = PAIR ? 2 * m_q + (int)cta_rank : m_q;
-                if (!mbar_wait(out_full + 8 * b, bphase, wc, tagbits | 108)) break;
+                if (!warp_wait(out_full + 8 * b, bphase, wc, tagbits | 108)) break;
                 const uint32_t src = smem_base + p.out_off + b * p.out_bytes;
                 if (SUP) {
                     // column slab sl of the staged tile is M tile tile * sup + sl
@@ -736,17 +727,17 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 for (int sl = 0; sl < p.n_slabs; ++sl)
                     if (n_t * p.bn + sl * p.slab_w < p.c_out)
                         tma_store_2d(&map_y, src + sl * (TILE_M * p.slab_w), n_t * p.bn + sl * p.slab_w, m_t * TILE_M);
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                tma_store_commit();
                 // the buffer is free again as soon as the store has read it (the next tiles use the others)
-                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-                mbar_arrive(out_free + 8 * b);
+                tma_store_wait_read();
+                warp_arrive(out_free + 8 * b);
                 if (++b == p.out_bufs) { b = 0; bphase ^= 1; }
             }
-            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+            tma_store_wait();
         }
     } else if (warp == FETCH_WARP) {
         // ------------------------------------------------------------------ residual fetcher
-        if (RES && lane == 0) {
+        if (RES) {
             grid_dependency_wait();
             // residual tiles go straight into the output ring (the epilogue converts them in place): a buffer is
             // loaded as soon as the store of the tile that used it before has read it, up to out_bufs - 1 tiles ahead
@@ -757,19 +748,19 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             for (int tile = worker; tile < total_tiles; tile += n_workers, ++local) {
                 const int m_q = fast_div(tile, p.div_n_tiles), n_t = tile - m_q * p.n_tiles;
             const int m_t = PAIR ? 2 * m_q + (int)cta_rank : m_q;
-                if (!mbar_wait(out_free + 8 * rb, rphase ^ 1, wc, tagbits | 106)) { ok = false; break; }
+                if (!warp_wait(out_free + 8 * rb, rphase ^ 1, wc, tagbits | 106)) { ok = false; break; }
                 const uint32_t fb = res_full + 8 * rb;
-                mbar_expect_tx(fb, p.tx_res);
+                warp_expect_tx(fb, p.tx_res);
                 if (p.rows) {
                     const int img = fast_div(m_t, p.div_bands);
                     const int y0 = (m_t - img * p.win_bands) * p.win_r;
                     for (int sl = 0; sl < p.n_slabs; ++sl)
                         tma_load_4d(smem_base + p.out_off + rb * p.out_bytes + sl * (TILE_M * p.slab_w), &map_r, fb,
-                                    n_t * p.bn + sl * p.slab_w, 0, y0, img);
+                                    n_t * p.bn + sl * p.slab_w, 0, y0, img, lane == sl);
                 } else
                 for (int sl = 0; sl < p.n_slabs; ++sl)
                     tma_load_2d(smem_base + p.out_off + rb * p.out_bytes + sl * (TILE_M * p.slab_w), &map_r, fb,
-                                n_t * p.bn + sl * p.slab_w, m_t * TILE_M);
+                                n_t * p.bn + sl * p.slab_w, m_t * TILE_M, lane == sl);
                 if (++rb == p.out_bufs) { rb = 0; rphase ^= 1; }
             }
             if (!ok && local > 0) {

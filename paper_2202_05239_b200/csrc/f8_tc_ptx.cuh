@@ -136,48 +136,79 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, const W
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, wc, code));
 }
 
+// The warps that issue MMAs and copies run their loops as a whole and one lane is elected at the instruction itself (always the
+// same one, so a commit covers the warp's earlier MMAs or stores).  In a loop that a single lane runs, the compiler has to
+// keep every address and descriptor word in that lane's registers and move each of them to the uniform registers these
+// instructions read; a convergent loop over values known to be uniform (uniform(), votes on the waits) lives there
+// throughout.  Measured on the first-layer kernel: 195 -> 130 cycles per MMA of 64 columns with the epilogue warps at work.
+// What says so below is executed by a whole warp.
+#define F8_ELECT ".reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
+
+// (whole warp) one arrival / one arrival that announces bytes
+__device__ __forceinline__ void warp_arrive(uint32_t bar) {
+    asm volatile("{\n\t" F8_ELECT "@e mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void warp_expect_tx(uint32_t bar, uint32_t bytes) {
+    asm volatile("{\n\t" F8_ELECT "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes) : "memory");
+    __syncwarp();       // the announcement comes before any lane's load
+}
+
+// Bulk tensor copies.  Stores: whole warp.  A load is issued by the lanes whose `on` is not zero.
+#define F8_ON(n) ".reg .pred e;\n\tsetp.ne.b32 e, " n ", 0;\n\t"
 __device__ __forceinline__ void tma_load_im2col(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c, int w,
-                                                int h, int n, uint16_t off_w, uint16_t off_h) {
+                                                int h, int n, uint16_t off_w, uint16_t off_h, uint32_t on) {
     asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};" ::"r"(dst),
-        "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(off_w), "h"(off_h)
+        "{\n\t" F8_ON("%9") "@e cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};\n\t}" ::"r"(dst),
+        "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"(off_w), "h"(off_h), "r"(on)
         : "memory");
 }
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1,
-                                            int c2) {
+                                            int c2, uint32_t on) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-        "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
+        "{\n\t" F8_ON("%6") "@e cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5}], [%2];\n\t}" ::"r"(dst),
+        "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(on)
         : "memory");
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1) {
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, uint32_t on) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
-        "l"(map), "r"(bar), "r"(c0), "r"(c1)
+        "{\n\t" F8_ON("%5") "@e cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4}], [%2];\n\t}" ::"r"(dst),
+        "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(on)
         : "memory");
 }
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2,
-                                            int c3) {
+                                            int c3, uint32_t on) {
     asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(dst),
-        "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+        "{\n\t" F8_ON("%7") "@e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2];\n\t}" ::"r"(dst),
+        "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(on)
         : "memory");
 }
 __device__ __forceinline__ void tma_store_4d(const CUtensorMap *map, uint32_t src, int c0, int c1, int c2, int c3) {
-    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(map), "r"(src),
+    asm volatile("{\n\t" F8_ELECT "@e cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];\n\t}" ::"l"(map), "r"(src),
                  "r"(c0), "r"(c1), "r"(c2), "r"(c3)
                  : "memory");
 }
 // shared -> global tile store; rows / columns outside the tensor are clipped by the hardware
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t src, int c0, int c1) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(map), "r"(src),
+    asm volatile("{\n\t" F8_ELECT "@e cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];\n\t}" ::"l"(map), "r"(src),
                  "r"(c0), "r"(c1)
                  : "memory");
+}
+
+// (whole warp) closes the group of the stores issued so far; waits until all groups have been read from shared memory / are
+// complete.  Groups belong to the thread that issued the stores, the elected one.
+__device__ __forceinline__ void tma_store_commit() { asm volatile("{\n\t" F8_ELECT "@e cp.async.bulk.commit_group;\n\t}" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait_read() {
+    asm volatile("{\n\t" F8_ELECT "@e cp.async.bulk.wait_group.read 0;\n\t}" ::: "memory");
+    __syncwarp();
+}
+__device__ __forceinline__ void tma_store_wait() {
+    asm volatile("{\n\t" F8_ELECT "@e cp.async.bulk.wait_group 0;\n\t}" ::: "memory");
+    __syncwarp();
 }
 
 // Brings a tensor map (a kernel parameter) into the descriptor cache ahead of its first use by a bulk tensor copy.
@@ -208,16 +239,9 @@ __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_
         : "memory");
 }
 
-// The MMA-issuing warps run their loops as a whole and one lane is elected at the instruction itself (always the same one, so
-// a commit covers the warp's earlier MMAs).  In a loop that a single lane runs, the compiler has to keep every address and
-// descriptor word in that lane's registers and move each of them to the uniform registers the instruction reads; a
-// convergent loop over values known to be uniform (uniform(), votes on the waits) lives there throughout.  Measured on the
-// first-layer kernel: 195 -> 130 cycles per instruction of 64 columns with the epilogue warps at work.
-//
 // The K = 32 slices of one sub-chunk (kb / 32 of them), issued from one asm block: the shared-memory descriptors of the slices
 // differ only in their low words (start address, 16-byte units), so those are advanced with 32-bit adds inside the block and
 // the constant high word (SBO, version, swizzle mode) is attached by a register-pair move.
-#define F8_ELECT ".reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\t"
 #define F8_MMA_I8 "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, "
 #define F8_MMA_NEXT(off) \
     "add.u32 x, %1, " #off ";\n\tadd.u32 y, %2, " #off ";\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %3};\n\t" F8_MMA_I8 "t;\n\t"
@@ -291,25 +315,25 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t rank)
 __device__ __forceinline__ uint32_t pair_leader_bar(uint32_t bar) { return bar & 0xFEFFFFFFu; }
 
 __device__ __forceinline__ void tma_load_im2col_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c, int w, int h,
-                                                     int n, uint16_t off_w, uint16_t off_h) {
+                                                     int n, uint16_t off_w, uint16_t off_h, uint32_t on) {
     asm volatile(
-        "cp.async.bulk.tensor.4d.im2col.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};" ::"r"(dst),
-        "l"(map), "r"(pair_leader_bar(bar)), "r"(c), "r"(w), "r"(h), "r"(n), "h"(off_w), "h"(off_h)
+        "{\n\t" F8_ON("%9") "@e cp.async.bulk.tensor.4d.im2col.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};\n\t}" ::"r"(dst),
+        "l"(map), "r"(pair_leader_bar(bar)), "r"(c), "r"(w), "r"(h), "r"(n), "h"(off_w), "h"(off_h), "r"(on)
         : "memory");
 }
-__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2) {
+__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2, uint32_t on) {
     asm volatile(
-        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(dst),
-        "l"(map), "r"(pair_leader_bar(bar)), "r"(c0), "r"(c1), "r"(c2)
+        "{\n\t" F8_ON("%6") "@e cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4, %5}], [%2];\n\t}" ::"r"(dst),
+        "l"(map), "r"(pair_leader_bar(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(on)
         : "memory");
 }
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1) {
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, uint32_t on) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
-        "l"(map), "r"(pair_leader_bar(bar)), "r"(c0), "r"(c1)
+        "{\n\t" F8_ON("%5") "@e cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%3, %4}], [%2];\n\t}" ::"r"(dst),
+        "l"(map), "r"(pair_leader_bar(bar)), "r"(c0), "r"(c1), "r"(on)
         : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t cols) {
