@@ -337,7 +337,7 @@ const char *f8_last_error(void);
  * abandoned a bounded wait (the word is cleared), F8_ERR_CUDA on a CUDA error, else F8_OK. */
 f8_status f8_device_status(void);
 
-/* Number of tensor-core (tcgen05) convolution kernels this process has launched so far; lets a
+/* Number of tensor-core convolution kernels (tcgen05; mma.sync for small layers of a network) this process has launched so far; lets a
  * caller confirm which path a layer took. */
 long long f8_tc_launch_count(void);
 
@@ -359,6 +359,7 @@ void f8_debug_force_direct(int on);
  *   F8_PLAN_OFF_STEM_POOL_FUSION  the max pool behind a first layer runs as its own kernel
  *   F8_PLAN_OFF_LAYER_OVERLAP     f8_net_forward launches without programmatic dependent launch
  *   F8_PLAN_OFF_LAYER_FUSION      f8_net_forward runs a 64 -> 64 convolution and the 64 -> 256 pointwise layer behind it as two launches
+ *   F8_PLAN_OFF_SMALL_KERNEL      f8_net_forward runs layers of a few microseconds on the tcgen05 kernel as well
  *   F8_PLAN_OFF_LANES             f8_net_forward runs the whole batch as one sequence of launches on the caller's stream
  *   F8_PLAN_SYNC_LAYERS           f8_net_forward synchronises after every launch, so that a device fault is
  *                                 reported with the layer that raised it */
@@ -366,7 +367,7 @@ enum {
     F8_PLAN_OFF_RESIDENT_WEIGHTS = 1, F8_PLAN_OFF_WINDOWED = 2, F8_PLAN_OFF_DUAL_ISSUE = 4, F8_PLAN_OFF_ALT_PRODUCERS = 8,
     F8_PLAN_OFF_PAIRS = 16, F8_PLAN_OFF_DW_WALK = 32, F8_PLAN_OFF_STEM_KERNEL = 64, F8_PLAN_OFF_STEM_POOL_FUSION = 128,
     F8_PLAN_OFF_LAYER_OVERLAP = 256, F8_PLAN_OFF_LANES = 512, F8_PLAN_SYNC_LAYERS = 1024, F8_PLAN_OFF_DW_DP4A = 2048,
-    F8_PLAN_OFF_TILE_GROUPS = 4096, F8_PLAN_OFF_LAYER_FUSION = 8192
+    F8_PLAN_OFF_TILE_GROUPS = 4096, F8_PLAN_OFF_LAYER_FUSION = 8192, F8_PLAN_OFF_SMALL_KERNEL = 16384
 };
 void f8_debug_plan_options(unsigned off_mask);
 

@@ -485,6 +485,7 @@ struct Step {
     const void *res = nullptr;
     void *y = nullptr;
     bool use_tc = false;
+    bool small = false;       // use_tc: the kernel for layers of a few microseconds (no plan)
     bool fused_pool = false;  // kind -2: the stem kernel also computes the max pool that follows (layer + 1)
     bool has_sib = false;     // the launch also writes the output of the sibling layer behind it (layer + 1)
     F8Sibling sib;
@@ -1246,6 +1247,8 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                                return true;
                            }()) {
                     // planned above
+                } else if (!(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) && f8_small_tc_wanted(stp.g)) {
+                    stp.use_tc = stp.small = true;
                 } else if (f8_tc_supported(stp.g, (size_t)n * L.g.h * L.g.w * L.g.c)) {
                     PlanPtr plan = alloc_plan();
                     if (plan && f8_tc_plan_init(plan.get(), stp.g, L.q, dense_view(stp.x, stp.g), L.w, L.b, stp.res,
@@ -1339,7 +1342,10 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
             case F8_LAYER_LINEAR:
                 // the net owns its weights (uploaded at creation), so a layer's prologue and weight loads may
                 // overlap the tail of the previous layer
-                if (stp.use_tc) { e = f8_tc_launch(stp.plan.get(), net->overlap_layers, st); ++g_tc_launches; }
+                if (stp.small) {
+                    e = f8_launch_small_tc(stp.g, L.q, stp.x, L.w, L.b, stp.res, stp.y, st, net->overlap_layers, stp.has_sib ? &stp.sib : nullptr);
+                    ++g_tc_launches;
+                } else if (stp.use_tc) { e = f8_tc_launch(stp.plan.get(), net->overlap_layers, st); ++g_tc_launches; }
                 else e = f8_launch_conv_direct(stp.g, L.q, stp.x, L.w, L.b, stp.res, stp.y, st, net->overlap_layers,
                                                stp.has_sib ? &stp.sib : nullptr);
                 break;

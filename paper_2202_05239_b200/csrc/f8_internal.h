@@ -110,6 +110,14 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
                               const void *x, const int8_t *w_core, const int32_t *bias, void *y, int *status_word, int tag,
                               cudaStream_t st, bool overlap_previous);
 
+// ---- small layers (f8_small_tc.cu): implicit GEMM on mma.sync for layers bound by latency; every output kind, shortcut and
+// sibling; c a multiple of 16, c_out of 4, weights, bias, shortcut and outputs 16-byte aligned.  `wanted`: the rule by which a
+// network prefers it to the tcgen05 kernel.
+bool f8_small_tc_supported(const F8ConvGeom &g);
+bool f8_small_tc_wanted(const F8ConvGeom &g);
+cudaError_t f8_launch_small_tc(const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
+                               const void *res, void *y, cudaStream_t st, bool overlap_previous, const F8Sibling *sib = nullptr);
+
 // Device status word (0 = fine); allocated once per device on first use, together with a host-visible copy of its
 // first word that kernels write through (f8_status_host_code reads it without synchronising).
 int *f8_status_word();

@@ -1,0 +1,50 @@
+"""GPU parity (bit-exact) of the kernel for layers of a few microseconds (mma.sync implicit GEMM), which f8_net_forward
+takes for small dense layers: networks of one or two layers at the edges of its tiles and of its K chunks."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2202_05239_b200 import synth
+from gpu_util import Guarded, api, assert_equal_arrays, random_conv_layer, random_input
+
+pytestmark = pytest.mark.gpu
+
+# (h, w, c, c_out, k, stride, pad, n, x_signed, y_dtype, with_res)
+CASES = [
+    (1, 1, 2048, 1000, 1, 1, 0, 1, False, synth.S32, False),     # a fully connected layer for one image
+    (1, 1, 48, 16, 1, 1, 0, 33, True, synth.U8, False),          # 33 rows: one row in the second tile; K of 48 bytes
+    (14, 14, 256, 256, 3, 1, 1, 1, False, synth.U8, True),       # 18 chunks through the eight-stage ring; shortcut
+    (7, 9, 16, 48, 3, 2, 1, 3, True, synth.S8, False),           # one unit per tap: a chunk spans eight taps; ragged columns
+    (15, 17, 80, 112, 5, 1, 2, 1, False, synth.U8, False),       # chunks straddle taps (80 of 128 bytes)
+    (31, 29, 32, 64, 1, 2, 0, 2, False, synth.S8, False),        # strided 1x1
+    (56, 56, 64, 256, 1, 1, 0, 1, False, synth.U8, True),        # 64 x 64 tiles
+    (40, 41, 96, 272, 1, 1, 0, 2, True, synth.S8, True),         # 64 x 64 tiles, ragged in both directions
+]
+
+
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_small_layer(ref, case):
+    h, w, c, c_out, k, stride, pad, n, xs, y_dtype, with_res = CASES[case]
+    rng = np.random.default_rng(2100 + case)
+    layer = random_conv_layer(rng, h=h, w=w, c=c, c_out=c_out, k=k, stride=stride, pad=pad, x_signed=xs, y_dtype=y_dtype, with_res=with_res)
+    layers = [layer]
+    if with_res:      # the shortcut comes from a second layer over the same image
+        short = random_conv_layer(rng, h=h, w=w, c=c, c_out=c_out, k=k, stride=stride, pad=pad, x_signed=xs, y_dtype=layer.r_dtype,
+                                  with_res=False, fl_x=layer.fl_x)
+        short.fl_y = layer.fl_r
+        layer.res = 1
+        layers = [short, layer]
+    a = api()
+    x = random_input(rng, n, layers[0])
+    want = ref.net_forward(layers, x)
+    net = a.Net(layers, n)
+    guards = [Guarded((n, l.ho, l.wo, l.c_out), a.torch_dtype(l.y_dtype)) for l in layers]
+    before = a.f8_tc_launch_count()
+    net.forward(a.to_device(x), dump=[g.t for g in guards])
+    torch.cuda.synchronize()
+    a.f8_device_status()
+    assert a.f8_tc_launch_count() - before == len(layers)
+    for i, g in enumerate(guards):
+        assert g.intact()
+        assert_equal_arrays(g.t.cpu().numpy().reshape(want[i + 1].shape), want[i + 1], f"layer {i}: ")
+    net.close()
