@@ -58,3 +58,19 @@ def test_private_formats_versus_realigning_one_tensor(ref):
     unclipped = y_f.cpu().numpy() < 255
     assert np.max(np.abs(direct - twice)[unclipped]) <= 1
     assert np.any(direct != twice)          # the double rounding is visible: the readings are not identical
+
+
+@pytest.mark.parametrize("n,offset", [(16, 0), (15, 0), (4097, 0), (70001, 1), (4096 * 3 + 16, 8), (200, 4)])
+def test_requantize_dual_edges(ref, n, offset):
+    """Block and thread edges, the ragged tail, and tensors that start off the vector alignment (offset elements)."""
+    a = api()
+    rng = np.random.default_rng(n + offset)
+    acc = rng.integers(-(1 << 31), 1 << 31, size=n + offset).astype(np.int32)
+    accd = a.to_device(acc)[offset:]
+    y1 = torch.zeros(n + offset + 32, dtype=torch.int8, device="cuda")
+    y2 = torch.zeros(n + offset + 32, dtype=torch.uint8, device="cuda")
+    a.f8_requantize_dual_fixed(accd, 24, y1[offset:offset + n], synth.S8, 0, y2[offset:offset + n], synth.U8, 1)
+    torch.cuda.synchronize()
+    assert np.array_equal(y1[offset:offset + n].cpu().numpy().astype(np.int64), _want(ref, acc[offset:], 24, 0, synth.S8))
+    assert np.array_equal(y2[offset:offset + n].cpu().numpy().astype(np.int64), _want(ref, acc[offset:], 24, 1, synth.U8))
+    assert not y1[offset + n:].any() and not y2[offset + n:].any() and not y1[:offset].any()
