@@ -13,103 +13,151 @@
 // powers of two is exact, and floor(log2(r)) is taken from the exponent of r.  Only the summation order of the
 // variance is free; it is fixed too (per-block partial sums reduced in index order), so results are reproducible.
 //
-// The work is four small launches: row scales -> partial sums -> format and bias -> quantised weights.  It is bound by memory
-// traffic: the fp32 weights are read twice and one byte per weight is written.
+// Two launches: partial sums; then format, bias and quantised weights.  Every block of the second adds the partial sums up again
+// (at most 16 KB out of L2) instead of waiting for a launch of its own that does, and has its first weights in registers before
+// the first launch has finished (programmatic dependent launch).  A block takes 4096 consecutive weights of the whole tensor
+// at a time, whatever rows they belong to, so rows that are no multiple of that leave no block with a remainder.  The
+// fp32 weights are read twice (the second time from L2 up to about 30 M weights) and one byte per weight is written.
+// [512 x 4608]: 23.6 us (four launches, chunks of rows) -> 14.2 us, of which the host needs 14 to enqueue.
 #include <math.h>
+
+#include <algorithm>
 
 #include "f8_internal.h"
 
 namespace {
 
 constexpr int FOLD_THREADS = 256;
-constexpr int FOLD_CHUNK = 4096;         // weights of one row handled by one block iteration
+constexpr int FOLD_CHUNK = 4096;         // weights a block takes at a time
+constexpr int FOLD_PER_THREAD = FOLD_CHUNK / FOLD_THREADS;
 constexpr int FOLD_MAX_BLOCKS = 1024;
+constexpr int FOLD_MAX_ROWS = 1024;      // row scales a block keeps in shared memory (a chunk of shorter rows divides per weight)
 
 struct FoldParams {
     int c_out, k;
-    int chunks_per_row;
-    long long items;                      // c_out * chunks_per_row
+    long long n;                          // c_out * k
+    int blocks;
     double ratio;                         // eta_in / eta_out
     double eta_out;
     int fl_x, fl_min, fl_max;
-    int vec4;                             // k % 4 == 0 and w 16-byte, w_q 4-byte aligned: four weights per thread and access
     const float *w, *gamma, *sigma, *beta, *mu;
     int8_t *w_q;
     int32_t *b_q;
     int *fl_w;
-    double *partial;                      // [blocks][2], then [2]: mean, std
-    double *scale;                        // [c_out]: (gamma / sigma) * ratio, written by the first launch
+    double *partial;                      // [blocks][2]
 };
 
-__global__ void __launch_bounds__(FOLD_THREADS) fold_scale_kernel(const FoldParams p) {
-    const int i = blockIdx.x * FOLD_THREADS + threadIdx.x;
-    if (i < p.c_out) p.scale[i] = __dmul_rn(__ddiv_rn((double)__ldg(p.gamma + i), (double)__ldg(p.sigma + i)), p.ratio);
+__device__ __forceinline__ double row_scale(const FoldParams &p, int row) {
+    return __dmul_rn(__ddiv_rn((double)__ldg(p.gamma + row), (double)__ldg(p.sigma + row)), p.ratio);
 }
 
-__device__ __forceinline__ double row_scale(const FoldParams &p, int row) { return p.scale[row]; }
+// Scales of the rows the chunk at e0 touches, once per chunk (false: too many rows for the table).
+__device__ __forceinline__ bool stage_scales(const FoldParams &p, long long e0, double *sc, int *row0) {
+    const int r0 = (int)(e0 / p.k), r1 = (int)((min(e0 + FOLD_CHUNK, p.n) - 1) / p.k);
+    *row0 = r0;
+    const bool fits = r1 - r0 < FOLD_MAX_ROWS;
+    __syncthreads();                      // the previous chunk's scales have been used
+    if (fits)
+        for (int i = threadIdx.x; i <= r1 - r0; i += FOLD_THREADS) sc[i] = row_scale(p, r0 + i);
+    __syncthreads();
+    return fits;
+}
 
+// The 16 weights of this thread in the chunk at e0.  VEC: k is a multiple of four (a group of four lies in one row) and w is
+// 16-byte aligned: groups of four, 1024 weights apart; else single weights, 256 apart.
+template <bool VEC>
+__device__ __forceinline__ long long fold_index(long long e0, int j) {
+    return VEC ? e0 + (long long)(j >> 2) * (4 * FOLD_THREADS) + 4 * threadIdx.x + (j & 3) : e0 + (long long)j * FOLD_THREADS + threadIdx.x;
+}
+template <bool VEC>
+__device__ __forceinline__ void load_weights(const FoldParams &p, long long e0, float (&f)[FOLD_PER_THREAD]) {
+    if (VEC) {
+#pragma unroll
+        for (int g = 0; g < FOLD_PER_THREAD / 4; ++g) {
+            const long long e = fold_index<true>(e0, 4 * g);
+            const float4 t = e < p.n ? __ldg((const float4 *)(p.w + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            f[4 * g] = t.x; f[4 * g + 1] = t.y; f[4 * g + 2] = t.z; f[4 * g + 3] = t.w;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < FOLD_PER_THREAD; ++j) {
+            const long long e = fold_index<false>(e0, j);
+            f[j] = e < p.n ? __ldg(p.w + e) : 0.f;
+        }
+    }
+}
+// Scale of weight j of this thread (groups of four share one when VEC).
+template <bool VEC>
+__device__ __forceinline__ double weight_scale(const FoldParams &p, long long e0, int j, bool table, const double *sc, int row0) {
+    const long long e = fold_index<VEC>(e0, j);
+    if (e >= p.n) return 0.0;
+    const int row = (int)((uint32_t)e / (uint32_t)p.k);              // n < 2^31
+    return table ? sc[row - row0] : row_scale(p, row);
+}
+
+// Adds s1, s2 over the block in a fixed order; the result is in every thread.
+__device__ __forceinline__ void block_sum(double &s1, double &s2) {
+    __shared__ double r1[FOLD_THREADS / 32], r2[FOLD_THREADS / 32];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, d);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, d);
+    }
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) { r1[threadIdx.x >> 5] = s1; r2[threadIdx.x >> 5] = s2; }
+    __syncthreads();
+    s1 = s2 = 0.0;
+#pragma unroll
+    for (int i = 0; i < FOLD_THREADS / 32; ++i) { s1 += r1[i]; s2 += r2[i]; }
+}
+
+template <bool VEC>
 __global__ void __launch_bounds__(FOLD_THREADS) fold_stats_kernel(const FoldParams p) {
+    __shared__ double sc[FOLD_MAX_ROWS];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     double s1 = 0.0, s2 = 0.0;
-    for (long long item = blockIdx.x; item < p.items; item += gridDim.x) {
-        const int row = (int)(item / p.chunks_per_row), chunk = (int)(item - (long long)row * p.chunks_per_row);
-        const double sc = row_scale(p, row);
-        const float *wr = p.w + (size_t)row * p.k;
-        const int j1 = min(p.k, (chunk + 1) * FOLD_CHUNK);
-        if (p.vec4) {       // rows are multiples of four weights and 16-byte aligned: one 16-byte load per thread
-            for (int j = chunk * FOLD_CHUNK + 4 * threadIdx.x; j < j1; j += 4 * FOLD_THREADS) {
-                const float4 f = __ldg((const float4 *)(wr + j));
-                const double v0 = __dmul_rn(sc, (double)f.x), v1 = __dmul_rn(sc, (double)f.y);
-                const double v2 = __dmul_rn(sc, (double)f.z), v3 = __dmul_rn(sc, (double)f.w);
-                s1 += (v0 + v1) + (v2 + v3);
-                s2 += (v0 * v0 + v1 * v1) + (v2 * v2 + v3 * v3);
-            }
-        } else
-        for (int j = chunk * FOLD_CHUNK + threadIdx.x; j < j1; j += FOLD_THREADS) {
-            const double v = __dmul_rn(sc, (double)__ldg(wr + j));
+    for (long long e0 = (long long)blockIdx.x * FOLD_CHUNK; e0 < p.n; e0 += (long long)gridDim.x * FOLD_CHUNK) {
+        float f[FOLD_PER_THREAD];
+        load_weights<VEC>(p, e0, f);
+        int row0;
+        const bool table = stage_scales(p, e0, sc, &row0);
+        double scale = 0.0;
+#pragma unroll
+        for (int j = 0; j < FOLD_PER_THREAD; ++j) {
+            if (!VEC || (j & 3) == 0) scale = weight_scale<VEC>(p, e0, j, table, sc, row0);
+            const double v = __dmul_rn(scale, (double)f[j]);
             s1 += v;
             s2 += v * v;
         }
     }
-    // block reduction in a fixed order
-    __shared__ double r1[FOLD_THREADS], r2[FOLD_THREADS];
-    r1[threadIdx.x] = s1;
-    r2[threadIdx.x] = s2;
-    __syncthreads();
-    for (int step = FOLD_THREADS / 2; step > 0; step >>= 1) {
-        if ((int)threadIdx.x < step) {
-            r1[threadIdx.x] += r1[threadIdx.x + step];
-            r2[threadIdx.x] += r2[threadIdx.x + step];
-        }
-        __syncthreads();
-    }
+    block_sum(s1, s2);
     if (threadIdx.x == 0) {
-        p.partial[2 * blockIdx.x] = r1[0];
-        p.partial[2 * blockIdx.x + 1] = r2[0];
+        p.partial[2 * blockIdx.x] = s1;
+        p.partial[2 * blockIdx.x + 1] = s2;
     }
 }
 
-__global__ void __launch_bounds__(FOLD_THREADS) fold_format_kernel(const FoldParams p, const int blocks) {
-    __shared__ double r1[FOLD_THREADS], r2[FOLD_THREADS];
+template <bool VEC>
+__global__ void __launch_bounds__(FOLD_THREADS) fold_quant_kernel(const FoldParams p) {
+    __shared__ double sc[FOLD_MAX_ROWS];
     __shared__ int fl_s;
+    // the inputs were complete before the first launch started; what that launch writes is read behind the wait
+    long long e0 = (long long)blockIdx.x * FOLD_CHUNK;
+    float f[FOLD_PER_THREAD];
+    load_weights<VEC>(p, e0, f);
+    int row0;
+    bool table = stage_scales(p, e0, sc, &row0);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     double s1 = 0.0, s2 = 0.0;
-    for (int b = threadIdx.x; b < blocks; b += FOLD_THREADS) {
+    for (int b = threadIdx.x; b < p.blocks; b += FOLD_THREADS) {
         s1 += p.partial[2 * b];
         s2 += p.partial[2 * b + 1];
     }
-    r1[threadIdx.x] = s1;
-    r2[threadIdx.x] = s2;
-    __syncthreads();
-    for (int step = FOLD_THREADS / 2; step > 0; step >>= 1) {
-        if ((int)threadIdx.x < step) {
-            r1[threadIdx.x] += r1[threadIdx.x + step];
-            r2[threadIdx.x] += r2[threadIdx.x + step];
-        }
-        __syncthreads();
-    }
+    block_sum(s1, s2);
     if (threadIdx.x == 0) {
-        const double n = (double)p.c_out * (double)p.k;
-        const double mean = r1[0] / n;
-        double var = r2[0] / n - mean * mean;
+        const double n = (double)p.n;
+        const double mean = s1 / n;
+        double var = s2 / n - mean * mean;
         if (!(var > 0.0)) var = 0.0;
         const double sd = sqrt(var);
         int fl = p.fl_max;                                   // a constant tensor: the finest format allowed
@@ -119,52 +167,60 @@ __global__ void __launch_bounds__(FOLD_THREADS) fold_format_kernel(const FoldPar
         }
         fl = max(p.fl_min, min(p.fl_max, fl));
         fl_s = fl;
-        *p.fl_w = fl;
-        p.partial[2 * blocks] = mean;
-        p.partial[2 * blocks + 1] = sd;
+        if (blockIdx.x == 0) *p.fl_w = fl;
     }
     __syncthreads();
-    const int fa = p.fl_x + fl_s;
-    for (int i = threadIdx.x; i < p.c_out; i += FOLD_THREADS) {
+    const int fl = fl_s;
+    const double pow2 = scalbn(1.0, fl);          // multiplying by a power of two is exact
+    const int fa = p.fl_x + fl;
+    for (int i = (int)(blockIdx.x * FOLD_THREADS + threadIdx.x); i < p.c_out; i += (int)gridDim.x * FOLD_THREADS) {
         const double gs = __ddiv_rn((double)__ldg(p.gamma + i), (double)__ldg(p.sigma + i));
         const double be = __ddiv_rn(__dsub_rn((double)__ldg(p.beta + i), __dmul_rn(gs, (double)__ldg(p.mu + i))), p.eta_out);
         double t = floor(__dadd_rn(scalbn(be, fa), 0.5));
         t = fmin(fmax(t, -2147483648.0), 2147483647.0);
         p.b_q[i] = (int32_t)t;
     }
-}
-
-__global__ void __launch_bounds__(FOLD_THREADS) fold_quant_kernel(const FoldParams p) {
-    const int fl = *p.fl_w;
-    const double pow2 = scalbn(1.0, fl);          // multiplying by a power of two is exact
-    for (long long item = blockIdx.x; item < p.items; item += gridDim.x) {
-        const int row = (int)(item / p.chunks_per_row), chunk = (int)(item - (long long)row * p.chunks_per_row);
-        const double sc = row_scale(p, row);
-        const float *wr = p.w + (size_t)row * p.k;
-        int8_t *qr = p.w_q + (size_t)row * p.k;
-        const int j1 = min(p.k, (chunk + 1) * FOLD_CHUNK);
-        if (p.vec4) {
-            for (int j = chunk * FOLD_CHUNK + 4 * threadIdx.x; j < j1; j += 4 * FOLD_THREADS) {
-                const float4 f = __ldg((const float4 *)(wr + j));
-                const float in[4] = {f.x, f.y, f.z, f.w};
-                uint32_t packed = 0;
+    while (true) {
+        double scale = 0.0;
+        uint32_t packed = 0;
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                    const double v = __dmul_rn(__dmul_rn(sc, (double)in[t]), pow2);
-                    const int q = (int)floor(__dadd_rn(fmin(fmax(v, -127.0), 127.0), 0.5));
-                    packed |= (uint32_t)(q & 0xff) << (8 * t);
+        for (int j = 0; j < FOLD_PER_THREAD; ++j) {
+            if (!VEC || (j & 3) == 0) scale = weight_scale<VEC>(p, e0, j, table, sc, row0);
+            // floor is monotone and the bounds are whole numbers: clipping behind it is clipping in front of it
+            const double v = __dmul_rn(__dmul_rn(scale, (double)f[j]), pow2);
+            const int q = min(max(__double2int_rd(__dadd_rn(v, 0.5)), -127), 127);
+            const long long e = fold_index<VEC>(e0, j);
+            if (VEC) {
+                packed |= (uint32_t)(q & 0xff) << (8 * (j & 3));
+                if ((j & 3) == 3) {
+                    if (e < p.n) *(uint32_t *)(p.w_q + e - 3) = packed;
+                    packed = 0;
                 }
-                *(uint32_t *)(qr + j) = packed;
+            } else if (e < p.n) {
+                p.w_q[e] = (int8_t)q;
             }
-        } else
-        for (int j = chunk * FOLD_CHUNK + threadIdx.x; j < j1; j += FOLD_THREADS) {
-            const double v = __dmul_rn(__dmul_rn(sc, (double)__ldg(wr + j)), pow2);
-            qr[j] = (int8_t)(int)floor(__dadd_rn(fmin(fmax(v, -127.0), 127.0), 0.5));
         }
+        e0 += (long long)gridDim.x * FOLD_CHUNK;
+        if (e0 >= p.n) break;
+        load_weights<VEC>(p, e0, f);
+        table = stage_scales(p, e0, sc, &row0);
     }
 }
 
-int fold_blocks(long long items) { return (int)std::min<long long>(items, FOLD_MAX_BLOCKS); }
+template <bool VEC>
+cudaError_t launch_fold(const FoldParams &p, cudaStream_t st) {
+    fold_stats_kernel<VEC><<<p.blocks, FOLD_THREADS, 0, st>>>(p);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)p.blocks);
+    cfg.blockDim = dim3(FOLD_THREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fold_quant_kernel<VEC>, p);
+}
 
 }   // namespace
 
@@ -188,22 +244,16 @@ f8_status f8_fold_quantize_fixed(const f8_fold_desc *d, const float *w, const fl
         return f8_set_error(F8_ERR_ALIGN, "workspace must be 8-byte aligned, w / bias_q / fl_w 4-byte aligned");
     FoldParams p;
     p.c_out = d->c_out; p.k = d->k;
-    p.chunks_per_row = (d->k + FOLD_CHUNK - 1) / FOLD_CHUNK;
-    p.items = (long long)d->c_out * p.chunks_per_row;
+    p.n = (long long)d->c_out * d->k;
+    p.blocks = (int)std::min<long long>((p.n + FOLD_CHUNK - 1) / FOLD_CHUNK, FOLD_MAX_BLOCKS);
     p.ratio = d->eta_in / d->eta_out;
     p.eta_out = d->eta_out;
     p.fl_x = d->fl_x; p.fl_min = d->fl_w_min; p.fl_max = d->fl_w_max;
-    p.vec4 = (d->k % 4 == 0 && ((uintptr_t)w & 15) == 0 && ((uintptr_t)w_q & 3) == 0) ? 1 : 0;
+    const bool vec4 = d->k % 4 == 0 && ((uintptr_t)w & 15) == 0 && ((uintptr_t)w_q & 3) == 0;
     p.w = w; p.gamma = gamma; p.sigma = sigma; p.beta = beta; p.mu = mu;
     p.w_q = w_q; p.b_q = bias_q; p.fl_w = fl_w; p.partial = (double *)workspace;
-    p.scale = p.partial + 2 * FOLD_MAX_BLOCKS + 2;
-    cudaStream_t st = (cudaStream_t)cuda_stream;
-    const int blocks = fold_blocks(p.items);
-    fold_scale_kernel<<<(d->c_out + FOLD_THREADS - 1) / FOLD_THREADS, FOLD_THREADS, 0, st>>>(p);
-    fold_stats_kernel<<<blocks, FOLD_THREADS, 0, st>>>(p);
-    fold_format_kernel<<<1, FOLD_THREADS, 0, st>>>(p, blocks);
-    fold_quant_kernel<<<blocks, FOLD_THREADS, 0, st>>>(p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = vec4 ? launch_fold<true>(p, (cudaStream_t)cuda_stream) : launch_fold<false>(p, (cudaStream_t)cuda_stream);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return f8_set_error(F8_ERR_CUDA, cudaGetErrorString(e));
     return F8_OK;
 }

@@ -20,6 +20,9 @@ FOLD_CASES = [
     (17, 5, 0.5, 0, 24),           # tiny and ragged
     (96, 4608, 0.8, 8, 7),         # rows longer than a chunk; paper's FL range 0..7
     (32, 27, 30.0, 2, 7),          # large weights: FL clamps at 0 and codes saturate
+    (5000, 1, 0.4, 3, 24),         # more rows per block than the table of row scales holds
+    (2051, 2051, 0.05, 5, 24),     # rows and chunks never line up, single-weight accesses; a second chunk per block
+    (1200, 4096, 0.05, 5, 24),     # the same with groups of four
 ]
 
 
