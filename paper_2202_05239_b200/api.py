@@ -86,12 +86,19 @@ def _ptr(t: Optional[torch.Tensor]):
         return None
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("tensors must be contiguous CUDA tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+# The current stream's handle without a Stream object around it: building one takes 3.4 us, the handle 0.3 us, and a call that
+# enqueues a small layer 15 us in all.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_get_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
+def _stream(stream):
+    if stream is None and _raw_stream is not None and _get_device is not None:
+        return _raw_stream(_get_device())
+    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
 
 
 def conv_desc(layer: "synth.Layer", n: int) -> ConvDesc:
