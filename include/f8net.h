@@ -124,7 +124,7 @@ f8_status f8_conv2d_fixed(const f8_conv_desc *desc, const void *x, const int8_t 
  *   - F8_S32_RELU allowed for y_dtype / y2_dtype: the sum behind a ReLU, max(v, 0), unrounded, int32 in the format
  *     F = max(fl_x + fl_w, fl_r) of the aligned sum (F8_S32: the sum itself).
  * Both 8-bit outputs equal what two f8_conv2d_fixed calls with fl_y and fl_y2 would give.  Precondition as for every
- * layer: the aligned sum fits int32.  Runs with direct stores (not the staged TMA epilogue); same validation errors. */
+ * layer: the aligned sum fits int32.  Same validation errors. */
 f8_status f8_conv2d_siblings_fixed(const f8_conv_desc *desc, int y2_dtype, int fl_y2, const void *x,
                                    const int8_t *w_ohwi, const int32_t *bias, const void *residual, void *y, void *y2,
                                    void *workspace, size_t workspace_bytes, void *cuda_stream);

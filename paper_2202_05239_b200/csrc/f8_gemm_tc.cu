@@ -136,7 +136,12 @@ struct TcParams {
     uint32_t out_off, bias_off;   // byte offsets behind the stages: two output tiles, two residual
                                            // tiles, int32 bias' of all padded columns
     F8Requant q;
-    F8Sibling sib;            // second consumer of the same sums (generic epilogue only)
+    F8Sibling sib;            // second consumer of the same sums (generic and wide epilogues)
+    // Wide epilogue (EPI_WIDE): tiles of at most 128 columns; a buffer of the ring holds a 32-bit tile (in column slabs of 32
+    // values; a 32-bit shortcut lands there and a 32-bit output replaces it in place) and up to two 8-bit tiles
+    int wide_out32;           // 0: no 32-bit output, 1: y, 2: y2
+    int wide_slabs;           // slabs of the 32-bit tile (0: no 32-bit tile)
+    uint32_t wide_q1, wide_q2;   // where the 8-bit tiles of y and y2 start; an 8-bit shortcut shares y2's (in place)
     int vec_bytes2;           // widest aligned store of the second output's rows
     int mul_acc, mul_res;     // 2^q.sh_acc, 2^q.sh_res (kept opaque to the compiler, see the epilogue)
     int *status;
@@ -237,9 +242,77 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams &p, const int (&ac
     if (p.sib.y2) store_chunk((uint8_t *)p.sib.y2, p.sib.y_kind, p.sib.s, p.sib.lo, p.sib.hi, v, o, nvalid, p.c_out, p.vec_bytes2);
 }
 
+// Wide epilogue: 16 channels of one row whose accumulator load is in flight; everything else lies in the ring buffer `buf`.
+__device__ __forceinline__ uint4 wide_quantize(const int (&v)[16], int s, bool sgn) {
+    uint32_t o[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        int t[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t[k] = f8_rshift_round(v[4 * g + k], s);
+        uint32_t hi;
+        if (sgn) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) t[k] = max(t[k], -127);
+            asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, 0;" : "=r"(hi) : "r"(t[3]), "r"(t[2]));
+            asm("cvt.pack.sat.s8.s32.b32 %0, %1, %2, %3;" : "=r"(o[g]) : "r"(t[1]), "r"(t[0]), "r"(hi));
+        } else {
+            asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(hi) : "r"(t[3]), "r"(t[2]));
+            asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(o[g]) : "r"(t[1]), "r"(t[0]), "r"(hi));
+        }
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+__device__ __forceinline__ void wide_chunk(const TcParams &p, int (&v)[16], uint32_t buf, uint32_t bias_addr, int row, int col,
+                                           const uint32_t (&rsel)[4], int mul_acc, int mul_res) {
+    // 32-bit tile: slabs of 32 columns, 128-byte rows; 8-bit tiles: slab_w bytes a row
+    const uint32_t w_row = buf + (uint32_t)(col >> 5) * (TILE_M * 128) + (uint32_t)row * 128;
+    const uint32_t w_chunk = (uint32_t)(col & 31) >> 2, w_swz = (uint32_t)row & 7;
+    uint32_t q_off = (uint32_t)row * p.slab_w + (uint32_t)col;
+    q_off ^= ((q_off >> 7) & p.swz_mask) << 4;
+    uint4 r[4];
+    if (p.q.has_res) {
+        if (p.q.r_s32) {
+#pragma unroll
+            for (int g = 0; g < 4; ++g) r[g] = lds128(w_row + (((w_chunk + g) ^ w_swz) << 4));
+        } else {
+            const uint4 b = lds128(buf + p.wide_q2 + q_off);
+            const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r[g].x) : "r"(bw[g]), "r"(rsel[0]));
+                asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r[g].y) : "r"(bw[g]), "r"(rsel[1]));
+                asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r[g].z) : "r"(bw[g]), "r"(rsel[2]));
+                asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r[g].w) : "r"(bw[g]), "r"(rsel[3]));
+            }
+        }
+    } else {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) r[g] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    tmem_ld_wait16(v);
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        const uint4 b = lds128(bias_addr + 16 * g);
+        v[4 * g] = v[4 * g] * mul_acc + (int)b.x + (int)r[g].x * mul_res;
+        v[4 * g + 1] = v[4 * g + 1] * mul_acc + (int)b.y + (int)r[g].y * mul_res;
+        v[4 * g + 2] = v[4 * g + 2] * mul_acc + (int)b.z + (int)r[g].z * mul_res;
+        v[4 * g + 3] = v[4 * g + 3] * mul_acc + (int)b.w + (int)r[g].w * mul_res;
+    }
+    if (p.wide_out32 != 1) sts128(buf + p.wide_q1 + q_off, wide_quantize(v, p.q.s, p.q.y_kind == F8_S8));
+    if (p.sib.y2 && p.wide_out32 != 2) sts128(buf + p.wide_q2 + q_off, wide_quantize(v, p.sib.s, p.sib.y_kind == F8_S8));
+    if (p.wide_out32) {
+        const int lo = (p.wide_out32 == 1 ? p.q.y_kind : p.sib.y_kind) == F8_S32_RELU ? 0 : (int)0x80000000;
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+            sts128(w_row + (((w_chunk + g) ^ w_swz) << 4),
+                   make_uint4((uint32_t)max(v[4 * g], lo), (uint32_t)max(v[4 * g + 1], lo), (uint32_t)max(v[4 * g + 2], lo), (uint32_t)max(v[4 * g + 3], lo)));
+    }
+}
+
 // ----------------------------------------------------------------------------- the kernel
 
-enum { EPI_GENERIC = 0, EPI_U8 = 1, EPI_U8_RES = 2, EPI_S8 = 3, EPI_S8_RES = 4 };
+enum { EPI_GENERIC = 0, EPI_U8 = 1, EPI_U8_RES = 2, EPI_S8 = 3, EPI_S8_RES = 4, EPI_WIDE = 5 };
 
 // MODE 0: one 128-row tile per hand-over.  MODE 2: groups of M tiles (TcParams::sup).  MODE 1 (PAIR below):
 // PAIR: two CTAs of a cluster share 256-row tiles (tcgen05 cta_group::2): each loads its own 128 rows of activations and
@@ -248,10 +321,11 @@ template <int EPI, int MODE>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                        const __grid_constant__ CUtensorMap map_y, const __grid_constant__ CUtensorMap map_r,
-                       const TcParams p) {
+                       const __grid_constant__ CUtensorMap map_y2, const TcParams p) {
     constexpr bool PAIR = MODE == 1;                                // CTA pairs
     constexpr bool SUP = MODE == 2;                                 // groups of M tiles per hand-over (TcParams::sup)
     constexpr bool STAGED = EPI != EPI_GENERIC;                     // output (and residual) through shared memory + TMA
+    constexpr bool WIDE = EPI == EPI_WIDE;                          // a 32-bit output or shortcut, or two outputs (TcParams::wide_*)
     constexpr bool RES = EPI == EPI_U8_RES || EPI == EPI_S8_RES;
     constexpr bool SGN = EPI == EPI_S8 || EPI == EPI_S8_RES;
 
@@ -288,7 +362,8 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         prefetch_tensormap(&map_a);
         prefetch_tensormap(&map_b);
         if (STAGED) prefetch_tensormap(&map_y);
-        if (RES) prefetch_tensormap(&map_r);
+        if (RES || (WIDE && p.q.has_res)) prefetch_tensormap(&map_r);
+        if (WIDE && p.sib.y2) prefetch_tensormap(&map_y2);
     }
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -711,7 +786,13 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             const int m_t = PAIR ? 2 * m_q + (int)cta_rank : m_q;
                 if (!warp_wait(out_full + 8 * b, bphase, wc, tagbits | 108)) break;
                 const uint32_t src = smem_base + p.out_off + b * p.out_bytes;
-                if (SUP) {
+                if (WIDE) {
+                    const int c0 = n_t * p.bn, m0 = m_t * TILE_M;
+                    if (p.wide_out32 != 1) tma_store_2d(&map_y, src + p.wide_q1, c0, m0);
+                    if (p.sib.y2 && p.wide_out32 != 2) tma_store_2d(&map_y2, src + p.wide_q2, c0, m0);
+                    for (int sl = 0; p.wide_out32 && sl < p.wide_slabs; ++sl)
+                        if (c0 + 32 * sl < p.c_out) tma_store_2d(p.wide_out32 == 1 ? &map_y : &map_y2, src + sl * (TILE_M * 128), 4 * (c0 + 32 * sl), m0);
+                } else if (SUP) {
                     // column slab sl of the staged tile is M tile tile * sup + sl
                     const int subs = min(p.sup, p.m_tiles - tile * p.sup);
                     for (int sl = 0; sl < subs; ++sl)
@@ -737,7 +818,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         }
     } else if (warp == FETCH_WARP) {
         // ------------------------------------------------------------------ residual fetcher
-        if (RES) {
+        if (RES || (WIDE && p.q.has_res)) {
             grid_dependency_wait();
             // residual tiles go straight into the output ring (the epilogue converts them in place): a buffer is
             // loaded as soon as the store of the tile that used it before has read it, up to out_bufs - 1 tiles ahead
@@ -751,7 +832,14 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 if (!warp_wait(out_free + 8 * rb, rphase ^ 1, wc, tagbits | 106)) { ok = false; break; }
                 const uint32_t fb = res_full + 8 * rb;
                 warp_expect_tx(fb, p.tx_res);
-                if (p.rows) {
+                if (WIDE) {
+                    const uint32_t dst = smem_base + p.out_off + rb * p.out_bytes;
+                    if (p.q.r_s32)
+                        for (int sl = 0; sl < p.wide_slabs; ++sl)
+                            tma_load_2d(dst + sl * (TILE_M * 128), &map_r, fb, 4 * (n_t * p.bn + 32 * sl), m_t * TILE_M, lane == sl);
+                    else
+                        tma_load_2d(dst + p.wide_q2, &map_r, fb, n_t * p.bn, m_t * TILE_M, lane == 0);
+                } else if (p.rows) {
                     const int img = fast_div(m_t, p.div_bands);
                     const int y0 = (m_t - img * p.win_bands) * p.win_r;
                     for (int sl = 0; sl < p.n_slabs; ++sl)
@@ -795,7 +883,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 // issuers are already at work: the prologue of a CTA starts when the previous layer's CTA has left the SM,
                 // and a round trip to global memory there would be paid by every layer.
                 int *bias_all = (int *)(smem + p.bias_off);
-                const int rnd = 1 << (p.q.s - 1);
+                const int rnd = WIDE ? 0 : 1 << (p.q.s - 1);      // (two outputs round at different places)
                 for (int i = (int)threadIdx.x - FIRST_EPI_WARP * 32; i < p.n_tiles * p.bn; i += NUM_EPI_WARPS * 32)
                     bias_all[i] = ((i < p.c_out && p.bias) ? (__ldg(p.bias + i) << p.q.sh_acc) : 0) + rnd;
                 asm volatile("bar.sync 1, %0;" ::"n"(NUM_EPI_WARPS * 32) : "memory");
@@ -834,7 +922,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 // free): that wait is over long before the accumulator is complete, so it costs the chain accumulator ->
                 // epilogue -> accumulator nothing.
                 bool got;
-                if (RES) got = mbar_wait(res_full + 8 * ob, ophase, wc, tagbits | 107);
+                if (RES || (WIDE && p.q.has_res)) got = mbar_wait(res_full + 8 * ob, ophase, wc, tagbits | 107);
                 else got = mbar_wait(out_free + 8 * ob, ophase ^ 1, wc, tagbits | 109);
                 got = mbar_wait(tfull_bar + 8 * acc, acc_phase, wc, tagbits | 104) && got;
                 if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
@@ -852,6 +940,14 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                         else mbar_arrive(tempty_bar + 8 * acc);
                     }
                 };
+                if (WIDE) {
+                    for (int i = 0; i < my_nch; ++i) {
+                        int v[16];
+                        tmem_ld16(t_addr + i * 16, v);
+                        wide_chunk(p, v, out_buf, bias_s + 64 * i, tile_row, (ch_begin + i) * 16, rsel, mul_acc, mul_res);
+                    }
+                    release_acc();
+                } else {
                 int va[16], vb[16];
                 if (my_nch > 0) tmem_ld16(t_addr, va);
                 else release_acc();
@@ -873,6 +969,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                         else release_acc();
                         sts128(out_buf + so[i + 1], epilogue_fast16<RES, SGN>(vb, bias_s + 64 * (i + 1), rw, mul_acc, mul_res, rsel, p.q.s));
                     }
+                }
                 }
                 // the output part is written: make the writes visible to the TMA and tell the mover (and, through it, the
                 // fetcher)
@@ -1046,6 +1143,7 @@ struct F8TcPlan {
     CUtensorMap map_b;
     CUtensorMap map_y;
     CUtensorMap map_r;
+    CUtensorMap map_y2;
     TcParams p;
     int grid;
     size_t smem;
@@ -1097,20 +1195,40 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
     p.pad_h = g.pad_h;
     p.pad_w = g.pad_w;
     p.kb = choose_kb(g.c);
+    const bool has_sib = sib && sib->y2;
     // residual layers are bound by the epilogue, not by the main loop: prefer 64-byte K chunks so that a
     // 256-wide tile (half the tiles, half the A re-reads) still leaves room for the pipeline stages
     // (not the K-heavy ones -- a 3x3 layer with a shortcut, as in basic residual blocks: those keep 128-byte chunks and
     // 256-wide tiles, which makes them CTA pairs; the three 32-KiB buffers of the output ring leave three 32-KiB stages)
     const bool k_heavy_res = q.has_res && g.c % 128 == 0 && g.c_out % 256 == 0 && g.kh * g.kw * (g.c / 128) >= 8;
-    if (q.has_res && g.c_out > 128 && p.kb == 128 && g.c <= 256 && !k_heavy_res) p.kb = 64;
+    if (q.has_res && g.c_out > 128 && p.kb == 128 && g.c <= 256 && !k_heavy_res && !q.r_s32 && !has_sib) p.kb = 64;
     p.c_chunks = (g.c + p.kb - 1) / p.kb;
     p.epi = EPI_GENERIC;
-    const bool has_sib = sib && sib->y2;
     if ((q.y_kind == F8_U8 || q.y_kind == F8_S8) && q.s >= 1 && q.s <= 24 && g.c_out % 16 == 0 && !has_sib && !q.r_s32)
         p.epi = q.y_kind == F8_U8 ? (q.has_res ? EPI_U8_RES : EPI_U8) : (q.has_res ? EPI_S8_RES : EPI_S8);
+    // 32-bit outputs or shortcuts and second outputs go through shared memory as well (at most one of the outputs in 32 bits; small
+    // tensors, which have no plain [M, c_out] tile geometry, keep the direct stores).  Direct stores write 16 bytes per row and
+    // instruction and read a 32-bit shortcut the same way, behind the accumulator: 3x3 64 -> 64 at 56 x 56 with a 32-bit
+    // shortcut and a 32-bit second output, batch 128, 138 -> 79 us, 1x1 / 2 64 -> 128 to 32 bits 41 -> 20.5 us.
+    auto is32 = [](int kind) { return kind == F8_S32 || kind == F8_S32_RELU; };
+    const bool pointwise1 = g.kh == 1 && g.kw == 1 && g.stride_h == 1 && g.stride_w == 1 && g.pad_h == 0 && g.pad_w == 0;
+    const bool big_x = (size_t)xv.dim_c * xv.dim_w * xv.dim_h * xv.dim_n >= 128 * 1024;
+    if (p.epi == EPI_GENERIC && g.c_out % 16 == 0 && (big_x || pointwise1) && (is32(q.y_kind) || (q.s >= 1 && q.s <= 31)) &&
+        (!has_sib || is32(sib->y_kind) || (sib->s >= 1 && sib->s <= 31)) && !(has_sib && is32(q.y_kind) && is32(sib->y_kind)) &&
+        (g.c_out > 16 || !(is32(q.y_kind) || q.r_s32 || (has_sib && is32(sib->y_kind)))))
+        p.epi = EPI_WIDE;
+    const bool wide = p.epi == EPI_WIDE;
     const bool staged = p.epi != EPI_GENERIC;
-    p.bn = staged ? (k_heavy_res ? 256 : choose_bn_staged(g.c_out, q.has_res != 0, p.kb)) : choose_bn(g.c_out);
+    p.bn = wide ? (g.c_out > 32 ? 64 : 32) : staged ? (k_heavy_res ? 256 : choose_bn_staged(g.c_out, q.has_res != 0, p.kb)) : choose_bn(g.c_out);
     p.m_tiles = (p.M + TILE_M - 1) / TILE_M;
+    if (wide && g.c_out >= 128) {
+        // 64-wide tiles leave room for three (two) buffers of the ring; where 128-wide ones give every SM one tile at most, a single
+        // buffer will do and the activations are read half as often (3x3 256 -> 256 at 14 x 14, batch 33: 22.5 -> 18.5 us)
+        int sm_count = 148, dev0 = 0;
+        cudaGetDevice(&dev0);
+        cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev0);
+        if ((long long)p.m_tiles * ((g.c_out + 127) / 128) <= sm_count && (long long)p.m_tiles * ((g.c_out + 63) / 64) > sm_count) p.bn = 128;
+    }
     if (!staged) {
         // few output pixels (a fully connected layer): narrower N tiles until every SM has one, the weights are
         // what has to be streamed and each CTA then streams its own slice of them
@@ -1161,7 +1279,7 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
         {
             const bool one_k = g.kh == 1 && g.kw == 1 && g.c <= p.kb;
             const int gsz = p.bn <= 64 ? 4 : 2;
-            if (one_k && !q.has_res && p.bn <= 128 && g.c_out <= p.bn && g.c_out % 16 == 0 && !p.pair && g.stride_h == 1 &&
+            if (one_k && !wide && !q.has_res && p.bn <= 128 && g.c_out <= p.bn && g.c_out % 16 == 0 && !p.pair && g.stride_h == 1 &&
                 g.stride_w == 1 && g.pad_h == 0 && g.pad_w == 0 && p.m_tiles >= 148 * 4 * gsz &&
                 !(f8_plan_options_off() & (F8_PLAN_OFF_TILE_GROUPS | F8_PLAN_OFF_RESIDENT_WEIGHTS))) {
                 p.sup = gsz;
@@ -1174,6 +1292,17 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
                 p.out_bufs = 2;
                 p.epi_groups = 4;
             }
+        }
+        if (wide) {
+            p.wide_out32 = is32(q.y_kind) ? 1 : (has_sib && is32(sib->y_kind) ? 2 : 0);
+            p.wide_slabs = p.wide_out32 || q.r_s32 ? (p.bn + 31) / 32 : 0;
+            const uint32_t w32 = (uint32_t)p.wide_slabs * TILE_M * 128, w8 = (uint32_t)(TILE_M * p.bn);
+            const bool q1 = p.wide_out32 != 1, q2 = (has_sib && p.wide_out32 != 2) || (q.has_res && !q.r_s32);
+            p.wide_q1 = w32;
+            p.wide_q2 = w32 + (q1 ? w8 : 0);
+            p.out_bytes = w32 + (q1 ? w8 : 0) + (q2 ? w8 : 0);
+            p.out_bufs = p.bn == 128 ? 1 : (q.has_res ? 3 : 2);
+            p.epi_groups = p.bn >= 64 ? 4 : 2;
         }
         staging = (size_t)p.out_bytes * p.out_bufs + bias_bytes;
     }
@@ -1203,7 +1332,7 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
         return cudaErrorInvalidValue;
     }
     p.tx_sub = p.tx_a + (p.b_res ? 0u : p.tx_b);
-    p.tx_res = p.out_bytes;
+    p.tx_res = wide ? (uint32_t)(TILE_M * p.bn * (q.r_s32 ? 4 : 1)) : p.out_bytes;
     // Windowed mode for 3x3 / stride 1 / pad 1 layers whose weights can stay resident: whole padded rows are loaded once
     // per tile and every filter tap reads them at a shifted row offset.  Worth it when whole rows fill most of a tile
     // and the im2col loads are what bounds the layer: measured, 128-channel layers gain 1.8x (the resident weights
@@ -1212,7 +1341,7 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
     // scheduler partition are busy -- an MMA-only loop issues one every 52 cycles -- and whole-row tiles are 12.5 % more
     // tiles).
     p.win = 0;
-    if (staged && !p.pair && p.kb == 128 && g.kh == 3 && g.kw == 3 && g.stride_h == 1 && g.stride_w == 1 && g.pad_h == 1 && g.pad_w == 1 &&
+    if (staged && !wide && !p.pair && p.kb == 128 && g.kh == 3 && g.kw == 3 && g.stride_h == 1 && g.stride_w == 1 && g.pad_h == 1 && g.pad_w == 1 &&
         g.pad_h_end < 0 && p.n_tiles == 1 && g.w + 2 <= TILE_M && g.w == g.wo && g.h == g.ho && g.c % p.kb == 0 &&
         !(off & (F8_PLAN_OFF_WINDOWED | F8_PLAN_OFF_RESIDENT_WEIGHTS))) {
         const int wp = g.w + 2;
@@ -1395,7 +1524,27 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
     // output / residual [M, c_out] bytes, one box = one column slab of a tile
     plan->map_y = plan->map_b;
     plan->map_r = plan->map_b;
-    if (staged && p.rows) {
+    plan->map_y2 = plan->map_b;
+    if (wide) {
+        // [M, c_out] of 8-bit values in boxes of bn columns, or of 32-bit values (four bytes each) in boxes of 32 columns
+        auto encode = [&](CUtensorMap *map, const void *base, bool w32, CUtensorMapL2promotion promo) {
+            const cuuint64_t row = (cuuint64_t)g.c_out * (w32 ? 4 : 1);
+            cuuint64_t dims[2] = {row, (cuuint64_t)p.M};
+            cuuint64_t strides[1] = {row};
+            cuuint32_t box[2] = {w32 ? 128u : (cuuint32_t)p.slab_w, (cuuint32_t)TILE_M};
+            cuuint32_t estr[2] = {1, 1};
+            const CUtensorMapSwizzle sw = w32 || p.slab_w == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                          : (p.slab_w == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+            return g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(base), dims, strides, box, estr,
+                                  CU_TENSOR_MAP_INTERLEAVE_NONE, sw, promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+        };
+        if (!encode(&plan->map_y, y, p.wide_out32 == 1, CU_TENSOR_MAP_L2_PROMOTION_NONE) ||
+            (has_sib && !encode(&plan->map_y2, sib->y2, p.wide_out32 == 2, CU_TENSOR_MAP_L2_PROMOTION_NONE)) ||
+            (q.has_res && !encode(&plan->map_r, res, q.r_s32 != 0, CU_TENSOR_MAP_L2_PROMOTION_L2_128B))) {
+            *why = "cuTensorMapEncodeTiled rejected an output tensor";
+            return cudaErrorInvalidValue;
+        }
+    } else if (staged && p.rows) {
         // output / residual as (C_out, W, H, N); one box = one column slab of win_r rows of W + 2 positions
         cuuint64_t dims[4] = {(cuuint64_t)g.c_out, (cuuint64_t)g.wo, (cuuint64_t)g.ho, (cuuint64_t)g.n};
         cuuint64_t strides[3] = {(cuuint64_t)g.c_out, (cuuint64_t)g.c_out * g.wo, (cuuint64_t)g.c_out * g.wo * g.ho};
@@ -1449,7 +1598,7 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
     {
         int *info = f8_last_plan_info();
         info[0] = (p.b_res ? F8_PLAN_RESIDENT_WEIGHTS : 0) | (p.win ? F8_PLAN_WINDOWED : 0) | (p.dual_issue ? F8_PLAN_DUAL_ISSUE : 0) |
-                  (p.alt ? F8_PLAN_ALT_PRODUCERS : 0) | (p.a_plain ? F8_PLAN_PLAIN_MATRIX : 0) | (staged ? F8_PLAN_STAGED_EPILOGUE : 0) | (p.rowt ? F8_PLAN_ROW_TILES : 0) |
+                  (p.alt ? F8_PLAN_ALT_PRODUCERS : 0) | (p.a_plain ? F8_PLAN_PLAIN_MATRIX : 0) | (staged && !wide ? F8_PLAN_STAGED_EPILOGUE : 0) | (p.rowt ? F8_PLAN_ROW_TILES : 0) |
                   (p.pair ? F8_PLAN_PAIRS : 0) | (p.sup ? F8_PLAN_TILE_GROUPS : 0);
         info[1] = p.epi; info[2] = p.bn; info[3] = p.kb; info[4] = p.stages; info[5] = p.group;
         info[6] = p.m_tiles; info[7] = p.n_tiles; info[8] = plan->grid; info[9] = staged ? p.out_bufs : 0;
@@ -1467,6 +1616,7 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f8_conv_gemm_tc_kernel<EPI_U8_RES, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f8_conv_gemm_tc_kernel<EPI_S8, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f8_conv_gemm_tc_kernel<EPI_S8_RES, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f8_conv_gemm_tc_kernel<EPI_WIDE, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f8_conv_gemm_tc_kernel<EPI_U8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f8_conv_gemm_tc_kernel<EPI_U8_RES, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f8_conv_gemm_tc_kernel<EPI_S8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -1516,7 +1666,7 @@ cudaError_t launch_variant(const F8TcPlan *plan, bool overlap_previous, cudaStre
         else
             (void)cudaGetLastError();
     }
-    return cudaLaunchKernelEx(&cfg, f8_conv_gemm_tc_kernel<EPI, MODE>, plan->map_a, plan->map_b, plan->map_y, plan->map_r, plan->p);
+    return cudaLaunchKernelEx(&cfg, f8_conv_gemm_tc_kernel<EPI, MODE>, plan->map_a, plan->map_b, plan->map_y, plan->map_r, plan->map_y2, plan->p);
 }
 }   // namespace
 
@@ -1543,6 +1693,7 @@ cudaError_t f8_tc_launch(const F8TcPlan *plan, bool overlap_previous, cudaStream
         case EPI_U8_RES: return launch_variant<EPI_U8_RES, 0>(plan, overlap_previous, st);
         case EPI_S8: return launch_variant<EPI_S8, 0>(plan, overlap_previous, st);
         case EPI_S8_RES: return launch_variant<EPI_S8_RES, 0>(plan, overlap_previous, st);
+        case EPI_WIDE: return launch_variant<EPI_WIDE, 0>(plan, overlap_previous, st);
         default: return launch_variant<EPI_GENERIC, 0>(plan, overlap_previous, st);
     }
 }

@@ -25,6 +25,13 @@ CASES = [
     (14, 14, 24, 40, 3, 1, 2, False, U8, S8, S32, False),        # channel counts off the 16-byte rule: CUDA-core kernel
     (9, 9, 16, 16, 3, 2, 1, True, S32R, S32, S8, False),         # small tensor: CUDA-core kernel, both outputs 32-bit
     (12, 12, 32, 24, 1, 1, 40, False, U8, S32, U8, True),        # c_out = 24 on the tensor cores: ragged stores of both outputs
+    # 32-bit tiles through shared memory: 128-wide tiles with a single buffer, one per SM
+    (14, 14, 128, 256, 3, 1, 33, False, U8, S32R, S32, True),
+    (28, 28, 64, 96, 1, 1, 4, True, S32, S8, None, True),        # 96 of 128 columns: the last slab of 32 values does not exist
+    (33, 31, 64, 48, 1, 1, 3, False, S32R, None, U8, True),      # 48 columns, 3069 pixels: ragged rows and slabs; 8-bit shortcut, one output
+    (31, 30, 64, 32, 3, 2, 5, False, S8, U8, S8, True),          # 32-wide tiles, two 8-bit outputs, 8-bit shortcut in place
+    (20, 20, 64, 16, 1, 1, 9, False, U8, S8, S8, True),          # 16 columns in a 32-wide tile, no 32-bit tile
+    (20, 20, 64, 16, 1, 1, 9, False, U8, S32, S8, True),         # 16 columns in 32 bits: direct stores
 ]
 
 
