@@ -230,7 +230,8 @@ int f8_net_last_launch_count(const f8_net *net);
 
 /* Number of those kernels that ran two layers at once (a 64 -> 64 convolution and the 64 -> 256 pointwise layer that
  * alone reads its output: see f8_conv_pointwise_fixed).  f8_net_forward does that wherever the shapes allow; the
- * first layer's output then exists in device memory only in a pass that asks for layer dumps. */
+ * first layer's output then exists in device memory only in a pass that asks for layer dumps.  Depthwise 3x3 layers
+ * and the pointwise layers behind them are counted too where they run as one launch (where that is the faster way). */
 int f8_net_fused_pairs(const f8_net *net);
 
 /* Per-layer timing.  With profiling on, f8_net_forward records a CUDA event after every kernel it
@@ -358,8 +359,11 @@ void f8_debug_force_direct(int on);
  *   F8_PLAN_OFF_STEM_KERNEL       first layers take the packed-row-pair GEMM instead of the first-layer kernel
  *   F8_PLAN_OFF_STEM_POOL_FUSION  the max pool behind a first layer runs as its own kernel
  *   F8_PLAN_OFF_LAYER_OVERLAP     f8_net_forward launches without programmatic dependent launch
- *   F8_PLAN_OFF_LAYER_FUSION      f8_net_forward runs a 64 -> 64 convolution and the 64 -> 256 pointwise layer behind it as two launches
+ *   F8_PLAN_OFF_LAYER_FUSION      f8_net_forward runs a 64 -> 64 convolution and the 64 -> 256 pointwise layer behind it as two launches,
+ *                                 and a depthwise 3x3 layer and the pointwise layer behind it too
  *   F8_PLAN_OFF_SMALL_KERNEL      f8_net_forward runs layers of a few microseconds on the tcgen05 kernel as well
+ *   F8_PLAN_OFF_DWPW_RULE         f8_net_forward runs every depthwise 3x3 + pointwise pair that one kernel can take in one launch,
+ *                                 not only those where that is faster
  *   F8_PLAN_OFF_LANES             f8_net_forward runs the whole batch as one sequence of launches on the caller's stream
  *   F8_PLAN_SYNC_LAYERS           f8_net_forward synchronises after every launch, so that a device fault is
  *                                 reported with the layer that raised it */
@@ -367,7 +371,8 @@ enum {
     F8_PLAN_OFF_RESIDENT_WEIGHTS = 1, F8_PLAN_OFF_WINDOWED = 2, F8_PLAN_OFF_DUAL_ISSUE = 4, F8_PLAN_OFF_ALT_PRODUCERS = 8,
     F8_PLAN_OFF_PAIRS = 16, F8_PLAN_OFF_DW_WALK = 32, F8_PLAN_OFF_STEM_KERNEL = 64, F8_PLAN_OFF_STEM_POOL_FUSION = 128,
     F8_PLAN_OFF_LAYER_OVERLAP = 256, F8_PLAN_OFF_LANES = 512, F8_PLAN_SYNC_LAYERS = 1024, F8_PLAN_OFF_DW_DP4A = 2048,
-    F8_PLAN_OFF_TILE_GROUPS = 4096, F8_PLAN_OFF_LAYER_FUSION = 8192, F8_PLAN_OFF_SMALL_KERNEL = 16384
+    F8_PLAN_OFF_TILE_GROUPS = 4096, F8_PLAN_OFF_LAYER_FUSION = 8192, F8_PLAN_OFF_SMALL_KERNEL = 16384,
+    F8_PLAN_OFF_DWPW_RULE = 32768
 };
 void f8_debug_plan_options(unsigned off_mask);
 

@@ -259,6 +259,7 @@ PLAN_OFF_LAYER_OVERLAP, PLAN_OFF_LANES, PLAN_SYNC_LAYERS, PLAN_OFF_DW_DP4A = 256
 PLAN_OFF_TILE_GROUPS = 4096
 PLAN_OFF_LAYER_FUSION = 8192
 PLAN_OFF_SMALL_KERNEL = 16384
+PLAN_OFF_DWPW_RULE = 32768
 PLAN_RESIDENT_WEIGHTS, PLAN_WINDOWED, PLAN_DUAL_ISSUE, PLAN_ALT_PRODUCERS = 1, 2, 4, 8
 PLAN_PLAIN_MATRIX, PLAN_STAGED_EPILOGUE, PLAN_PAIRS, PLAN_ROW_TILES = 16, 32, 64, 128
 PLAN_TILE_GROUPS = 256

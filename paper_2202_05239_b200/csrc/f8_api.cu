@@ -140,6 +140,16 @@ FusedPlanPtr alloc_fused_plan() {
     return FusedPlanPtr((F8FusedPlan *)p);
 }
 
+struct DwPwPlanDeleter { void operator()(F8DwPwPlan *p) const { free(p); } };
+using DwPwPlanPtr = std::unique_ptr<F8DwPwPlan, DwPwPlanDeleter>;
+
+DwPwPlanPtr alloc_dwpw_plan() {
+    const size_t size = (f8_dwpw_plan_size() + 63) / 64 * 64;
+    void *p = aligned_alloc(64, size);
+    if (p) memset(p, 0, size);
+    return DwPwPlanPtr((F8DwPwPlan *)p);
+}
+
 // The second consumer of a layer's sum: its quantizer relative to the format F of the aligned sum.
 f8_status make_sibling(const f8_conv_desc *d, const F8Requant &q, int y2_dtype, int fl_y2, void *y2, F8Sibling *sib) {
     if (y2_dtype != F8_U8 && y2_dtype != F8_S8 && y2_dtype != F8_S32 && y2_dtype != F8_S32_RELU)
@@ -502,7 +512,9 @@ struct Step {
     PlanPtr plan;
     // kind -3: this layer and the pointwise layer behind it (layer + 1) in one launch; y is that layer's output,
     // y_mid NULL or where a copy of this layer's own output goes
+    // kind -4: the same for a depthwise layer and the pointwise layer behind it
     FusedPlanPtr fplan;
+    DwPwPlanPtr dplan;
     void *y_mid = nullptr;
     F8ConvGeom g;
 };
@@ -663,11 +675,13 @@ void classify_tensors(const f8_net *net, const std::vector<Region> &regions, std
 // Layer i and the pointwise layer behind it may run as one launch (the two-layer kernel): layer i + 1 is a 1x1 convolution
 // that alone reads layer i's output, and the channel counts are the kernel's.  (Whether they do is decided per plan: the
 // batch must make the input large enough, and both layers must lie in the same run of the schedule.)
-bool pair_candidate(const f8_net *net, int i) {
+bool pair_candidate(const f8_net *net, int i, bool *depthwise = nullptr) {
     const int nl = (int)net->layers.size();
     if (i + 1 >= nl) return false;
     const NetLayer &L = net->layers[i], &P = net->layers[i + 1];
-    if (L.d.kind != F8_LAYER_CONV || L.packed || L.has_sibling || L.q.has_res) return false;
+    const bool dw = L.d.kind == F8_LAYER_DWCONV;
+    if (depthwise) *depthwise = dw;
+    if ((L.d.kind != F8_LAYER_CONV && !dw) || L.packed || L.has_sibling || L.q.has_res) return false;
     if (P.d.kind != F8_LAYER_CONV || P.has_sibling || P.packed || P.d.src != i + 1 || P.g.kh != 1 || P.g.kw != 1 || P.g.stride_h != 1 ||
         P.g.stride_w != 1 || P.g.pad_h != 0 || P.g.pad_w != 0)
         return false;
@@ -677,7 +691,7 @@ bool pair_candidate(const f8_net *net, int i) {
         if (net->layers[l2].d.src == i + 1 || (net->layers[l2].q.has_res && net->layers[l2].d.res == i + 1)) return false;
     F8ConvGeom g = L.g;
     g.n = net->max_batch;   // the size rule is checked again with the real batch when a plan is made
-    return f8_fused_supported(g, L.q, P.g.c_out, P.q);
+    return dw ? f8_dwpw_supported(g, L.q, P.g.c_out, P.q) : f8_fused_supported(g, L.q, P.g.c_out, P.q);
 }
 
 size_t assign_offsets(const f8_net *net, int batch, std::vector<size_t> *off, size_t *pack_off,
@@ -1030,7 +1044,7 @@ int f8_net_lanes(const f8_net *net) { return net ? net->last_lanes : 0; }
 int f8_net_fused_pairs(const f8_net *net) {
     int n = 0;
     if (net)
-        for (const Step &stp : net->steps) n += stp.kind == -3 ? 1 : 0;
+        for (const Step &stp : net->steps) n += stp.kind == -3 || stp.kind == -4 ? 1 : 0;
     return n;
 }
 
@@ -1063,7 +1077,7 @@ f8_status f8_net_get_layer_ms(f8_net *net, float *ms, int *on_tensor_cores) {
     if (on_tensor_cores)
         for (const Step &stp : net->steps)
             if (stp.kind >= 0 && stp.use_tc) on_tensor_cores[stp.layer] = 1;
-            else if (stp.kind == -3) on_tensor_cores[stp.layer] = on_tensor_cores[stp.layer + 1] = 1;
+            else if (stp.kind == -3 || stp.kind == -4) on_tensor_cores[stp.layer] = on_tensor_cores[stp.layer + 1] = 1;
     return F8_OK;
 }
 
@@ -1233,7 +1247,8 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                                // the next layer is a 1x1 convolution that alone reads this layer's output, both lie in the
                                // same run of the schedule, and the shapes are the two-layer kernel's.
                                if (g_plan_off & F8_PLAN_OFF_LAYER_FUSION) return false;
-                               if (!pair_candidate(net, i) || layer_region[i] != layer_region[i + 1]) return false;
+                               bool dw = false;
+                               if (!pair_candidate(net, i, &dw) || dw || layer_region[i] != layer_region[i + 1]) return false;
                                const NetLayer &P = net->layers[i + 1];
                                if (!f8_fused_supported(stp.g, L.q, P.g.c_out, P.q)) return false;
                                FusedPlanPtr fp = alloc_fused_plan();
@@ -1265,6 +1280,28 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                         f8_tc_plan_set_tag(plan.get(), i + 1);
                         stp.plan = std::move(plan);
                     }
+                }
+            }
+            if (L.d.kind == F8_LAYER_DWCONV && !g_force_direct &&
+                !(g_plan_off & (F8_PLAN_OFF_LAYER_FUSION | F8_PLAN_OFF_DW_DP4A | F8_PLAN_OFF_DW_WALK)) && pair_candidate(net, i) &&
+                layer_region[i] == layer_region[i + 1]) {
+                // a depthwise layer and the pointwise layer that alone reads its output
+                const NetLayer &P = net->layers[i + 1];
+                DwPwPlanPtr dp;
+                const char *why = "";
+                void *mid = layer_dump ? tensor_ptr(i + 1) : nullptr;
+                if (f8_dwpw_supported(stp.g, L.q, P.g.c_out, P.q) &&
+                    ((g_plan_off & F8_PLAN_OFF_DWPW_RULE) || f8_dwpw_wanted(stp.g, P.g.c_out, P.q.has_res != 0)))
+                    dp = alloc_dwpw_plan();
+                if (dp && f8_dwpw_plan_init(dp.get(), stp.g, L.q, P.g.c_out, P.q, stp.x, L.w, L.b, P.w, P.b, P.q.has_res ? tensor_ptr(P.d.res) : nullptr,
+                                            mid, tensor_ptr(i + 2), f8_status_word(), &why) == cudaSuccess) {
+                    f8_dwpw_plan_set_tag(dp.get(), i + 2);
+                    stp.kind = -4;
+                    stp.use_tc = true;
+                    stp.y = tensor_ptr(i + 2);
+                    stp.y_mid = mid;
+                    stp.dplan = std::move(dp);
+                    skip_layer = i + 1;
                 }
             }
             ln.steps.push_back(std::move(stp));
@@ -1342,6 +1379,10 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                 e = f8_fused_launch(stp.fplan.get(), net->overlap_layers, st);
                 ++g_tc_launches;
                 break;
+            case -4:
+                e = f8_dwpw_launch(stp.dplan.get(), net->overlap_layers, st);
+                ++g_tc_launches;
+                break;
             case -1:
                 e = f8_launch_pack_stem_pairs(stp.g.n, L.g.h, L.g.w, L.g.c, L.pack_cpad, L.pack_hp, L.pack_wp, L.pack_left, stp.x, stp.y, st,
                                               net->overlap_layers);
@@ -1376,7 +1417,7 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
         ++launches;
         if (prof) {
             cudaEventRecord(net->events[launches], st);
-            net->event_layer.push_back(stp.fused_pool || stp.kind == -3 ? stp.layer + 1 : stp.layer);
+            net->event_layer.push_back(stp.fused_pool || stp.kind == -3 || stp.kind == -4 ? stp.layer + 1 : stp.layer);
         }
         // copies of the outputs this step wrote: its layer's (the pooling layer's when fused), and a sibling's
         auto dump_layer = [&](int out_layer, const void *src) -> cudaError_t {
@@ -1393,8 +1434,8 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                                      cudaMemcpyDeviceToDevice, st);
         };
         if (stp.kind != -1) {
-            e = dump_layer(stp.fused_pool || stp.kind == -3 ? stp.layer + 1 : stp.layer, stp.y);
-            if (e == cudaSuccess && stp.kind == -3 && stp.y_mid) e = dump_layer(stp.layer, stp.y_mid);
+            e = dump_layer(stp.fused_pool || stp.kind == -3 || stp.kind == -4 ? stp.layer + 1 : stp.layer, stp.y);
+            if (e == cudaSuccess && (stp.kind == -3 || stp.kind == -4) && stp.y_mid) e = dump_layer(stp.layer, stp.y_mid);
             if (e == cudaSuccess && stp.has_sib) e = dump_layer(stp.layer + 1, stp.sib.y2);
             if (e != cudaSuccess) return cuda_fail(e, "layer dump copy");
         }

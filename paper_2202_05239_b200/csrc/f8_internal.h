@@ -102,6 +102,18 @@ cudaError_t f8_fused_plan_init(F8FusedPlan *plan, const F8ConvGeom &g1, const F8
 void f8_fused_plan_set_tag(F8FusedPlan *plan, int tag);
 cudaError_t f8_fused_launch(const F8FusedPlan *plan, bool overlap_previous, cudaStream_t st);
 
+// ---- two layers in one launch (f8_dwpw_tc.cu): a depthwise 3x3 convolution (unsigned 8-bit output) and the pointwise
+// convolution behind it (8-bit output, optional 8-bit shortcut).  `wanted`: the rule by which a network prefers it to two launches.
+struct F8DwPwPlan;
+bool f8_dwpw_supported(const F8ConvGeom &g1, const F8Requant &q1, int c_out2, const F8Requant &q2);
+bool f8_dwpw_wanted(const F8ConvGeom &g1, int c_out2, bool res);
+size_t f8_dwpw_plan_size();
+cudaError_t f8_dwpw_plan_init(F8DwPwPlan *plan, const F8ConvGeom &g1, const F8Requant &q1, int c_out2, const F8Requant &q2, const void *x,
+                              const int8_t *w_dw, const int32_t *bias1, const int8_t *w_pw, const int32_t *bias2, const void *res,
+                              void *y_mid, void *y, int *status_word, const char **why);
+void f8_dwpw_plan_set_tag(F8DwPwPlan *plan, int tag);
+cudaError_t f8_dwpw_launch(const F8DwPwPlan *plan, bool overlap_previous, cudaStream_t st);
+
 // ---- first-layer kernel (f8_stem_tc.cu): stride-2 convolution over an image with <= 4 channels, optionally fused
 // with the 3x3 / 2 / pad 1 max pool behind it.  kh2 row pairs per window starting `top` pairs above the output row,
 // `left` zero cells in front of a row, `slices` 32-byte K slices per row pair; w_core is [K / 16][c_out][16].
