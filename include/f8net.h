@@ -363,7 +363,7 @@ void f8_debug_force_direct(int on);
  *                                 and a depthwise 3x3 layer and the pointwise layer behind it too
  *   F8_PLAN_OFF_SMALL_KERNEL      f8_net_forward runs layers of a few microseconds on the tcgen05 kernel as well
  *   F8_PLAN_OFF_DWPW_RULE         f8_net_forward runs every depthwise 3x3 + pointwise pair that one kernel can take in one launch,
- *                                 not only those where that is faster
+ *                                 not only those where that is faster, and every depthwise layer that the tensor-core kernel can take on it
  *   F8_PLAN_OFF_LANES             f8_net_forward runs the whole batch as one sequence of launches on the caller's stream
  *   F8_PLAN_SYNC_LAYERS           f8_net_forward synchronises after every launch, so that a device fault is
  *                                 reported with the layer that raised it */

@@ -150,6 +150,16 @@ DwPwPlanPtr alloc_dwpw_plan() {
     return DwPwPlanPtr((F8DwPwPlan *)p);
 }
 
+struct DwPlanDeleter { void operator()(F8DwPlan *p) const { free(p); } };
+using DwPlanPtr = std::unique_ptr<F8DwPlan, DwPlanDeleter>;
+
+DwPlanPtr alloc_dw_plan() {
+    const size_t size = (f8_dw_tc_plan_size() + 63) / 64 * 64;
+    void *p = aligned_alloc(64, size);
+    if (p) memset(p, 0, size);
+    return DwPlanPtr((F8DwPlan *)p);
+}
+
 // The second consumer of a layer's sum: its quantizer relative to the format F of the aligned sum.
 f8_status make_sibling(const f8_conv_desc *d, const F8Requant &q, int y2_dtype, int fl_y2, void *y2, F8Sibling *sib) {
     if (y2_dtype != F8_U8 && y2_dtype != F8_S8 && y2_dtype != F8_S32 && y2_dtype != F8_S32_RELU)
@@ -515,6 +525,7 @@ struct Step {
     // kind -4: the same for a depthwise layer and the pointwise layer behind it
     FusedPlanPtr fplan;
     DwPwPlanPtr dplan;
+    DwPlanPtr wplan;
     void *y_mid = nullptr;
     F8ConvGeom g;
 };
@@ -1304,6 +1315,17 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                     skip_layer = i + 1;
                 }
             }
+            if (L.d.kind == F8_LAYER_DWCONV && !g_force_direct && stp.kind == F8_LAYER_DWCONV &&
+                !(g_plan_off & (F8_PLAN_OFF_DW_DP4A | F8_PLAN_OFF_DW_WALK)) && f8_dw_tc_supported(stp.g, L.q) &&
+                ((g_plan_off & F8_PLAN_OFF_DWPW_RULE) || f8_dw_tc_wanted(stp.g))) {
+                DwPlanPtr wp = alloc_dw_plan();
+                const char *why = "";
+                if (wp && f8_dw_tc_plan_init(wp.get(), stp.g, L.q, stp.x, L.w, L.b, stp.y, f8_status_word(), &why) == cudaSuccess) {
+                    f8_dw_tc_plan_set_tag(wp.get(), i + 1);
+                    stp.use_tc = true;
+                    stp.wplan = std::move(wp);
+                }
+            }
             ln.steps.push_back(std::move(stp));
         };
         for (int k = 0; k < lanes; ++k) {
@@ -1399,7 +1421,8 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                                                stp.has_sib ? &stp.sib : nullptr);
                 break;
             case F8_LAYER_DWCONV:
-                e = f8_launch_dwconv(stp.g, L.q, stp.x, L.w, L.b, stp.res, stp.y, st, net->overlap_layers);
+                if (stp.wplan) { e = f8_dw_tc_launch(stp.wplan.get(), net->overlap_layers, st); ++g_tc_launches; }
+                else e = f8_launch_dwconv(stp.g, L.q, stp.x, L.w, L.b, stp.res, stp.y, st, net->overlap_layers);
                 break;
             case F8_LAYER_MAXPOOL:
                 e = f8_launch_maxpool(stp.g.n, L.g.h, L.g.w, L.g.c, L.d.conv.kh, L.d.conv.stride, L.d.conv.pad, L.g.x_signed,

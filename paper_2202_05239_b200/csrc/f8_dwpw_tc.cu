@@ -734,6 +734,10 @@ bool f8_dwpw_wanted(const F8ConvGeom &g1, int c_out2, bool res) {
     g2.pad_h = g2.pad_w = 0;
     if (f8_small_tc_wanted(g2)) return false;
     const double m = (double)g1.n * g1.ho * g1.wo, c = g1.c, n = c_out2;
+    // Larger layers are faster apart, with the depthwise one on f8_dw_tc_kernel, which shares an instruction among three vertical taps
+    // where this one spends one on each.  From where on depends on what the pointwise layer adds: whole networks with the line at
+    // 2.4 and at 8 million outputs, MobileNet V2 (one part) at batch 64 487.8 and 480.9 us, MobileNet V1 (two to eight) 258.2 and 265.0.
+    if (m * c >= (g1.stride_h == 1 && p.parts == 1 ? 8.0e6 : 2.4e6)) return false;
     const double tiles = p.win ? (double)g1.n * p.win_bands : std::ceil(m / DP_TILE_M);
     const double issue = p.slabs * (p.win ? 2600.0 : 4500.0), parts = p.parts * p.bn2 / 128.0;
     const double convert = p.slabs * 1000.0 + std::max(parts, 0.5) * 1300.0 + 600.0;

@@ -114,6 +114,16 @@ cudaError_t f8_dwpw_plan_init(F8DwPwPlan *plan, const F8ConvGeom &g1, const F8Re
 void f8_dwpw_plan_set_tag(F8DwPwPlan *plan, int tag);
 cudaError_t f8_dwpw_launch(const F8DwPwPlan *plan, bool overlap_previous, cudaStream_t st);
 
+// ---- depthwise 3x3 on the tensor cores (f8_dw_tc.cu), 8-bit output, no shortcut
+struct F8DwPlan;
+bool f8_dw_tc_supported(const F8ConvGeom &g, const F8Requant &q);
+bool f8_dw_tc_wanted(const F8ConvGeom &g);
+size_t f8_dw_tc_plan_size();
+cudaError_t f8_dw_tc_plan_init(F8DwPlan *plan, const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias, void *y,
+                               int *status_word, const char **why);
+void f8_dw_tc_plan_set_tag(F8DwPlan *plan, int tag);
+cudaError_t f8_dw_tc_launch(const F8DwPlan *plan, bool overlap_previous, cudaStream_t st);
+
 // ---- first-layer kernel (f8_stem_tc.cu): stride-2 convolution over an image with <= 4 channels, optionally fused
 // with the 3x3 / 2 / pad 1 max pool behind it.  kh2 row pairs per window starting `top` pairs above the output row,
 // `left` zero cells in front of a row, `slices` 32-byte K slices per row pair; w_core is [K / 16][c_out][16].
