@@ -377,9 +377,11 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
 //   * The maximum over three columns works on 16-bit lanes of packed bytes: the high bytes of a lane decide whatever lies
 //     below them, so a word costs two three-operand maxima and three shifts.
 //   * Without a pool a thread stores its pixel's channels straight from registers.
-// Measured (224 x 224 images, batch 256, B200): 7 x 7 to 64 channels with the pool 140 -> 82 us, 3 x 3 to 32 channels without a
-// pool 105 -> 62 us; one image 21 -> 17 us.  The pooling conversion is what bounds the first (its warps wait 10 % of the time;
-// the instruction slots are 55 % used), the packing of the lines the second (a fourth packing warp: no change).
+//   * Three-channel rows of a multiple of four pixels are read four pixels at a time, from three words, instead of two words around
+//     every pixel: half the loads, no shift by a variable amount.
+// Measured (224 x 224 images, batch 256, B200): 7 x 7 to 64 channels with the pool 140 -> 82 us, with four pixels at a time 103 -> 91
+// (timed inside a network); 3 x 3 to 32 channels without a pool 105 -> 62 us, 69.7 -> 54.6; one image 21 -> 17 us.  The pooling
+// conversion is what bounds the first, the packing of the lines the second (a fourth packing warp: 97.6 and 57.8).
 constexpr int ROWS_EPI_WARPS = 8;
 constexpr int ROWS_PACK_WARPS = 3;
 constexpr int ROWS_MMA_WARP = ROWS_EPI_WARPS + ROWS_PACK_WARPS;
@@ -398,8 +400,13 @@ __device__ __forceinline__ uint32_t max3_bytes(uint32_t a, uint32_t b, uint32_t 
     return __byte_perm(hi, lo, 0x3715);
 }
 
+// How the packing warps read the image: byte by byte; the two aligned words around a pixel (FAST above); or, three channels and rows
+// of a multiple of four pixels that start at a word, four pixels from three words.
+constexpr int READ_BYTES = 0, READ_WORDS = 1, READ_QUADS = 2;
+constexpr int ROWS_QUADS = (2 * STEM_MAX_CELLS / 4 + 32 * ROWS_PACK_WARPS - 1) / (32 * ROWS_PACK_WARPS);      // of two lines, per thread
+
 // CH: 16-byte chunks per pixel this instantiation has registers for (2 or 4; p.cpr <= CH).
-template <int CH, bool POOL, bool SIGNED, bool FAST>
+template <int CH, bool POOL, bool SIGNED, int READ>
 __global__ void __launch_bounds__(ROWS_THREADS, 2) f8_stem_rows_tc_kernel(const StemParams p, const int units_total) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t line_bars[ROWS_AHEAD];      // the lines a step adds have been packed
@@ -480,7 +487,18 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) f8_stem_rows_tc_kernel(const 
         // The words of a line's pixels, all requested before the first is used (a load behind a branch of its own, with its
         // use in the same branch, waits for memory once per cell: 4000 cycles a line instead of 900); combined when the line
         // is stored.
+        constexpr bool FAST = READ == READ_WORDS;
         uint32_t raw[2][ROWS_CELLS][2][FAST ? 2 : 1];        // two lines at a time
+        // READ_QUADS: item pt + 96 j is a quad of the two lines
+        const int quads = p.w / 4;
+        uint32_t quad[ROWS_QUADS][2][3], quad_off[ROWS_QUADS];
+        int quad_line[ROWS_QUADS];                           // 0, 1; 2: none
+#pragma unroll
+        for (int j = 0; j < ROWS_QUADS; ++j) {
+            const int i = pt + j * 32 * ROWS_PACK_WARPS;
+            quad_line[j] = i < quads ? 0 : (i < 2 * quads ? 1 : 2);
+            quad_off[j] = (uint32_t)(i - (quad_line[j] == 1 ? quads : 0));
+        }
         uint32_t row_off[2][2] = {{0u, 0u}, {0u, 0u}}, second_mask[2] = {0u, 0u};
         auto load_lines = [&](int img, int pr0) {
 #pragma unroll
@@ -489,6 +507,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) f8_stem_rows_tc_kernel(const 
                 row_off[l][0] = ((uint32_t)img * p.h + 2u * pr) * img_row_bytes;
                 second_mask[l] = 2 * pr + 1 < p.h ? 0xffffffffu : 0u;
                 row_off[l][1] = row_off[l][0] + (img_row_bytes & second_mask[l]);
+                if (READ != READ_QUADS)
 #pragma unroll
                 for (int i = 0; i < ROWS_CELLS; ++i)
 #pragma unroll
@@ -501,6 +520,34 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) f8_stem_rows_tc_kernel(const 
                             raw[l][i][e][0] = load_pixel<false>(p.x, off, last_word, p.c);
                         }
                     }
+            }
+            if (READ == READ_QUADS)
+#pragma unroll
+                for (int j = 0; j < ROWS_QUADS; ++j)
+                    if (quad_line[j] < 2)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e)
+#pragma unroll
+                            for (int w = 0; w < 3; ++w)
+                                quad[j][e][w] = ldg32(p.x + (quad_line[j] == 0 ? row_off[0][e] : row_off[1][e]) + 12u * quad_off[j] + 4u * w);
+        };
+        auto store_quads = [&](int line, int n) {
+#pragma unroll
+            for (int j = 0; j < ROWS_QUADS; ++j) {
+                if (quad_line[j] >= n) continue;
+                uint2 *dst = (uint2 *)(line_ptr + ((line + quad_line[j]) & (ROWS_LINES - 1)) * STEM_SLOT_BYTES) + p.left + 4 * quad_off[j];
+                const uint32_t mask = quad_line[j] == 0 ? second_mask[0] : second_mask[1];
+                uint32_t px[2][4];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const uint32_t *w = quad[j][e];
+                    px[e][0] = w[0] & 0xffffffu;
+                    px[e][1] = __funnelshift_r(w[0], w[1], 24) & 0xffffffu;
+                    px[e][2] = __funnelshift_r(w[1], w[2], 16) & 0xffffffu;
+                    px[e][3] = w[2] >> 8;
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) dst[i] = make_uint2(px[0][i], px[1][i] & mask);
             }
         };
         auto line_cell = [&](int l, int i) {
@@ -530,6 +577,8 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) f8_stem_rows_tc_kernel(const 
                 if (!__all_sync(0xffffffffu, got)) { ok = false; break; }
                 const int pr_end = min(p.hp, 2 * r + 1 - p.top + p.kh2);
                 while (pr < pr_end) {
+                    if (READ == READ_QUADS) store_quads(line, min(2, pr_end - pr));
+                    else
 #pragma unroll
                     for (int l = 0; l < 2; ++l)
                         if (pr + l < pr_end) {
@@ -748,13 +797,14 @@ StemKernel pick_wide(bool fast) {
     return fast ? f8_stem_tc_kernel<POOL, SIGNED, true> : f8_stem_tc_kernel<POOL, SIGNED, false>;
 }
 template <int CH, bool POOL, bool SIGNED>
-StemKernel pick_rows(bool fast) {
-    return fast ? f8_stem_rows_tc_kernel<CH, POOL, SIGNED, true> : f8_stem_rows_tc_kernel<CH, POOL, SIGNED, false>;
+StemKernel pick_rows(int read) {
+    return read == READ_QUADS ? f8_stem_rows_tc_kernel<CH, POOL, SIGNED, READ_QUADS>
+                              : (read == READ_WORDS ? f8_stem_rows_tc_kernel<CH, POOL, SIGNED, READ_WORDS> : f8_stem_rows_tc_kernel<CH, POOL, SIGNED, READ_BYTES>);
 }
 template <int CH>
-StemKernel pick_rows(bool pool, bool sgn, bool fast) {
-    if (pool) return sgn ? pick_rows<CH, true, true>(fast) : pick_rows<CH, true, false>(fast);
-    return sgn ? pick_rows<CH, false, true>(fast) : pick_rows<CH, false, false>(fast);
+StemKernel pick_rows(bool pool, bool sgn, int read) {
+    if (pool) return sgn ? pick_rows<CH, true, true>(read) : pick_rows<CH, true, false>(read);
+    return sgn ? pick_rows<CH, false, true>(read) : pick_rows<CH, false, false>(read);
 }
 StemKernel pick_wide(bool pool, bool sgn, bool fast) {
     if (pool) return sgn ? pick_wide<true, true>(fast) : pick_wide<true, false>(fast);
@@ -801,8 +851,9 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
     p.wait_limit = f8_wait_limit_cycles();
 
     const bool fast = ((uintptr_t)x & 3) == 0 && ((size_t)g.n * g.h * g.w * g.c) % 4 == 0;
+    const int read = !fast ? READ_BYTES : (g.c == 3 && g.w % 4 == 0 && left + g.w <= STEM_MAX_CELLS ? READ_QUADS : READ_WORDS);
     const bool sgn = p.signed_out != 0;
-    StemKernel kernel = !rows ? pick_wide(pool != 0, sgn, fast) : (p.cpr > 2 ? pick_rows<4>(pool != 0, sgn, fast) : pick_rows<2>(pool != 0, sgn, fast));
+    StemKernel kernel = !rows ? pick_wide(pool != 0, sgn, fast) : (p.cpr > 2 ? pick_rows<4>(pool != 0, sgn, read) : pick_rows<2>(pool != 0, sgn, read));
     const size_t smem = rows ? stem_rows_smem_bytes(kh2, slices, g.c_out, pool != 0) : stem_smem_bytes(kh2, slices, g.c_out);
     const int threads = rows ? ROWS_THREADS : STEM_THREADS, accs = rows ? ROWS_ACCS : 2;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024));

@@ -107,6 +107,8 @@ ROWS_EDGE_CASES = [
     (256, 256, 3, 64, 7, 3, 1, synth.U8, True),     # 128 outputs per row; as many bands as rows
     (33, 31, 3, 64, 8, 4, 5, synth.S8, True),       # windows of eight taps: five row pairs, six per step
     (95, 97, 3, 16, 3, 1, 2, synth.U8, True),       # byte count of a row not a multiple of four
+    (33, 32, 3, 48, 7, 3, 4, synth.U8, True),       # four pixels at a time, the last row without a partner
+    (31, 4, 3, 16, 3, 1, 5, synth.S8, False),       # one group of four pixels per row
 ]
 
 
