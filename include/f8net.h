@@ -401,6 +401,13 @@ enum {
 };
 int f8_debug_last_plan(int *info, int n);
 
+/* How the kernel that runs a depthwise 3x3 layer and the pointwise layer with c_out channels behind it in one launch would cut
+ * them (host arithmetic only; n >= 12 ints are written, the count is returned, 0 when the pair does not fit the kernel):
+ * [0] whether f8_net_forward prefers it, [1] tiles, [2] slabs of 128 channels, [3] slots that hold converted slabs, [4] parts of
+ * the output channels, [5] accumulators of the pointwise layer, [6] second epilogue deferred behind the next tile's slabs,
+ * [7] activation loads per slab, [8] activation stages, [9] weight stages, [10] weights resident, [11] output buffers. */
+int f8_debug_dwpw_layout(const f8_conv_desc *dw, int c_out, int residual, int *info, int n);
+
 /* Bound of every in-kernel barrier wait, in milliseconds at the maximum SM clock (0 restores the default of
  * about two seconds).  Process-wide; for kernels launched after the call. */
 void f8_debug_set_wait_limit_ms(double ms);

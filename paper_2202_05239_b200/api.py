@@ -298,6 +298,18 @@ def f8_debug_last_plan() -> dict:
     return dict(zip(keys, [int(x) for x in v]))
 
 
+_lib.f8_debug_dwpw_layout.argtypes = [ctypes.POINTER(ConvDesc), _ci, _ci, ctypes.POINTER(_ci), _ci]
+
+
+def f8_debug_dwpw_layout(desc: ConvDesc, c_out: int, residual: bool) -> Optional[dict]:
+    """How the depthwise + pointwise kernel would cut this pair of layers; None when it does not take them."""
+    v = (ctypes.c_int * 12)()
+    if _lib.f8_debug_dwpw_layout(ctypes.byref(desc), c_out, 1 if residual else 0, v, 12) != 12:
+        return None
+    keys = ("wanted", "tiles", "slabs", "slots", "parts", "accs2", "defer", "loads", "a_stages", "w_stages", "w_res", "out_bufs")
+    return dict(zip(keys, v))
+
+
 def f8_debug_set_wait_limit_ms(ms: float):
     _lib.f8_debug_set_wait_limit_ms(ms)
 

@@ -303,6 +303,13 @@ int f8_debug_last_plan(int *info, int n) {
     return m;
 }
 
+int f8_debug_dwpw_layout(const f8_conv_desc *dw, int c_out, int residual, int *info, int n) {
+    F8ConvGeom g;
+    F8Requant q;
+    if (!info || n < 12 || c_out <= 0 || check_conv(dw, true, false, &g, &q) != F8_OK) return 0;
+    return f8_dwpw_layout_info(g, c_out, residual != 0, info);
+}
+
 void f8_debug_set_wait_limit_ms(double ms) {
     int dev = 0, khz = 1965000;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev);

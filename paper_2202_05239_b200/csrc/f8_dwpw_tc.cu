@@ -658,8 +658,10 @@ bool dp_layout(const F8ConvGeom &g, int c_out, bool res, DpParams *p, size_t *sm
         p->w_bytes = (uint32_t)((p->bn2 * DP_SLAB + 1023) / 1024 * 1024);
         // With one part GEMM 2 lets go of a tile's slabs one by one; several parts read all of them over again, so all have to be there
         // at once -- twice, if the epilogue of a tile's parts is to wait until the next tile's slabs have been converted.
+        // With a single accumulator that wait must not depend on GEMM 2 of the next tile: it cannot start before that epilogue has read
+        // the accumulator, so it lets go of no slab, and the next tile's slabs have to fit the slots without it.
         p->slots = p->parts > 1 ? std::max(2, p->slabs) : 2;
-        p->defer = p->parts > 1 ? 0 : 1;
+        p->defer = p->parts > 1 || (p->accs2 == 1 && p->slabs > p->slots) ? 0 : 1;
         if (p->slots > DP_MAX_SLOTS) continue;
         const int tiles = p->parts * p->slabs, min_a = 2;
         for (p->out_bufs = 2; p->out_bufs >= 1; --p->out_bufs) {
@@ -741,12 +743,23 @@ bool f8_dwpw_wanted(const F8ConvGeom &g1, int c_out2, bool res) {
     const double tiles = p.win ? (double)g1.n * p.win_bands : std::ceil(m / DP_TILE_M);
     const double issue = p.slabs * (p.win ? 2600.0 : 4500.0), parts = p.parts * p.bn2 / 128.0;
     const double convert = p.slabs * 1000.0 + std::max(parts, 0.5) * 1300.0 + 600.0;
-    // without `defer` GEMM 2 and the second epilogue do not overlap the tile's own slabs
-    const double tile = p.defer ? std::max(issue, convert) + 800.0 : issue + p.parts * (p.slabs * (2.0 * p.bn2 + 200.0) + 1500.0);
+    // several parts without `defer`: GEMM 2 and the second epilogue do not overlap the tile's own slabs
+    const double tile = p.defer || p.parts == 1 ? std::max(issue, convert) + 800.0 : issue + p.parts * (p.slabs * (2.0 * p.bn2 + 200.0) + 1500.0);
     const double fused = 6.5 + (std::ceil(tiles / 148.0) * tile + 3000.0) / 1900.0;
     const double dw = 7.0 + m * c * (g1.stride_h == 1 ? 0.62e-6 : 1.35e-6);
     const double pw = std::max(8.0, 9.0 + std::max(m * (c + n) / 6.4e6, m * c * n / 1.0e9));
     return fused < 0.9 * (dw + pw);
+}
+
+int f8_dwpw_layout_info(const F8ConvGeom &g1, int c_out2, bool res, int *info) {
+    DpParams p;
+    size_t smem;
+    if (!dp_layout(g1, c_out2, res, &p, &smem)) return 0;
+    const int tiles = p.win ? g1.n * p.win_bands : (g1.n * g1.ho * g1.wo + DP_TILE_M - 1) / DP_TILE_M;
+    const int v[12] = {f8_dwpw_wanted(g1, c_out2, res) ? 1 : 0, tiles, p.slabs, p.slots, p.parts, p.accs2, p.defer, p.win ? 1 : DP_TAPS,
+                       p.a_stages, p.w_stages, p.w_res, p.out_bufs};
+    std::copy(v, v + 12, info);
+    return 12;
 }
 
 cudaError_t f8_dwpw_plan_init(F8DwPwPlan *plan, const F8ConvGeom &g1, const F8Requant &q1, int c_out2, const F8Requant &q2, const void *x,

@@ -107,6 +107,7 @@ cudaError_t f8_fused_launch(const F8FusedPlan *plan, bool overlap_previous, cuda
 struct F8DwPwPlan;
 bool f8_dwpw_supported(const F8ConvGeom &g1, const F8Requant &q1, int c_out2, const F8Requant &q2);
 bool f8_dwpw_wanted(const F8ConvGeom &g1, int c_out2, bool res);
+int f8_dwpw_layout_info(const F8ConvGeom &g1, int c_out2, bool res, int *info /* 12; see f8_debug_dwpw_layout */);
 size_t f8_dwpw_plan_size();
 cudaError_t f8_dwpw_plan_init(F8DwPwPlan *plan, const F8ConvGeom &g1, const F8Requant &q1, int c_out2, const F8Requant &q2, const void *x,
                               const int8_t *w_dw, const int32_t *bias1, const int8_t *w_pw, const int32_t *bias2, const void *res,

@@ -21,7 +21,14 @@ CASES = [
     (7, 7, 960, 160, 1, 40, False, synth.S8, True),        # eight slabs, wide part, shortcut
     (56, 56, 64, 128, 2, 60, False, synth.U8, False),      # half a slab, many tiles per CTA
     (9, 7, 192, 96, 1, 130, True, synth.U8, True),         # ragged last tile, 96 of 128 columns, shortcut in u8 / s8
+    # more slabs than slots and several tiles per CTA: the slots are used again while the epilogue of the tile before is open
+    (14, 14, 384, 64, 1, 230, False, synth.S8, False),     # two accumulators, three or four tiles per CTA
+    (14, 14, 320, 96, 1, 160, True, synth.S8, True),       # the same with a shortcut
+    (37, 37, 400, 144, 1, 14, False, synth.U8, False),     # one wide part, one accumulator
+    (13, 13, 544, 144, 1, 90, False, synth.U8, True),      # the same with five slabs and a shortcut
+    (14, 14, 528, 160, 2, 420, True, synth.S8, False),     # the same at stride 2
 ]
+SLOT_REUSE = {10: 2, 11: 2, 12: 1, 13: 1, 14: 1}           # case: accumulators of the pointwise layer
 
 
 @pytest.mark.parametrize("case", range(len(CASES)))
@@ -42,6 +49,9 @@ def test_depthwise_pointwise(ref, request, case):
         layers = [short, dw, pw]
     x = random_input(rng, n, layers[0])
     want = ref.net_forward(layers, x)
+    if case in SLOT_REUSE:
+        lay = a.f8_debug_dwpw_layout(a.conv_desc(dw, n), c_out, with_res)
+        assert lay["accs2"] == SLOT_REUSE[case] and lay["slabs"] > lay["slots"] and lay["tiles"] > 148 * lay["accs2"]
     net = a.Net(layers, n)
     a.f8_debug_plan_options(32768)      # the pair in one launch wherever the kernel applies, not only where it is the faster one
     request.addfinalizer(lambda: a.f8_debug_plan_options(0))
