@@ -925,16 +925,25 @@ f8_status f8_net_create(const f8_layer_desc *layers, int n_layers, const int8_t 
     // Stored channel counts: intermediate 8-bit tensors whose channel count is not a multiple of 16 (24 in
     // MobileNetV2) are padded with channels that are identically zero -- zero weights and bias produce them,
     // zero weights consume them -- so the arithmetic of the real channels is untouched.
+    // Tensors whose elements a launch addresses with one channel count have the same number stored: input and output of a
+    // pooling or depthwise layer, a shortcut and the output it is added to, both outputs of a sum.  Where one of them is the caller's
+    // (the network's input or output) or a layer's 32-bit output, none of them is padded.
     net->t_cp = net->t_c;
-    for (int t = 1; t < n_layers; ++t)
-        if (net->t_elem[t] == 1 && net->t_c[t] % 16 != 0) net->t_cp[t] = (net->t_c[t] + 15) / 16 * 16;
-    // both outputs of a launch have the same number of stored channels
-    for (int i = 1; i < n_layers; ++i)
-        if (net->layers[i].d.kind == F8_LAYER_SIBLING) {
-            if (i + 1 == n_layers && net->t_cp[i] != net->t_c[i])
-                return cleanup(fail(F8_ERR_UNSUPPORTED, "layer %d: the network output cannot be the sibling of a layer with padded channels", i));
-            net->t_cp[i + 1] = net->t_cp[i];
-        }
+    std::vector<int> same(n_layers + 1);
+    for (int t = 0; t <= n_layers; ++t) same[t] = t;
+    auto root = [&](int t) { while (same[t] != t) t = same[t]; return t; };
+    for (int i = 0; i < n_layers; ++i) {
+        const NetLayer &L = net->layers[i];
+        if (L.d.kind != F8_LAYER_CONV && L.d.kind != F8_LAYER_LINEAR) same[root(L.d.src)] = root(i + 1);
+        if (L.q.has_res && L.d.res >= 0) same[root(L.d.res)] = root(i + 1);
+    }
+    std::vector<char> plain(n_layers + 1, 0);
+    for (int t = 0; t <= n_layers; ++t)
+        if (t == 0 || t == n_layers || (net->t_elem[t] != 1 && net->layers[t - 1].d.kind != F8_LAYER_SIBLING)) plain[root(t)] = 1;
+    for (int t = 0; t <= n_layers; ++t)
+        if (!plain[root(t)] && net->t_c[t] % 16 != 0) net->t_cp[t] = (net->t_c[t] + 15) / 16 * 16;
+    if (net->layers[n_layers - 1].d.kind == F8_LAYER_SIBLING && net->t_elem[n_layers - 1] == 1 && net->t_c[n_layers] % 16 != 0)
+        return cleanup(fail(F8_ERR_UNSUPPORTED, "layer %d: the network output cannot be the sibling of a layer with padded channels", n_layers - 1));
     // second pass (everything validated): upload the parameters
     for (int i = 0; i < n_layers; ++i) {
         NetLayer &L = net->layers[i];

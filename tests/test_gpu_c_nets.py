@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from paper_2202_05239_b200 import synth
-from gpu_util import api, Guarded, assert_equal_arrays
+from gpu_util import api, Guarded, assert_equal_arrays, random_conv_layer, random_input
 
 pytestmark = pytest.mark.gpu
 
@@ -233,3 +233,63 @@ def test_host_pipeline_matches_oracle(ref):
         want = ref.net_forward(layers, x.numpy(), keep_all=False)[-1]
         assert np.array_equal(y.numpy(), want), f"batch {i}"
     pipe.close()
+
+
+def _pool(kind, src, x, k=3, stride=2, pad=1):
+    k = x.ho if kind == synth.GAP else k
+    return synth.Layer(kind, "pool", src, -1, x.ho, x.wo, x.c_out, x.c_out, k, k, 1 if kind == synth.GAP else stride, 0 if kind == synth.GAP else pad,
+                       x.y_dtype, x.y_dtype, 0, x.fl_y, 0, x.fl_y, 0, None, None)
+
+
+def _channel_nets(case):
+    """Networks whose tensors of 24 (or 3) channels meet the caller's tensors through layers that keep the channel count."""
+    rng = np.random.default_rng(5200 + case)
+
+    def conv(c, c_out, k=1, size=9, fl_x=4, kind=synth.CONV, src=0, res=None, y_dtype=synth.U8):
+        l = random_conv_layer(rng, h=size, w=size, c=c, c_out=c_out, k=k, stride=1, pad=k // 2, x_signed=False, y_dtype=y_dtype, with_res=res is not None,
+                              kind=kind, fl_x=fl_x, fl_w=6, fl_y=4, fl_r=4)
+        l.src, l.res, l.r_dtype = src, -1 if res is None else res, synth.U8
+        return l
+    a = conv(16, 24)
+    if case == 0:       # the network's input goes through a pool
+        first = conv(3, 3)
+        p = _pool(synth.MAXPOOL, 0, first)
+        return [p, conv(3, 16, size=p.ho, src=1)]
+    if case == 1:       # ... and through a depthwise layer
+        return [conv(24, 24, k=3, kind=synth.DWCONV), conv(24, 16, src=1)]
+    if case == 2:       # the network's output comes from a max pool, ...
+        return [a, _pool(synth.MAXPOOL, 1, a)]
+    if case == 3:       # ... a global average, ...
+        return [a, conv(24, 24, k=3, src=1), _pool(synth.GAP, 2, a)]
+    if case == 4:       # ... a depthwise layer, ...
+        return [a, conv(24, 24, k=3, kind=synth.DWCONV, src=1)]
+    if case == 5:       # ... a layer with a shortcut, ...
+        return [a, conv(24, 24, src=1), conv(24, 24, src=2, res=1)]
+    if case == 6:       # ... or a chain of them, one end of which another layer reads
+        d = conv(24, 24, k=3, kind=synth.DWCONV, src=1)
+        return [a, d, conv(24, 24, src=2, res=1), conv(24, 24, k=3, kind=synth.DWCONV, src=3)]
+    # the network's input is the shortcut
+    return [conv(24, 16), conv(16, 24, src=1, res=0), conv(24, 16, src=2)]
+
+
+@pytest.mark.parametrize("direct", [False, True])
+@pytest.mark.parametrize("case", range(8))
+def test_channels_that_are_no_multiple_of_16_at_the_ends_of_a_network(ref, request, case, direct):
+    a = api()
+    layers, batch = _channel_nets(case), 5
+    x = random_input(np.random.default_rng(case), batch, layers[0])
+    want = ref.net_forward(layers, x)
+    a.f8_debug_force_direct(direct)
+    request.addfinalizer(lambda: a.f8_debug_force_direct(False))
+    net = a.Net(layers, batch)
+    guards = [Guarded(_layer_shape(l, batch), a.torch_dtype(l.y_dtype)) for l in layers]
+    out, ws = Guarded((batch,) + net.out_shape, net.out_dtype), Guarded((net.workspace_bytes(batch),), torch.uint8)
+    net.forward(a.to_device(x), out=out.t, workspace=ws.t, dump=[g.t for g in guards])
+    torch.cuda.synchronize()
+    a.f8_device_status()
+    assert out.intact() and ws.intact()
+    assert_equal_arrays(out.t.cpu().numpy().reshape(want[-1].shape), want[-1], "output: ")
+    for i, g in enumerate(guards):
+        assert g.intact()
+        assert_equal_arrays(g.t.cpu().numpy().reshape(want[i + 1].shape), want[i + 1], f"layer {i}: ")
+    net.close()
