@@ -1213,10 +1213,26 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
     auto is32 = [](int kind) { return kind == F8_S32 || kind == F8_S32_RELU; };
     const bool pointwise1 = g.kh == 1 && g.kw == 1 && g.stride_h == 1 && g.stride_w == 1 && g.pad_h == 0 && g.pad_w == 0;
     const bool big_x = (size_t)xv.dim_c * xv.dim_w * xv.dim_h * xv.dim_n >= 128 * 1024;
+    // How a buffer of the ring is cut for tiles of bn columns, and whether two pipeline stages fit beside the ring and the table of
+    // all biases (a fully connected layer to 32 bits: up to 27000 outputs; beyond that direct stores, which need neither: 64 x 512
+    // to 50000 outputs 25 us, on the CUDA cores 1550).
+    auto wide_ring = [&](int bn) {
+        p.wide_out32 = is32(q.y_kind) ? 1 : (has_sib && is32(sib->y_kind) ? 2 : 0);
+        p.wide_slabs = p.wide_out32 || q.r_s32 ? (bn + 31) / 32 : 0;
+        const uint32_t w32 = (uint32_t)p.wide_slabs * TILE_M * 128, w8 = (uint32_t)(TILE_M * bn);
+        const bool q1 = p.wide_out32 != 1, q2 = (has_sib && p.wide_out32 != 2) || (q.has_res && !q.r_s32);
+        p.wide_q1 = w32;
+        p.wide_q2 = w32 + (q1 ? w8 : 0);
+        p.out_bytes = w32 + (q1 ? w8 : 0) + (q2 ? w8 : 0);
+        p.out_bufs = bn == 128 ? 1 : (q.has_res ? 3 : 2);
+        const size_t tables = ((size_t)(g.c_out + bn - 1) / bn * bn * 4 + 1023) / 1024 * 1024 + ((size_t)g.kh * g.kw * p.c_chunks * 8 + 1023) / 1024 * 1024;
+        const size_t stage = (size_t)(TILE_M * p.kb + 1023) / 1024 * 1024 + (size_t)(bn * p.kb + 1023) / 1024 * 1024;
+        return (size_t)p.out_bytes * p.out_bufs + tables + 2 * stage + 1024 <= SMEM_LIMIT;
+    };
     if (p.epi == EPI_GENERIC && g.c_out % 16 == 0 && (big_x || pointwise1) && (is32(q.y_kind) || (q.s >= 1 && q.s <= 31)) &&
         (!has_sib || is32(sib->y_kind) || (sib->s >= 1 && sib->s <= 31)) && !(has_sib && is32(q.y_kind) && is32(sib->y_kind)) &&
         (g.c_out > 16 || !(is32(q.y_kind) || q.r_s32 || (has_sib && is32(sib->y_kind)))))
-        p.epi = EPI_WIDE;
+        p.epi = wide_ring(g.c_out > 32 ? 64 : 32) ? EPI_WIDE : EPI_GENERIC;
     const bool wide = p.epi == EPI_WIDE;
     const bool staged = p.epi != EPI_GENERIC;
     p.bn = wide ? (g.c_out > 32 ? 64 : 32) : staged ? (k_heavy_res ? 256 : choose_bn_staged(g.c_out, q.has_res != 0, p.kb)) : choose_bn(g.c_out);
@@ -1227,7 +1243,8 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
         int sm_count = 148, dev0 = 0;
         cudaGetDevice(&dev0);
         cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev0);
-        if ((long long)p.m_tiles * ((g.c_out + 127) / 128) <= sm_count && (long long)p.m_tiles * ((g.c_out + 63) / 64) > sm_count) p.bn = 128;
+        if ((long long)p.m_tiles * ((g.c_out + 127) / 128) <= sm_count && (long long)p.m_tiles * ((g.c_out + 63) / 64) > sm_count && wide_ring(128))
+            p.bn = 128;
     }
     if (!staged) {
         // few output pixels (a fully connected layer): narrower N tiles until every SM has one, the weights are
@@ -1294,14 +1311,7 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
             }
         }
         if (wide) {
-            p.wide_out32 = is32(q.y_kind) ? 1 : (has_sib && is32(sib->y_kind) ? 2 : 0);
-            p.wide_slabs = p.wide_out32 || q.r_s32 ? (p.bn + 31) / 32 : 0;
-            const uint32_t w32 = (uint32_t)p.wide_slabs * TILE_M * 128, w8 = (uint32_t)(TILE_M * p.bn);
-            const bool q1 = p.wide_out32 != 1, q2 = (has_sib && p.wide_out32 != 2) || (q.has_res && !q.r_s32);
-            p.wide_q1 = w32;
-            p.wide_q2 = w32 + (q1 ? w8 : 0);
-            p.out_bytes = w32 + (q1 ? w8 : 0) + (q2 ? w8 : 0);
-            p.out_bufs = p.bn == 128 ? 1 : (q.has_res ? 3 : 2);
+            wide_ring(p.bn);
             p.epi_groups = p.bn >= 64 ? 4 : 2;
         }
         staging = (size_t)p.out_bytes * p.out_bufs + bias_bytes;

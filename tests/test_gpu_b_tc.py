@@ -235,3 +235,11 @@ def test_linear_on_tensor_cores(ref):
     layer = synth.Layer(synth.LINEAR, "fc", 0, -1, 1, 1, k, out, 1, 1, 1, 0, synth.U8, synth.S32, synth.U8, 6, 9, 3, 0, wgt, bias)
     x = rng.integers(0, 256, size=(n, k)).astype(np.uint8)
     check_layer(ref, layer, x, expect_tc=True)
+
+
+@pytest.mark.parametrize("c,c_out,n", [(512, 26992, 40), (512, 27024, 40), (512, 50000, 33), (96, 57344, 200)])
+def test_fully_connected_layers_with_many_outputs(ref, c, c_out, n):
+    """32-bit outputs on both sides of the channel count whose bias table fits beside the staged epilogue's buffers."""
+    layer = random_conv_layer(np.random.default_rng(c_out), h=1, w=1, c=c, c_out=c_out, k=1, stride=1, pad=0, x_signed=False, y_dtype=synth.S32,
+                              with_res=False)
+    check_layer(ref, layer, random_input(np.random.default_rng(1), n, layer), expect_tc=True)

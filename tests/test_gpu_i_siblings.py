@@ -32,6 +32,7 @@ CASES = [
     (31, 30, 64, 32, 3, 2, 5, False, S8, U8, S8, True),          # 32-wide tiles, two 8-bit outputs, 8-bit shortcut in place
     (20, 20, 64, 16, 1, 1, 9, False, U8, S8, S8, True),          # 16 columns in a 32-wide tile, no 32-bit tile
     (20, 20, 64, 16, 1, 1, 9, False, U8, S32, S8, True),         # 16 columns in 32 bits: direct stores
+    (8, 8, 64, 16384, 1, 1, 5, False, U8, S32R, S32, True),      # so many channels that no ring fits beside their biases: direct stores
 ]
 
 
