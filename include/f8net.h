@@ -338,8 +338,8 @@ const char *f8_last_error(void);
  * abandoned a bounded wait (the word is cleared), F8_ERR_CUDA on a CUDA error, else F8_OK. */
 f8_status f8_device_status(void);
 
-/* Number of tensor-core convolution kernels (tcgen05; mma.sync for small layers of a network) this process has launched so far; lets a
- * caller confirm which path a layer took. */
+/* Number of tensor-core convolution kernels (tcgen05; mma.sync for small layers, of a network or called by themselves) this process
+ * has launched so far; lets a caller confirm which path a layer took. */
 long long f8_tc_launch_count(void);
 
 /* Test hook: non-zero routes every dense layer to the CUDA-core kernel (same results). */
@@ -361,7 +361,7 @@ void f8_debug_force_direct(int on);
  *   F8_PLAN_OFF_LAYER_OVERLAP     f8_net_forward launches without programmatic dependent launch
  *   F8_PLAN_OFF_LAYER_FUSION      f8_net_forward runs a 64 -> 64 convolution and the 64 -> 256 pointwise layer behind it as two launches,
  *                                 and a depthwise 3x3 layer and the pointwise layer behind it too
- *   F8_PLAN_OFF_SMALL_KERNEL      f8_net_forward runs layers of a few microseconds on the tcgen05 kernel as well
+ *   F8_PLAN_OFF_SMALL_KERNEL      layers of a few microseconds run on the tcgen05 kernel as well (where it takes none, on the CUDA cores)
  *   F8_PLAN_OFF_DWPW_RULE         f8_net_forward runs every depthwise 3x3 + pointwise pair that one kernel can take in one launch,
  *                                 not only those where that is faster, and every depthwise layer that the tensor-core kernel can take on it
  *   F8_PLAN_OFF_LANES             f8_net_forward runs the whole batch as one sequence of launches on the caller's stream
@@ -390,8 +390,10 @@ int f8_net_micro_batching(const f8_net *net, int *images);
 void f8_debug_set_lanes(int lanes);
 int f8_net_lanes(const f8_net *net);
 
-/* What the most recent tensor-core plan of this process decided (n <= 10 ints are written, the count is returned):
- * [0] flags below, [1] epilogue variant (0 generic, 1 u8, 2 u8 + residual, 3 s8, 4 s8 + residual), [2] N tile,
+/* What the most recent tcgen05 plan of this process decided (n <= 10 ints are written, the count is returned; all zero when the
+ * last single-layer call, or the last network planned, made none):
+ * [0] flags below, [1] epilogue variant (0 generic, 1 u8, 2 u8 + residual, 3 s8, 4 s8 + residual, 5 with a 32-bit
+ * output or shortcut or a second output), [2] N tile,
  * [3] K bytes per chunk, [4] pipeline stages, [5] K chunks per stage, [6] M tiles, [7] N tiles, [8] CTAs launched,
  * [9] staged output buffers.  Lets a test assert which path a case took and how many tiles each CTA walked. */
 enum {

@@ -183,6 +183,7 @@ f8_status make_sibling(const f8_conv_desc *d, const F8Requant &q, int y2_dtype, 
 f8_status run_dense(const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
                     const void *res, void *y, cudaStream_t st, const F8Sibling *sib = nullptr) {
     if (g.n == 0) return F8_OK;
+    std::fill(g_last_plan, g_last_plan + 10, 0);      // (no plan unless the tcgen05 kernel makes one below)
     const size_t x_bytes = (size_t)g.n * g.h * g.w * g.c;
     // Inputs of a few tiles: the kernel for small layers, which needs no tensor maps (encoding four of them takes the host longer
     // than the layer takes the GPU).  16 x 16 x 16, 3 x 3: 6.8 -> 5.1 us on the host.
@@ -1147,6 +1148,7 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
     net->overlap_layers = !(g_plan_off & F8_PLAN_OFF_LAYER_OVERLAP);
     net->sync_layers = (g_plan_off & F8_PLAN_SYNC_LAYERS) != 0;
     if (replan) {
+        std::fill(g_last_plan, g_last_plan + 10, 0);
         net->steps.clear();
         net->plan_batch = -1;
         const int lanes = lanes_for(net, batch);

@@ -48,3 +48,22 @@ def test_small_layer(ref, case):
         assert g.intact()
         assert_equal_arrays(g.t.cpu().numpy().reshape(want[i + 1].shape), want[i + 1], f"layer {i}: ")
     net.close()
+
+
+def test_the_last_plan_is_not_that_of_an_earlier_call(ref):
+    """f8_debug_last_plan reports the tcgen05 plan of the last call, and none where that call made none."""
+    a = api()
+    rng = np.random.default_rng(2300)
+    large = random_conv_layer(rng, h=28, w=28, c=128, c_out=128, k=3, stride=1, pad=1, x_signed=False, y_dtype=synth.U8, with_res=False)
+    small = random_conv_layer(rng, h=16, w=16, c=16, c_out=16, k=3, stride=1, pad=1, x_signed=False, y_dtype=synth.U8, with_res=False)
+    xl, xs = a.to_device(random_input(rng, 2, large)), a.to_device(random_input(rng, 1, small))
+    a.run_layer(large, xl)
+    assert a.f8_debug_last_plan()["m_tiles"] > 0
+    a.run_layer(small, xs)
+    assert not any(a.f8_debug_last_plan().values())
+    a.run_layer(large, xl)
+    net = a.Net([small], 1)
+    net.forward(xs)
+    assert not any(a.f8_debug_last_plan().values())
+    torch.cuda.synchronize()
+    net.close()
