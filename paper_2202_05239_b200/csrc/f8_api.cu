@@ -180,14 +180,18 @@ f8_status make_sibling(const f8_conv_desc *d, const F8Requant &q, int y2_dtype, 
     return F8_OK;
 }
 
+// One 8-bit output, and a shortcut of 8 bits or none.
+bool is_bits8(const F8Requant &q, const F8Sibling *sib) { return (q.y_kind == F8_U8 || q.y_kind == F8_S8) && !q.r_s32 && !(sib && sib->y2); }
+
 f8_status run_dense(const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
                     const void *res, void *y, cudaStream_t st, const F8Sibling *sib = nullptr) {
     if (g.n == 0) return F8_OK;
     std::fill(g_last_plan, g_last_plan + 10, 0);      // (no plan unless the tcgen05 kernel makes one below)
     const size_t x_bytes = (size_t)g.n * g.h * g.w * g.c;
     // Inputs of a few tiles: the kernel for small layers, which needs no tensor maps (encoding four of them takes the host longer
-    // than the layer takes the GPU).  16 x 16 x 16, 3 x 3: 6.8 -> 5.1 us on the host.
-    if (!g_force_direct && !(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) && x_bytes < 16384 && f8_tc_supported(g, x_bytes) && f8_small_tc_supported(g)) {
+    // than the layer takes the GPU).  16 x 16 x 16, 3 x 3: 6.8 -> 5.1 us on the host.  Not with thousands of output channels or
+    // products per output (31 x 31 x 16, 3 x 3 to 4096 channels 28.9 us, on the tcgen05 kernel 15.7).
+    if (!g_force_direct && !(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) && f8_small_tc_wanted_alone(g, is_bits8(q, sib))) {
         const cudaError_t e = f8_launch_small_tc(g, q, x, w, bias, res, y, st, false, sib);
         if (e != cudaSuccess) return cuda_fail(e, "small conv launch");
         ++g_tc_launches;
@@ -1299,7 +1303,7 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                                return true;
                            }()) {
                     // planned above
-                } else if (!(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) && f8_small_tc_wanted(stp.g)) {
+                } else if (!(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) && f8_small_tc_wanted(stp.g, is_bits8(L.q, stp.has_sib ? &stp.sib : nullptr))) {
                     stp.use_tc = stp.small = true;
                 } else if (f8_tc_supported(stp.g, (size_t)n * L.g.h * L.g.w * L.g.c)) {
                     PlanPtr plan = alloc_plan();

@@ -734,7 +734,7 @@ bool f8_dwpw_wanted(const F8ConvGeom &g1, int c_out2, bool res) {
     g2.h = g1.ho; g2.w = g1.wo; g2.c_out = c_out2;
     g2.kh = g2.kw = g2.stride_h = g2.stride_w = 1;
     g2.pad_h = g2.pad_w = 0;
-    if (f8_small_tc_wanted(g2)) return false;
+    if (f8_small_tc_wanted(g2, true)) return false;
     const double m = (double)g1.n * g1.ho * g1.wo, c = g1.c, n = c_out2;
     // Larger layers are faster apart, with the depthwise one on f8_dw_tc_kernel, which shares an instruction among three vertical taps
     // where this one spends one on each.  From where on depends on what the pointwise layer adds: whole networks with the line at

@@ -1173,6 +1173,27 @@ bool f8_tc_supported(const F8ConvGeom &g, size_t x_bytes) {
     return true;
 }
 
+F8TcTiles f8_tc_tiles(const F8ConvGeom &g, bool bits8) {
+    F8TcTiles t;
+    t.kb = choose_kb(g.c);
+    t.chunks = g.kh * g.kw * ((g.c + t.kb - 1) / t.kb);
+    const bool pointwise = g.kh == 1 && g.kw == 1 && g.stride_h == 1 && g.stride_w == 1 && g.pad_h == 0 && g.pad_w == 0;
+    const bool big = (size_t)g.n * g.h * g.w * g.c >= 128 * 1024;
+    t.row_tiles = !big && !pointwise && g.wo <= TILE_M;
+    const int rows = t.row_tiles ? std::min(TILE_M / g.wo, g.ho) : 1;
+    const long long m_tiles = t.row_tiles ? (long long)g.n * ((g.ho + rows - 1) / rows) : ((long long)g.n * g.ho * g.wo + TILE_M - 1) / TILE_M;
+    if (bits8 && g.c_out % 16 == 0) {
+        t.bn = choose_bn_staged(g.c_out, false, t.kb);
+    } else if (g.c_out % 16 == 0 && (big || pointwise)) {
+        t.bn = g.c_out > 32 ? 64 : 32;
+    } else {
+        t.bn = choose_bn(g.c_out);
+        while (t.bn > 32 && t.bn % 32 == 0 && m_tiles * ((g.c_out + t.bn - 1) / t.bn) < 148) t.bn /= 2;
+    }
+    t.tiles = m_tiles * ((g.c_out + t.bn - 1) / t.bn);
+    return t;
+}
+
 cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant &q, const F8TcTensorView &xv,
                             const int8_t *w, const int32_t *bias, const void *res, void *y, int *status_word,
                             const char **why, const F8Sibling *sib) {

@@ -76,6 +76,13 @@ struct F8TcTensorView {
 // True when this geometry can run on the tensor-core path.
 bool f8_tc_supported(const F8ConvGeom &g, size_t x_bytes);
 bool f8_tc_rowtile_ok(const F8ConvGeom &g);
+// How that path would cut the layer, for estimates of its time (bits8: one 8-bit output, shortcut of 8 bits or none).
+struct F8TcTiles {
+    int bn, kb, chunks;     // columns of a tile, bytes of a K chunk, chunks
+    long long tiles;
+    bool row_tiles;         // whole output rows per tile (small tensors)
+};
+F8TcTiles f8_tc_tiles(const F8ConvGeom &g, bool bits8);
 size_t f8_tc_plan_size();
 // Encodes tensor maps and tile schedule; returns cudaSuccess or an error (no launch).
 cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant &q, const F8TcTensorView &xv,
@@ -135,9 +142,10 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
 
 // ---- small layers (f8_small_tc.cu): implicit GEMM on mma.sync for layers bound by latency; every output kind, shortcut and
 // sibling; c a multiple of 16, c_out of 4, weights, bias, shortcut and outputs 16-byte aligned.  `wanted`: the rule by which a
-// network prefers it to the tcgen05 kernel.
+// network (`alone`: a single-layer call) prefers it to the other kernels; bits8: one 8-bit output, shortcut of 8 bits or none.
 bool f8_small_tc_supported(const F8ConvGeom &g);
-bool f8_small_tc_wanted(const F8ConvGeom &g);
+bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8);
+bool f8_small_tc_wanted_alone(const F8ConvGeom &g, bool bits8);
 cudaError_t f8_launch_small_tc(const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
                                const void *res, void *y, cudaStream_t st, bool overlap_previous, const F8Sibling *sib = nullptr);
 

@@ -273,24 +273,45 @@ bool f8_small_tc_supported(const F8ConvGeom &g) {
     return m > 0 && m < (1ll << 24) && k < (1ll << 24) && g.kh < 256 && g.kw < 256;
 }
 
-// Microseconds a layer takes between its neighbours on this kernel / on the tcgen05 kernel, fitted to event timings of the
-// layers of ResNet-18 / 50 and MobileNet V2 at batches 1 - 64 (B200).  Examples, this kernel against the other: 196 x 256 x 2304
-// (pixels x channels x K) 10.2 / 16.3, 784 x 512 x 128 8.2 / 12.3, 1 x 1000 x 2048 10.4 / 77.8 (not on tensor cores before),
-// 784 x 512 x 4608 22.5 / 22.6, 3136 x 512 x 128 14.3 / 12.1, 12544 x 384 x 64 22.5 / 12.2.
+// Microseconds a layer takes between its neighbours on this kernel / on the tcgen05 kernel / on the CUDA cores, fitted to event timings
+// of the layers of ResNet-18 / 50 and MobileNet V2 at batches 1 - 64 and of 480 layers with up to 2048 channels and filters up to 7 x 7
+// (B200).  Examples, this kernel against the other: 196 x 256 x 2304 (pixels x channels x K) 10.2 / 16.3, 784 x 512 x 128 8.2 / 12.3,
+// 1 x 1000 x 2048 10.4 / 77.8 (not on tensor cores before), 784 x 512 x 4608 22.5 / 22.6, 3136 x 512 x 128 14.3 / 12.1,
+// 12544 x 384 x 64 22.5 / 12.2; alone, 1250 x 184 x 12096 40.4 / 22.7, 2240 x 48 x 25088 72.1 / 41.4, 250 x 16 x 25600 45.6 / 28.0.
+// What decides beyond small sizes: a narrow tcgen05 tile costs half as much per K chunk as a 256-wide one, and this kernel's tiles
+// share the way from the L2 cache, twice as slow per chunk with one tile on every SM as with a few.
 static double small_us(const F8ConvGeom &g) {
     const double m = (double)g.n * g.ho * g.wo, n = g.c_out, k = (double)g.kh * g.kw * g.c;
-    const double big = std::ceil(m / 64) * std::ceil(n / 64);
-    if (big >= 148) return 7.3 + big / 148 * (1.7 + 0.0042 * k);
-    return 7.3 + std::max(1.0, std::ceil(m / 32) * std::ceil(n / 32) / 148 * 0.8) * 0.0015 * k;
+    const double big = std::ceil(m / 64) * std::ceil(n / 64) / 148;
+    // (64 x 64 tiles: from five chunks on the ring fills an SM, and a started round costs a whole one)
+    if (big >= 1) return 7.3 + (k > 5 * SM_KB ? std::ceil(big) : big) * (1.7 + 0.0042 * k);
+    const double full = std::ceil(m / 32) * std::ceil(n / 32) / 148;
+    return 7.3 + (full < 1 ? 0.0014 * (1 + full) : std::max(0.0028, 0.0012 * full)) * k;
 }
-static double tcgen05_us(const F8ConvGeom &g) {
-    const double k = (double)g.kh * g.kw * g.c;
-    return 10.3 + 0.0024 * k;
+static double tcgen05_us(const F8ConvGeom &g, bool bits8) {
+    const F8TcTiles t = f8_tc_tiles(g, bits8);
+    const double wide = 0.0024 * ((double)g.kh * g.kw * g.c);
+    // per chunk; 256-wide tiles with a very long K wait for memory on top
+    const double narrow = t.bn <= 32 ? (t.row_tiles ? 0.10 : 0.14) : (t.bn <= 64 ? (t.row_tiles ? 0.13 : (bits8 ? 0.17 : 0.22)) : 0.25);
+    const double tile = t.bn > 128 ? wide + 0.1 * std::max(0, t.chunks - 64) : std::min(wide, narrow * t.chunks);
+    // (32-bit or two outputs of small tensors leave by direct stores)
+    return (!bits8 && t.row_tiles ? 11.8 : 10.3) + std::ceil((double)t.tiles / 148) * tile;
+}
+// (only the tap inside the image counts there: one pixel, 3 x 3 x 800 to 24 channels 7.4 us, here 14.2)
+static double cuda_core_us(const F8ConvGeom &g) {
+    return g.h == 1 && g.w == 1 ? 7.0 + 0.0095 * g.c * std::max(1.0, (double)g.n * g.ho * g.wo * g.c_out / 256) : 1e9;
 }
 
-bool f8_small_tc_wanted(const F8ConvGeom &g) {
+bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8) {
     if (!f8_small_tc_supported(g)) return false;
-    return !f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c) || small_us(g) < tcgen05_us(g);
+    return small_us(g) < (f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c) ? tcgen05_us(g, bits8) : cuda_core_us(g));
+}
+
+// A call of its own, inputs below 16 KiB: the start of a launch is not hidden behind a neighbour, which costs this kernel about 1 us
+// less than the other (16 x 16 x 16, 3 x 3: 6.3 against 7.3 us) instead of 3.
+bool f8_small_tc_wanted_alone(const F8ConvGeom &g, bool bits8) {
+    const size_t x_bytes = (size_t)g.n * g.h * g.w * g.c;
+    return x_bytes < 16384 && f8_tc_supported(g, x_bytes) && f8_small_tc_supported(g) && small_us(g) + 1.0 < tcgen05_us(g, bits8);
 }
 
 cudaError_t f8_launch_small_tc(const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,

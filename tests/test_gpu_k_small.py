@@ -5,7 +5,7 @@ import pytest
 import torch
 
 from paper_2202_05239_b200 import synth
-from gpu_util import Guarded, api, assert_equal_arrays, random_conv_layer, random_input
+from gpu_util import Guarded, api, assert_equal_arrays, check_layer, random_conv_layer, random_input
 
 pytestmark = pytest.mark.gpu
 
@@ -66,4 +66,40 @@ def test_the_last_plan_is_not_that_of_an_earlier_call(ref):
     net.forward(xs)
     assert not any(a.f8_debug_last_plan().values())
     torch.cuda.synchronize()
+    net.close()
+
+
+# What a layer runs on by default: (h, w, c, c_out, k, stride, n, y_dtype, kernel in a network, kernel of a single-layer call)
+ROUTES = [
+    (16, 16, 16, 16, 3, 1, 1, synth.U8, "small", "small"),
+    (14, 14, 256, 256, 3, 1, 1, synth.U8, "small", "tcgen05"),
+    (31, 31, 16, 4096, 3, 1, 1, synth.U8, "tcgen05", "tcgen05"),      # more tiles than the machine holds at once
+    (5, 5, 320, 32, 5, 2, 2, synth.U8, "tcgen05", "tcgen05"),         # two narrow tiles, 8000 products per output
+    (17, 17, 768, 52, 3, 1, 7, synth.S32, "tcgen05", "tcgen05"),
+    (20, 20, 1344, 184, 3, 1, 1, synth.S8, "tcgen05", "tcgen05"),
+    (1, 1, 384, 128, 7, 1, 1, synth.U8, "cuda cores", "cuda cores"),  # one tap of 49 inside the image
+    (1, 1, 2048, 1000, 1, 1, 1, synth.S32, "small", "cuda cores"),
+]
+
+
+@pytest.mark.parametrize("case", range(len(ROUTES)))
+def test_which_kernel_a_layer_takes(ref, case):
+    h, w, c, c_out, k, stride, n, y_dtype, in_net, alone = ROUTES[case]
+    rng = np.random.default_rng(2400 + case)
+    layer = random_conv_layer(rng, h=h, w=w, c=c, c_out=c_out, k=k, stride=stride, pad=k // 2, x_signed=False, y_dtype=y_dtype, with_res=False)
+    a = api()
+
+    def taken(before):
+        tc = a.f8_tc_launch_count() - before
+        return "tcgen05" if a.f8_debug_last_plan()["m_tiles"] else ("small" if tc else "cuda cores")
+    x = random_input(rng, n, layer)
+    before = a.f8_tc_launch_count()
+    check_layer(ref, layer, x)
+    assert taken(before) == alone
+    net = a.Net([layer], n)
+    before = a.f8_tc_launch_count()
+    out = net.forward(a.to_device(x))
+    assert taken(before) == in_net
+    torch.cuda.synchronize()
+    assert_equal_arrays(out.cpu().numpy().reshape(n, layer.ho, layer.wo, c_out), ref.run_layer(layer, x))
     net.close()
