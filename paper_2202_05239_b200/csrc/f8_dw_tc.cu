@@ -457,7 +457,22 @@ bool f8_dw_tc_supported(const F8ConvGeom &g, const F8Requant &q) {
 // Setting up the diagonal blocks and filling the pipeline takes about 2 us more than the CUDA-core kernels need to start; per output
 // this kernel is the faster one.  Whole networks with the line at 0.8, 1.6 and 3.5 million outputs, pairs not fused: MobileNet V1 at
 // batch 16 170.8, 169.5, 182.9 us, MobileNet V2 at batch 16 313.1, 300.5, 300.9 us, at batch 64 487.8, 487.6, 500.0 us.
-bool f8_dw_tc_wanted(const F8ConvGeom &g) { return (double)g.n * g.ho * g.wo * g.c >= 1.6e6; }
+// That is with rows that fill the 128 positions of a tile.  A tile row costs the same however many of them hold an output, and the
+// CUDA cores take about 0.55 (stride 2: 1.1) us per million outputs: 64 x 64 x 1200 at batch 64 (one image of 66 positions per
+// block) 239.6 us here, 183.2 there; 78 x 78 x 48 at batch 221 52.8 and 41.2; stride 2, 98 x 98 x 1232 for one image 24.0 and 9.8.
+// Both sides were timed for 400 layers of 16 - 1600 channels; the estimates are of the longest run of a CTA.
+bool f8_dw_tc_wanted(const F8ConvGeom &g) {
+    const double outputs = (double)g.n * g.ho * g.wo * g.c;
+    if (outputs < 1.6e6) return false;
+    DwParams p;
+    dw_layout(g, &p);
+    const long long rows = (long long)p.groups * g.ho, per_slab = std::min<long long>(std::max(1, 148 / p.slabs), rows);
+    const double run = (double)((rows + per_slab - 1) / per_slab), filled = (double)(p.pitch * p.images) / DW_M;
+    // (slabs of 32 channels whose pixels do not start at whole 32-byte sectors move more of them)
+    const bool split = p.slab_w == 32 && g.c % 32 != 0;
+    if (g.stride_h == 1) return 0.83 * (split ? 1.2 : 1.0) * run < 4.0 + 0.52e-6 * outputs;
+    return (0.55 + 1.45 * filled) * (split ? 1.3 : 1.0) * run < 4.0 + 1.1e-6 * outputs;
+}
 
 cudaError_t f8_dw_tc_plan_init(F8DwPlan *plan, const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias, void *y,
                                int *status_word, const char **why) {

@@ -44,3 +44,27 @@ def test_depthwise(ref, request, case):
     assert a.f8_tc_launch_count() == before + 1 and out.intact()
     assert_equal_arrays(out.t.cpu().numpy().reshape(want.shape), want, "output: ")
     net.close()
+
+
+@pytest.mark.parametrize("h,c,stride,n,tensor_cores", [
+    (56, 144, 1, 33, True),         # two images of 58 positions in a tile row
+    (64, 144, 1, 33, False),        # one image of 66: half of every tile row is empty
+    (78, 48, 1, 80, False),
+    (98, 1232, 2, 1, False),        # one image in four blocks
+    (112, 96, 2, 16, True),
+    (7, 960, 1, 16, False),         # too few outputs to pay for the start
+])
+def test_which_kernel_a_depthwise_layer_takes(ref, h, c, stride, n, tensor_cores):
+    rng = np.random.default_rng(h + c)
+    a = api()
+    layer = random_conv_layer(rng, h=h, w=h, c=c, c_out=c, k=3, stride=stride, pad=1, x_signed=False, y_dtype=synth.U8, with_res=False,
+                              kind=synth.DWCONV, fl_w=6)
+    x = random_input(rng, n, layer)
+    net = a.Net([layer], n)
+    before = a.f8_tc_launch_count()
+    out = net.forward(a.to_device(x))
+    torch.cuda.synchronize()
+    a.f8_device_status()
+    assert a.f8_tc_launch_count() - before == (1 if tensor_cores else 0)
+    assert_equal_arrays(out.cpu().numpy().reshape(n, layer.ho, layer.wo, c), ref.run_layer(layer, x))
+    net.close()
