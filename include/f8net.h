@@ -299,9 +299,10 @@ f8_status f8_requantize_dual_fixed(long long n, const int32_t *acc, int fa, void
  * w [c_out, k] fp32 (k = kh * kw * c_in in the layout the convolution will use, e.g. OHWI), gamma / sigma /
  * beta / mu [c_out] fp32, w_q [c_out, k] int8, bias_q [c_out] int32, fl_w one int -- all DEVICE pointers; the
  * chosen fractional length is written to *fl_w on the device (read it back after the stream has finished).
+ * bias_q may be the memory of one of gamma, sigma, beta and mu; the outputs share no other memory with the inputs.
  * workspace: at least f8_fold_workspace_bytes() bytes of device memory, 8-byte aligned; its contents need not be
- * initialised and are overwritten.  Two kernels are enqueued on the stream; nothing is synchronised.
- * Errors: F8_ERR_NULL, F8_ERR_SHAPE (extents, non-positive eta), F8_ERR_FL_RANGE, F8_ERR_WORKSPACE,
+ * initialised and are overwritten.  Two kernels are enqueued on the stream (three when bias_q is the memory of gamma or sigma);
+ * nothing is synchronised.  Errors: F8_ERR_NULL, F8_ERR_SHAPE (extents, non-positive eta), F8_ERR_FL_RANGE, F8_ERR_WORKSPACE,
  * F8_ERR_ALIGN; nothing is launched when validation fails. */
 typedef struct {
     int c_out, k;

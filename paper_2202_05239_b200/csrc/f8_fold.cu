@@ -45,6 +45,7 @@ struct FoldParams {
     int32_t *b_q;
     int *fl_w;
     double *partial;                      // [blocks][2]
+    bool bias_last;                       // the biases overwrite gamma or sigma: in a launch behind the last use of the row scales
 };
 
 __device__ __forceinline__ double row_scale(const FoldParams &p, int row) {
@@ -137,6 +138,18 @@ __global__ void __launch_bounds__(FOLD_THREADS) fold_stats_kernel(const FoldPara
     }
 }
 
+// Biases, one thread each.
+__device__ __forceinline__ void write_biases(const FoldParams &p, int fl) {
+    const int fa = p.fl_x + fl;
+    for (int i = (int)(blockIdx.x * FOLD_THREADS + threadIdx.x); i < p.c_out; i += (int)gridDim.x * FOLD_THREADS) {
+        const double gs = __ddiv_rn((double)__ldg(p.gamma + i), (double)__ldg(p.sigma + i));
+        const double be = __ddiv_rn(__dsub_rn((double)__ldg(p.beta + i), __dmul_rn(gs, (double)__ldg(p.mu + i))), p.eta_out);
+        double t = floor(__dadd_rn(scalbn(be, fa), 0.5));
+        t = fmin(fmax(t, -2147483648.0), 2147483647.0);
+        p.b_q[i] = (int32_t)t;
+    }
+}
+
 template <bool VEC>
 __global__ void __launch_bounds__(FOLD_THREADS) fold_quant_kernel(const FoldParams p) {
     __shared__ double sc[FOLD_MAX_ROWS];
@@ -172,14 +185,7 @@ __global__ void __launch_bounds__(FOLD_THREADS) fold_quant_kernel(const FoldPara
     __syncthreads();
     const int fl = fl_s;
     const double pow2 = scalbn(1.0, fl);          // multiplying by a power of two is exact
-    const int fa = p.fl_x + fl;
-    for (int i = (int)(blockIdx.x * FOLD_THREADS + threadIdx.x); i < p.c_out; i += (int)gridDim.x * FOLD_THREADS) {
-        const double gs = __ddiv_rn((double)__ldg(p.gamma + i), (double)__ldg(p.sigma + i));
-        const double be = __ddiv_rn(__dsub_rn((double)__ldg(p.beta + i), __dmul_rn(gs, (double)__ldg(p.mu + i))), p.eta_out);
-        double t = floor(__dadd_rn(scalbn(be, fa), 0.5));
-        t = fmin(fmax(t, -2147483648.0), 2147483647.0);
-        p.b_q[i] = (int32_t)t;
-    }
+    if (!p.bias_last) write_biases(p, fl);
     while (true) {
         double scale = 0.0;
         uint32_t packed = 0;
@@ -207,6 +213,8 @@ __global__ void __launch_bounds__(FOLD_THREADS) fold_quant_kernel(const FoldPara
     }
 }
 
+__global__ void __launch_bounds__(FOLD_THREADS) fold_bias_kernel(const FoldParams p) { write_biases(p, *p.fl_w); }
+
 template <bool VEC>
 cudaError_t launch_fold(const FoldParams &p, cudaStream_t st) {
     fold_stats_kernel<VEC><<<p.blocks, FOLD_THREADS, 0, st>>>(p);
@@ -219,7 +227,9 @@ cudaError_t launch_fold(const FoldParams &p, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fold_quant_kernel<VEC>, p);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fold_quant_kernel<VEC>, p);
+    if (e == cudaSuccess && p.bias_last) fold_bias_kernel<<<(p.c_out + FOLD_THREADS - 1) / FOLD_THREADS, FOLD_THREADS, 0, st>>>(p);
+    return e;
 }
 
 }   // namespace
@@ -252,6 +262,9 @@ f8_status f8_fold_quantize_fixed(const f8_fold_desc *d, const float *w, const fl
     const bool vec4 = d->k % 4 == 0 && ((uintptr_t)w & 15) == 0 && ((uintptr_t)w_q & 3) == 0;
     p.w = w; p.gamma = gamma; p.sigma = sigma; p.beta = beta; p.mu = mu;
     p.w_q = w_q; p.b_q = bias_q; p.fl_w = fl_w; p.partial = (double *)workspace;
+    const size_t row_bytes = (size_t)d->c_out * 4;
+    auto meets = [&](const float *v) { return (uintptr_t)v < (uintptr_t)bias_q + row_bytes && (uintptr_t)bias_q < (uintptr_t)v + row_bytes; };
+    p.bias_last = meets(gamma) || meets(sigma);
     cudaError_t e = vec4 ? launch_fold<true>(p, (cudaStream_t)cuda_stream) : launch_fold<false>(p, (cudaStream_t)cuda_stream);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return f8_set_error(F8_ERR_CUDA, cudaGetErrorString(e));

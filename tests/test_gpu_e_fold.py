@@ -62,6 +62,29 @@ def test_fold_quantize(case):
     assert int((got_b != want_b).sum()) == 0
 
 
+@pytest.mark.parametrize("which", [1, 2, 3, 4])
+def test_biases_in_the_place_of_a_parameter(which):
+    """bias_q may be the memory of gamma, sigma, beta or mu: every parameter has been used before it is overwritten.  The tensor is
+    large enough that blocks compute row scales after others have written biases."""
+    a = api()
+    c_out, k = 2048, 4608
+    rng = np.random.default_rng(77)
+    w = rng.normal(0, 0.05, (c_out, k)).astype(np.float32)
+    params = [rng.uniform(0.5, 2.0, c_out).astype(np.float32) for _ in range(4)]
+    eta_in, eta_out = f8fold.eta_fix(5, 4.0), f8fold.eta_fix(4, 6.0)
+    want_w, want_b, want_fl, _ = f8fold.fold_quantize(w, *params, eta_in, eta_out, 5, 0, 24)
+    dev = [a.to_device(t) for t in [w] + params]
+    b_q = dev[which].view(torch.int32)
+    d = a.FoldDesc(c_out, k, 5, 0, 24, eta_in, eta_out)
+    w_q = torch.empty((c_out, k), dtype=torch.int8, device="cuda")
+    fl = torch.zeros(1, dtype=torch.int32, device="cuda")
+    a.f8_fold_quantize_fixed(d, *dev, w_q, b_q, fl, torch.empty(a.f8_fold_workspace_bytes(d), dtype=torch.uint8, device="cuda"))
+    torch.cuda.synchronize()
+    assert int(fl.item()) == want_fl
+    assert int((b_q.cpu().numpy() != want_b).sum()) == 0
+    assert int((w_q.cpu().numpy() != want_w).sum()) == 0
+
+
 def test_fold_constant_and_identity_cases():
     # identity BatchNorm, equal scaling factors: the plain signed quantiser with the format of Eq. 1
     rng = np.random.default_rng(99)
