@@ -277,22 +277,23 @@ bool f8_small_tc_supported(const F8ConvGeom &g) {
 // of the layers of ResNet-18 / 50 and MobileNet V2 at batches 1 - 64 and of 480 layers with up to 2048 channels and filters up to 7 x 7
 // (B200).  Examples, this kernel against the other: 196 x 256 x 2304 (pixels x channels x K) 10.2 / 16.3, 784 x 512 x 128 8.2 / 12.3,
 // 1 x 1000 x 2048 10.4 / 77.8 (not on tensor cores before), 784 x 512 x 4608 22.5 / 22.6, 3136 x 512 x 128 14.3 / 12.1,
-// 12544 x 384 x 64 22.5 / 12.2; alone, 1250 x 184 x 12096 40.4 / 22.7, 2240 x 48 x 25088 72.1 / 41.4, 250 x 16 x 25600 45.6 / 28.0.
+// 12544 x 384 x 64 22.5 / 12.2; alone, 1 x 1000 x 4096 10.5 / 13.2, 1 x 1000 x 12288 24.8 / 25.4, 1250 x 184 x 12096 40.4 / 22.7, 2240 x 48 x 25088 72.1 / 41.4, 250 x 16 x 25600 45.6 / 28.0.
 // What decides beyond small sizes: a narrow tcgen05 tile costs half as much per K chunk as a 256-wide one, and this kernel's tiles
 // share the way from the L2 cache, twice as slow per chunk with one tile on every SM as with a few.
 static double small_us(const F8ConvGeom &g) {
     const double m = (double)g.n * g.ho * g.wo, n = g.c_out, k = (double)g.kh * g.kw * g.c;
-    const double big = std::ceil(m / 64) * std::ceil(n / 64) / 148;
+    const double big = std::ceil(m / 64) * std::ceil(n / 64) / 148, full = std::ceil(m / 32) * std::ceil(n / 32) / 148;
+    // (one row of tiles reads every weight once, and hardly any activations)
+    if (m <= 32) return std::max(7.3, 5.5 + 0.0016 * k) + std::max(0.0, full - 1) * (0.6 + 0.0006 * k);
     // (64 x 64 tiles: from five chunks on the ring fills an SM, and a started round costs a whole one)
     if (big >= 1) return 7.3 + (k > 5 * SM_KB ? std::ceil(big) : big) * (1.7 + 0.0042 * k);
-    const double full = std::ceil(m / 32) * std::ceil(n / 32) / 148;
     return 7.3 + (full < 1 ? 0.0014 * (1 + full) : std::max(0.0028, 0.0012 * full)) * k;
 }
 static double tcgen05_us(const F8ConvGeom &g, bool bits8) {
     const F8TcTiles t = f8_tc_tiles(g, bits8);
     const double wide = 0.0024 * ((double)g.kh * g.kw * g.c);
     // per chunk; 256-wide tiles with a very long K wait for memory on top
-    const double narrow = t.bn <= 32 ? (t.row_tiles ? 0.10 : 0.14) : (t.bn <= 64 ? (t.row_tiles ? 0.13 : (bits8 ? 0.17 : 0.22)) : 0.25);
+    const double narrow = t.bn <= 32 ? (t.row_tiles ? 0.10 : (g.kh * g.kw == 1 ? 0.18 : 0.14)) : (t.bn <= 64 ? (t.row_tiles ? 0.13 : (bits8 ? 0.17 : 0.22)) : 0.25);
     const double tile = t.bn > 128 ? wide + 0.1 * std::max(0, t.chunks - 64) : std::min(wide, narrow * t.chunks);
     // (32-bit or two outputs of small tensors leave by direct stores)
     return (!bits8 && t.row_tiles ? 11.8 : 10.3) + std::ceil((double)t.tiles / 148) * tile;
@@ -307,11 +308,18 @@ bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8) {
     return small_us(g) < (f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c) ? tcgen05_us(g, bits8) : cuda_core_us(g));
 }
 
-// A call of its own, inputs below 16 KiB: the start of a launch is not hidden behind a neighbour, which costs this kernel about 1 us
-// less than the other (16 x 16 x 16, 3 x 3: 6.3 against 7.3 us) instead of 3.
+// A call of its own, inputs below 16 KiB.  Nothing hides the start of either kernel, this one's takes about 1.7 us less (16 x 16 x 16,
+// 3 x 3: 6.3 against 7.3 us with the tensor maps on the host), a tcgen05 chunk takes 0.12 us whatever its width in bytes (0.5 with
+// 256-wide tiles, of which there are few), and its direct stores 6 us per MB of 32-bit, 18 per MB of 8-bit values.  Fitted to 450 layers;
+// 31 x 31 x 16, 3 x 3 to 4096 channels 28.9 us here, 15.7 there; 13 x 13 x 48 of two images to 1784 9.3 and 22.9.
 bool f8_small_tc_wanted_alone(const F8ConvGeom &g, bool bits8) {
     const size_t x_bytes = (size_t)g.n * g.h * g.w * g.c;
-    return x_bytes < 16384 && f8_tc_supported(g, x_bytes) && f8_small_tc_supported(g) && small_us(g) + 1.0 < tcgen05_us(g, bits8);
+    if (x_bytes >= 16384 || !f8_tc_supported(g, x_bytes) || !f8_small_tc_supported(g)) return false;
+    const F8TcTiles t = f8_tc_tiles(g, bits8);
+    const bool pointwise = g.kh * g.kw == 1, direct = g.c_out % 16 != 0 || (!bits8 && (!pointwise || g.c_out > 27000));
+    const double chunk = t.bn <= 16 ? 0.14 : (t.bn <= 32 ? (pointwise ? 0.18 : 0.12) : (t.bn <= 64 ? 0.13 : (t.bn <= 128 ? 0.25 : 0.5)));
+    const double stores = direct ? (bits8 ? 18e-6 : 24e-6) * ((double)g.n * g.ho * g.wo * g.c_out) : 0.0;
+    return small_us(g) - 1.0 < 8.0 + std::ceil((double)t.tiles / 148) * t.chunks * chunk + stores;
 }
 
 cudaError_t f8_launch_small_tc(const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,

@@ -74,11 +74,13 @@ ROUTES = [
     (16, 16, 16, 16, 3, 1, 1, synth.U8, "small", "small"),
     (14, 14, 256, 256, 3, 1, 1, synth.U8, "small", "tcgen05"),
     (31, 31, 16, 4096, 3, 1, 1, synth.U8, "tcgen05", "tcgen05"),      # more tiles than the machine holds at once
-    (5, 5, 320, 32, 5, 2, 2, synth.U8, "tcgen05", "tcgen05"),         # two narrow tiles, 8000 products per output
+    (6, 6, 432, 96, 7, 2, 1, synth.S32, "tcgen05", "tcgen05"),        # two narrow tiles, 21168 products per output
+    (13, 13, 48, 1784, 3, 1, 2, synth.U8, "small", "small"),          # rows of 1784 bytes, which the other kernel stores directly
     (17, 17, 768, 52, 3, 1, 7, synth.S32, "tcgen05", "tcgen05"),
     (20, 20, 1344, 184, 3, 1, 1, synth.S8, "tcgen05", "tcgen05"),
     (1, 1, 384, 128, 7, 1, 1, synth.U8, "cuda cores", "cuda cores"),  # one tap of 49 inside the image
     (1, 1, 2048, 1000, 1, 1, 1, synth.S32, "small", "cuda cores"),
+    (1, 1, 4096, 1000, 1, 1, 1, synth.S32, "small", "small"),
 ]
 
 
@@ -103,3 +105,21 @@ def test_which_kernel_a_layer_takes(ref, case):
     torch.cuda.synchronize()
     assert_equal_arrays(out.cpu().numpy().reshape(n, layer.ho, layer.wo, c_out), ref.run_layer(layer, x))
     net.close()
+
+
+def test_current_stream_without_the_raw_handle(ref, monkeypatch):
+    """The binding takes the current stream's handle straight from torch where it can; the Stream object gives the same one."""
+    a = api()
+    rng = np.random.default_rng(2500)
+    layer = random_conv_layer(rng, h=12, w=12, c=32, c_out=32, k=3, stride=1, pad=1, x_signed=False, y_dtype=synth.U8, with_res=False)
+    x = random_input(rng, 2, layer)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        handle = a._stream(None)
+        assert handle == side.cuda_stream
+        monkeypatch.setattr(a, "_raw_stream", None)
+        assert a._stream(None) == handle
+        out = a.run_layer(layer, a.to_device(x))
+    assert a._stream(side) == handle
+    side.synchronize()
+    assert_equal_arrays(out.cpu().numpy(), ref.run_layer(layer, x))
