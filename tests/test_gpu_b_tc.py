@@ -66,6 +66,7 @@ SMALL_POINTWISE = [
 
 @pytest.mark.parametrize("case", range(len(SMALL_POINTWISE)))
 def test_small_pointwise_on_tensor_cores(ref, case):
+    from paper_2202_05239_b200 import api as a
     h, w, c, c_out, n, xs, y_dtype, with_res = SMALL_POINTWISE[case]
     rng = np.random.default_rng(700 + case)
     layer = random_conv_layer(rng, h=h, w=w, c=c, c_out=c_out, k=1, stride=1, pad=0, x_signed=xs, y_dtype=y_dtype,
@@ -74,6 +75,8 @@ def test_small_pointwise_on_tensor_cores(ref, case):
     assert 4096 <= x.size < 128 * 1024
     res = random_residual(rng, n, layer) if with_res else None
     check_layer(ref, layer, x, res, expect_tc=True)
+    # by default inputs below 16 KiB take the kernel for small layers; the tcgen05 plan they would have otherwise
+    check_layer(ref, layer, x, res, expect_tc=True, plan_off=a.PLAN_OFF_SMALL_KERNEL, expect_flags=a.PLAN_PLAIN_MATRIX)
 
 
 # layers that are not pointwise on tensors below 128 KiB (single-image inference): whole output rows per tile, one tiled
@@ -90,6 +93,8 @@ SMALL_ROW_TILED = [
     (9, 31, 16, 24, 3, 2, 0, 5, True, synth.S8, False),         # no padding, stride 2, c_out = 24
     (6, 100, 128, 64, 3, 1, 1, 1, False, synth.U8, False),      # one row of 100 positions per tile
     (6, 100, 64, 64, 3, 1, 1, 2, False, synth.U8, False),       # the same with 64-byte rows: row tiles
+    (16, 16, 16, 16, 3, 1, 1, 1, True, synth.U8, True),         # 4 KiB; 32-byte K chunks
+    (13, 11, 80, 48, 3, 2, 1, 1, False, synth.S32, False),      # 11 KiB, direct stores of 32-bit values
 ]
 
 
@@ -104,7 +109,8 @@ def test_small_layers_row_tiled_on_tensor_cores(ref, case):
     assert 4096 <= x.size < 128 * 1024
     res = random_residual(rng, n, layer) if with_res else None
     # the first and the last case are also eligible for the windowed mode (which reads through a tiled map as well)
-    check_layer(ref, layer, x, res, expect_tc=True, expect_flags=a.PLAN_WINDOWED if case in (0, 8) else a.PLAN_ROW_TILES)
+    check_layer(ref, layer, x, res, expect_tc=True, plan_off=a.PLAN_OFF_SMALL_KERNEL if x.size < 16384 else 0,
+                expect_flags=a.PLAN_WINDOWED if case in (0, 8) else a.PLAN_ROW_TILES)
 
 
 def test_extreme_operands_on_tensor_cores(ref):

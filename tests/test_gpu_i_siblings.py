@@ -25,6 +25,8 @@ CASES = [
     (14, 14, 24, 40, 3, 1, 2, False, U8, S8, S32, False),        # channel counts off the 16-byte rule: CUDA-core kernel
     (9, 9, 16, 16, 3, 2, 1, True, S32R, S32, S8, False),         # small tensor: CUDA-core kernel, both outputs 32-bit
     (12, 12, 32, 24, 1, 1, 40, False, U8, S32, U8, True),        # c_out = 24 on the tensor cores: ragged stores of both outputs
+    (12, 12, 64, 64, 3, 1, 1, False, U8, S32R, S32, True),       # 9 KiB: the kernel for small layers, 32-bit shortcut and second output
+    (11, 13, 48, 40, 1, 1, 2, True, S32, S8, U8, True),          # the same, 13 KiB, 40 of 64 channels, 8-bit shortcut
     # 32-bit tiles through shared memory: 128-wide tiles with a single buffer, one per SM
     (14, 14, 128, 256, 3, 1, 33, False, U8, S32R, S32, True),
     (28, 28, 64, 96, 1, 1, 4, True, S32, S8, None, True),        # 96 of 128 columns: the last slab of 32 values does not exist
