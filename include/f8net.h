@@ -108,9 +108,10 @@ typedef struct {
 /* Dense convolution (Eq. 6; residual add of Sec. 4.3; quantizer Eq. 2 / signed form).
  *   w_ohwi [c_out, kh, kw, c] int8; bias [c_out] int32 in format fl_x + fl_w or NULL (zero);
  *   residual NULL or [n, ho, wo, c_out] 8-bit (r_dtype, fl_r); y [n, ho, wo, c_out].
- * Layers with c % 16 == 0 whose input is at least 128 KiB run on the tensor cores
- * (tcgen05.mma kind::i8); every other shape takes a CUDA-core kernel with the same
- * result.  workspace: f8_conv_workspace_bytes(desc) bytes (may be 0 -> NULL allowed). */
+ * Layers with c % 16 == 0 and an input of at least 4 KiB run on the tensor cores
+ * (tcgen05.mma kind::i8, or mma.sync for layers of a few microseconds; below 128 KiB only
+ * pointwise layers and those whose output rows fit a tile); every other shape takes a CUDA-core
+ * kernel with the same result.  workspace: f8_conv_workspace_bytes(desc) bytes (may be 0 -> NULL allowed). */
 f8_status f8_conv2d_fixed(const f8_conv_desc *desc, const void *x, const int8_t *w_ohwi, const int32_t *bias,
                           const void *residual, void *y, void *workspace, size_t workspace_bytes,
                           void *cuda_stream);

@@ -22,9 +22,10 @@
 //
 // Where the pointwise layer has more output channels than an accumulator holds, its parts follow one another over the same
 // staged slabs, which then all have to be there at once (`slots` >= slabs).  Every wait is bounded (see f8_tc_ptx.cuh).
-// Bound: the tensor pipe (40 cycles x 36 per slab, bn2 / 2 per 32 bytes of K of a part).  Measured with the
-// rule of f8_dwpw_wanted, MobileNet V1 at batch 16 185 -> 169 us, at batch 4 133 -> 118 us, at batch 256 768 -> 764 us, MobileNet V2 at
-// batch 64 525 -> 508 us, at batch 8 251 -> 244 us.
+// Bound: the tensor pipe (40 cycles x 36 per slab, bn2 / 2 per 32 bytes of K of a part).  Measured with the rule of f8_dwpw_wanted
+// against two launches, the depthwise one on f8_dw_tc_kernel where a network prefers that: MobileNet V1 at batch 4 133.1 -> 121.3 us
+// (four pairs), at 8 148.7 -> 138.2, at 16 170.3 -> 168.2 (two), none from 32 on; MobileNet V2 at batch 8 250.7 -> 247.8 (one), at 32
+// 380.5 -> 376.2 (five), at 64 484.7 -> 478.9 (six); 37 x 37 x 400 to 144 channels at batch 14 19.9 -> 15.6.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
