@@ -784,6 +784,7 @@ bool f8_stem_tc_supported(const F8ConvGeom &g, const F8Requant &q, int kh2, int 
     if (g.c > 4 || g.stride_h != 2 || g.stride_w != 2) return false;
     if (g.wo > 128 || g.wo < 1 || g.c_out % 16 != 0 || g.c_out > 256) return false;
     if (q.has_res || (q.y_kind != F8_U8 && q.y_kind != F8_S8) || q.s < 1 || q.s > 24) return false;
+    if (g.pad_h >= g.kh) return false;       // output rows without an image row: no multiplication would write their sums
     if (kh2 < 1 || kh2 >= STEM_PAIR_SLOTS || slices < 1 || slices > 2) return false;       // windows of at most 64 bytes
     if (2 * (g.wo - 1) + slices * 4 > STEM_MAX_CELLS) return false;
     if ((size_t)g.n * g.h * g.w * g.c >= 0x7fffffffull || (size_t)g.n * std::max(g.ho, 1) >= 0x7fffffffull) return false;

@@ -127,3 +127,19 @@ def test_stem_rows_kernel_edges(ref, case):
     a.f8_device_status()
     assert a.f8_tc_launch_count() - before == 1 and net.last_launch_count == 1
     assert int((out.cpu().numpy().reshape(want.shape) != want).sum()) == 0
+
+
+@pytest.mark.parametrize("h,w,c_out,k,pad,with_pool", [(62, 66, 96, 3, 3, False), (50, 44, 32, 3, 5, True), (24, 20, 64, 3, 4, True), (30, 28, 128, 1, 2, False)])
+def test_padding_as_large_as_the_filter(ref, h, w, c_out, k, pad, with_pool):
+    """The first and last output rows then lie in the padding altogether: the quantised bias."""
+    rng = np.random.default_rng(h)
+    layers = _stem_net(rng, h, w, 3, c_out, k, pad, synth.U8, with_pool)
+    x = rng.integers(-128, 128, size=(9, h, w, 3)).astype(np.int8)
+    want = ref.net_forward(layers, x, keep_all=False)[-1]
+    a = api()
+    net = a.Net(layers, 9)
+    out = net.forward(a.to_device(x))
+    torch.cuda.synchronize()
+    a.f8_device_status()
+    assert int((out.cpu().numpy().reshape(want.shape) != want).sum()) == 0
+    net.close()
