@@ -997,7 +997,9 @@ f8_status f8_net_create(const f8_layer_desc *layers, int n_layers, const int8_t 
         // convolution with stride 1 over kw16 "channels" of an overlapping strided view (kh' row pairs cover
         // the kh rows; taps that fall outside the filter get zero weights), which the tensor-core path takes
         // with few, long TMA rows.  Kernel row r sits in pair j, half e with r = 2j + e + pad - 2*top.
-        if (kind == F8_LAYER_CONV && cp_in == d.c && cp_out == d.c_out && d.c <= 8 && d.stride == 2 &&
+        // (Only over the network's input: with the pool behind it such a layer writes a tensor that the plan of the workspace may have put
+        // in the place of an intermediate input.)
+        if (kind == F8_LAYER_CONV && L.d.src == 0 && cp_in == d.c && cp_out == d.c_out && d.c <= 8 && d.stride == 2 &&
             d.kw * 16 <= 256 && !L.has_sibling && !L.q.r_s32 && d.y_dtype != F8_S32_RELU) {
             L.packed = true;
             L.pack_left = d.pad;

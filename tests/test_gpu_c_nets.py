@@ -245,8 +245,8 @@ def _channel_nets(case):
     """Networks whose tensors of 24 (or 3) channels meet the caller's tensors through layers that keep the channel count."""
     rng = np.random.default_rng(5200 + case)
 
-    def conv(c, c_out, k=1, size=9, fl_x=4, kind=synth.CONV, src=0, res=None, y_dtype=synth.U8):
-        l = random_conv_layer(rng, h=size, w=size, c=c, c_out=c_out, k=k, stride=1, pad=k // 2, x_signed=False, y_dtype=y_dtype, with_res=res is not None,
+    def conv(c, c_out, k=1, size=9, fl_x=4, kind=synth.CONV, src=0, res=None, y_dtype=synth.U8, stride=1):
+        l = random_conv_layer(rng, h=size, w=size, c=c, c_out=c_out, k=k, stride=stride, pad=k // 2, x_signed=False, y_dtype=y_dtype, with_res=res is not None,
                               kind=kind, fl_x=fl_x, fl_w=6, fl_y=4, fl_r=4)
         l.src, l.res, l.r_dtype = src, -1 if res is None else res, synth.U8
         return l
@@ -268,15 +268,20 @@ def _channel_nets(case):
     if case == 6:       # ... or a chain of them, one end of which another layer reads
         d = conv(24, 24, k=3, kind=synth.DWCONV, src=1)
         return [a, d, conv(24, 24, src=2, res=1), conv(24, 24, k=3, kind=synth.DWCONV, src=3)]
-    # the network's input is the shortcut
-    return [conv(24, 16), conv(16, 24, src=1, res=0), conv(24, 16, src=2)]
+    if case == 7:       # the network's input is the shortcut
+        return [conv(24, 16), conv(16, 24, src=1, res=0), conv(24, 16, src=2)]
+    # a first layer in all but its place: stride 2 over three channels of an intermediate tensor, with a pool behind it
+    short = conv(3, 3, k=3, size=65, res=0)
+    down = conv(3, 16, k=3, size=65, src=1, stride=2)
+    p = _pool(synth.MAXPOOL, 2, down)
+    return [short, down, p, conv(16, 32, k=5, size=p.ho, src=3)]
 
 
 @pytest.mark.parametrize("direct", [False, True])
-@pytest.mark.parametrize("case", range(8))
+@pytest.mark.parametrize("case", range(9))
 def test_channels_that_are_no_multiple_of_16_at_the_ends_of_a_network(ref, request, case, direct):
     a = api()
-    layers, batch = _channel_nets(case), 5
+    layers, batch = _channel_nets(case), 200 if case == 8 else 5      # (case 8: so many that some images are read after others are done)
     x = random_input(np.random.default_rng(case), batch, layers[0])
     want = ref.net_forward(layers, x)
     a.f8_debug_force_direct(direct)
@@ -284,11 +289,13 @@ def test_channels_that_are_no_multiple_of_16_at_the_ends_of_a_network(ref, reque
     net = a.Net(layers, batch)
     guards = [Guarded(_layer_shape(l, batch), a.torch_dtype(l.y_dtype)) for l in layers]
     out, ws = Guarded((batch,) + net.out_shape, net.out_dtype), Guarded((net.workspace_bytes(batch),), torch.uint8)
-    net.forward(a.to_device(x), out=out.t, workspace=ws.t, dump=[g.t for g in guards])
-    torch.cuda.synchronize()
-    a.f8_device_status()
-    assert out.intact() and ws.intact()
-    assert_equal_arrays(out.t.cpu().numpy().reshape(want[-1].shape), want[-1], "output: ")
+    for dump in (None, [g.t for g in guards]):
+        out.t.zero_()
+        net.forward(a.to_device(x), out=out.t, workspace=ws.t, dump=dump)
+        torch.cuda.synchronize()
+        a.f8_device_status()
+        assert out.intact() and ws.intact()
+        assert_equal_arrays(out.t.cpu().numpy().reshape(want[-1].shape), want[-1], f"output, dump {dump is not None}: ")
     for i, g in enumerate(guards):
         assert g.intact()
         assert_equal_arrays(g.t.cpu().numpy().reshape(want[i + 1].shape), want[i + 1], f"layer {i}: ")
