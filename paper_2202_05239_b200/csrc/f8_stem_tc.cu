@@ -84,23 +84,33 @@ __device__ __forceinline__ uint32_t load_pixel(const uint8_t *x, uint32_t off, u
     return word;
 }
 
-// The one or two K slices of a row pair.  Executed by a whole warp, one lane issues: see mma_commit().
+// The one or two K slices of a row pair, issued by a lone thread or (WARP) by the elected lane of a whole warp, see mma_commit().
+template <bool WARP>
 __device__ __forceinline__ void stem_mma_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, const StemParams &p, uint32_t b_slice,
                                               uint32_t accumulate) {
-    if (p.slices == 2)
-        asm volatile("{\n\t" F8_ELECT ".reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\t"
-                     "setp.ne.b32 p, %7, 0;\n\tsetp.eq.b32 t, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t"
-                     "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, p;\n\t"
-                     "add.u32 x, %1, 2;\n\tadd.u32 y, %2, %5;\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %4};\n\t"
-                     "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, t;\n\t}" ::"r"(d_tmem),
-                     "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(b_slice), "r"(p.idesc), "r"(accumulate)
-                     : "memory");
-    else
-        asm volatile("{\n\t" F8_ELECT ".reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %6, 0;\n\t"
-                     "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t"
-                     "@e tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
-                     "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(p.idesc), "r"(accumulate)
-                     : "memory");
+#define STEM_TWO(elect, on) \
+    asm volatile("{\n\t" elect ".reg .pred p, t;\n\t.reg .b64 a, b;\n\t.reg .b32 x, y;\n\t" \
+                 "setp.ne.b32 p, %7, 0;\n\tsetp.eq.b32 t, 0, 0;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t" \
+                 on "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, p;\n\t" \
+                 "add.u32 x, %1, 2;\n\tadd.u32 y, %2, %5;\n\tmov.b64 a, {x, %3};\n\tmov.b64 b, {y, %4};\n\t" \
+                 on "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %6, t;\n\t}" ::"r"(d_tmem), \
+                 "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(b_slice), "r"(p.idesc), "r"(accumulate) \
+                 : "memory")
+#define STEM_ONE(elect, on) \
+    asm volatile("{\n\t" elect ".reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.ne.b32 p, %6, 0;\n\t" \
+                 "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %4};\n\t" \
+                 on "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem), \
+                 "r"(a_lo), "r"(b_lo), "r"(p.a_desc_hi), "r"(p.b_desc_hi), "r"(p.idesc), "r"(accumulate) \
+                 : "memory")
+    if (p.slices == 2) {
+        if (WARP) STEM_TWO(F8_ELECT, "@e ");
+        else STEM_TWO("", "");
+    } else {
+        if (WARP) STEM_ONE(F8_ELECT, "@e ");
+        else STEM_ONE("", "");
+    }
+#undef STEM_TWO
+#undef STEM_ONE
 }
 
 template <bool POOL, bool SIGNED, bool FAST>
@@ -195,7 +205,8 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
         for (int i = 0; i < 2; ++i)
             if (cell_on[i]) line[threadIdx.x + i * STEM_THREADS] = cell[i];
     };
-    // issue the MMAs of output row oy into accumulator kk & 1 (a whole warp)
+    // issue the MMAs of output row oy into accumulator kk & 1 (one thread: between this kernel's block barriers a whole warp that elects a
+    // lane is slower, 4 -> 128 channels, 128 x 128, batch 128 55.8 against 54.5 us, 250 x 250 3 -> 96, batch 8 15.0 against 14.0)
     const uint32_t a_lo0 = p.a_desc_lbo_sbo | ((pair_base & 0x3ffffu) >> 4), b_lo0 = p.b_desc_lbo_sbo | ((smem_base & 0x3ffffu) >> 4);
     const uint32_t b_slice = 2u * c_out;                 // 16-byte units between the K slices of the weights
     auto issue_row = [&](int oy, int kk) {
@@ -206,10 +217,10 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
             const int pr = oy - p.top + j;
             if (pr < 0 || pr >= p.hp) continue;          // rows above / below the image contribute nothing
             const uint32_t a_lo = a_lo0 + (uint32_t)(pr & (STEM_PAIR_SLOTS - 1)) * (STEM_SLOT_BYTES / 16);
-            stem_mma_pair(d_tmem, a_lo, b_lo, p, b_slice, accumulate);
+            stem_mma_pair<false>(d_tmem, a_lo, b_lo, p, b_slice, accumulate);
             accumulate = 1;
         }
-        mma_commit(smem_u32(&acc_bar[kk & 1]));
+        mma_commit_thread(smem_u32(&acc_bar[kk & 1]));
     };
 
     for (int u = u_begin; u < u_end;) {
@@ -234,8 +245,11 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
         if (warp == STEM_EPI_WARPS) {
-            tc_fence_after();
-            issue_row(oy_first, k);
+            if (lane == 0) {
+                tc_fence_after();
+                issue_row(oy_first, k);
+            }
+            __syncwarp();
         }
 
         for (int oy = oy_first; oy <= oy_last; ++oy, ++k) {
@@ -257,10 +271,11 @@ __global__ void __launch_bounds__(STEM_THREADS, 3) f8_stem_tc_kernel(const StemP
             const bool opens = oy == 0;
             const int py = oy >> 1;
             if (warp == STEM_EPI_WARPS) {
-                if (oy + 1 <= oy_last) {
+                if (lane == 0 && oy + 1 <= oy_last) {
                     tc_fence_after();
                     issue_row(oy + 1, k + 1);
                 }
+                __syncwarp();
             } else {
                 // ---- epilogue of row oy: thread = output pixel, 16 channels per accumulator load
                 // the accumulator is usually a few hundred cycles away: sleep on the barrier (the hardware wakes the
@@ -623,7 +638,7 @@ __global__ void __launch_bounds__(ROWS_THREADS, 2) f8_stem_rows_tc_kernel(const 
                         const int pr = 2 * r - p.top + j;
                         if (pr < 0 || pr >= p.hp) continue;          // rows above / below the image contribute nothing
                         const uint32_t a_lo = a_lo0 + (uint32_t)((line_of_pr + pr) & (ROWS_LINES - 1)) * (STEM_SLOT_BYTES / 16);
-                        stem_mma_pair(d_tmem, a_lo, b_lo, p, b_slice, accumulate);
+                        stem_mma_pair<true>(d_tmem, a_lo, b_lo, p, b_slice, accumulate);
                         accumulate = 1;
                     }
                     mma_commit(done_bar + 8 * (k % ROWS_AHEAD));
@@ -878,9 +893,11 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
     occ = std::min(occ, 512 / (accs * p.acc_cols));
     occ = std::max(1, std::min(occ, 4));
     const long long units = (long long)g.n * p.rows_per_img;
-    // bands of at least four units (with a pool every band computes one row above it again); when that leaves SMs idle, as many
-    // bands as there are units up to one per SM
-    long long grid = std::min<long long>((long long)sms * occ, std::max<long long>(units / 4, std::min<long long>(units, sms)));
+    // bands of at least four units (with a pool every band computes one row above it again); up to 64 channels, when that leaves SMs
+    // idle, as many bands as there are units up to one per SM (wider layers lose by it: 32 x 32, 3 -> 96 with the pool, batch 64 18.1
+    // against 17.3 us)
+    const long long bands = std::max<long long>(units / 4, rows ? std::min<long long>(units, sms) : 1);
+    const long long grid = std::min<long long>((long long)sms * occ, bands);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads);
