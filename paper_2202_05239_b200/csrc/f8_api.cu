@@ -160,6 +160,11 @@ DwPlanPtr alloc_dw_plan() {
     return DwPlanPtr((F8DwPlan *)p);
 }
 
+struct SmallPlanDeleter { void operator()(F8SmallPlan *p) const { free(p); } };
+using SmallPlanPtr = std::unique_ptr<F8SmallPlan, SmallPlanDeleter>;
+
+SmallPlanPtr alloc_small_plan() { return SmallPlanPtr((F8SmallPlan *)malloc(f8_small_plan_size())); }
+
 // The second consumer of a layer's sum: its quantizer relative to the format F of the aligned sum.
 f8_status make_sibling(const f8_conv_desc *d, const F8Requant &q, int y2_dtype, int fl_y2, void *y2, F8Sibling *sib) {
     if (y2_dtype != F8_U8 && y2_dtype != F8_S8 && y2_dtype != F8_S32 && y2_dtype != F8_S32_RELU)
@@ -191,11 +196,13 @@ f8_status run_dense(const F8ConvGeom &g, const F8Requant &q, const void *x, cons
     // Inputs of a few tiles: the kernel for small layers, which needs no tensor maps (encoding four of them takes the host longer
     // than the layer takes the GPU).  16 x 16 x 16, 3 x 3: 6.8 -> 5.1 us on the host.  Not with thousands of output channels or
     // products per output (31 x 31 x 16, 3 x 3 to 4096 channels 28.9 us, on the tcgen05 kernel 15.7).
-    if (!g_force_direct && !(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) && f8_small_tc_wanted_alone(g, is_bits8(q, sib))) {
-        const cudaError_t e = f8_launch_small_tc(g, q, x, w, bias, res, y, st, false, sib);
-        if (e != cudaSuccess) return cuda_fail(e, "small conv launch");
-        ++g_tc_launches;
-        return F8_OK;
+    if (!g_force_direct && !(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL)) {
+        const cudaError_t e = f8_launch_small_alone(g, q, is_bits8(q, sib), x, w, bias, res, y, st, sib);
+        if (e == cudaSuccess) {
+            ++g_tc_launches;
+            return F8_OK;
+        }
+        if (e != cudaErrorNotSupported) return cuda_fail(e, "small conv launch");
     }
     if (!g_force_direct && f8_tc_supported(g, x_bytes)) {
         PlanPtr plan = alloc_plan();
@@ -525,7 +532,7 @@ struct Step {
     const void *res = nullptr;
     void *y = nullptr;
     bool use_tc = false;
-    bool small = false;       // use_tc: the kernel for layers of a few microseconds (no plan)
+    SmallPlanPtr splan;       // use_tc: the kernel for layers of a few microseconds
     bool fused_pool = false;  // kind -2: the stem kernel also computes the max pool that follows (layer + 1)
     bool has_sib = false;     // the launch also writes the output of the sibling layer behind it (layer + 1)
     F8Sibling sib;
@@ -1305,12 +1312,19 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                                return true;
                            }()) {
                     // planned above
-                } else if (!(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) && f8_small_tc_wanted(stp.g, is_bits8(L.q, stp.has_sib ? &stp.sib : nullptr))) {
-                    stp.use_tc = stp.small = true;
+                } else if ([&]() -> bool {
+                               const F8Sibling *sib = stp.has_sib ? &stp.sib : nullptr;
+                               if ((g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) || !f8_small_tc_wanted(stp.g, is_bits8(L.q, sib))) return false;
+                               SmallPlanPtr sp = alloc_small_plan();
+                               if (!sp || f8_small_plan_init(sp.get(), stp.g, L.q, stp.x, L.w, L.b, stp.res, stp.y, sib, i + 1) != cudaSuccess) return false;
+                               stp.splan = std::move(sp);
+                               return true;
+                           }()) {
+                    stp.use_tc = true;
                 } else if (f8_tc_supported(stp.g, (size_t)n * L.g.h * L.g.w * L.g.c)) {
                     PlanPtr plan = alloc_plan();
                     if (plan && f8_tc_plan_init(plan.get(), stp.g, L.q, dense_view(stp.x, stp.g), L.w, L.b, stp.res,
-                                                stp.y, f8_status_word(), &why, stp.has_sib ? &stp.sib : nullptr) == cudaSuccess) {
+                                                stp.y, f8_status_word(), &why, stp.has_sib ? &stp.sib : nullptr, true) == cudaSuccess) {
                         stp.use_tc = true;
                         f8_tc_plan_set_tag(plan.get(), i + 1);
                         stp.plan = std::move(plan);
@@ -1437,8 +1451,8 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
             case F8_LAYER_LINEAR:
                 // the net owns its weights (uploaded at creation), so a layer's prologue and weight loads may
                 // overlap the tail of the previous layer
-                if (stp.small) {
-                    e = f8_launch_small_tc(stp.g, L.q, stp.x, L.w, L.b, stp.res, stp.y, st, net->overlap_layers, stp.has_sib ? &stp.sib : nullptr);
+                if (stp.splan) {
+                    e = f8_small_launch(stp.splan.get(), net->overlap_layers, st);
                     ++g_tc_launches;
                 } else if (stp.use_tc) { e = f8_tc_launch(stp.plan.get(), net->overlap_layers, st); ++g_tc_launches; }
                 else e = f8_launch_conv_direct(stp.g, L.q, stp.x, L.w, L.b, stp.res, stp.y, st, net->overlap_layers,

@@ -1132,6 +1132,23 @@ int choose_bn_staged(int c_out, bool has_res, int kb) {
     return bn;
 }
 
+int sm_count_here() {
+    int sm_count = 148, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
+    return sm_count;
+}
+
+// Layers whose tiles leave SMs idle: half as many columns per tile as long as every SM still has one tile at most.  A 128-byte chunk of K
+// takes 0.30 us with 256 columns, 0.17 us with 64 (3 x 3 256 -> 256 at 14 x 14 of four images 9.2 -> 6.0 us a layer, 512 -> 512 at
+// 7 x 7 of sixteen 14.2 -> 9.3); 32 columns gave nothing more.
+// Not 128 to 64 where a filter larger than 1 x 1 has a single tile of columns: its resident weights and whole-row windows are worth
+// more (3 x 3 128 -> 128 at 28 x 28 of eight images 4.4 us a layer, with 64-wide tiles 5.2).
+int narrow_bn(int bn, long long m_tiles, const F8ConvGeom &g, int sms) {
+    while (bn > 64 && m_tiles * ((g.c_out + bn / 2 - 1) / (bn / 2)) <= sms && !(bn >= g.c_out && bn <= 128 && g.kh * g.kw > 1)) bn /= 2;
+    return bn;
+}
+
 CUtensorMapSwizzle swizzle_for(int kb) {
     return kb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (kb == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
 }
@@ -1183,7 +1200,7 @@ F8TcTiles f8_tc_tiles(const F8ConvGeom &g, bool bits8) {
     const int rows = t.row_tiles ? std::min(TILE_M / g.wo, g.ho) : 1;
     const long long m_tiles = t.row_tiles ? (long long)g.n * ((g.ho + rows - 1) / rows) : ((long long)g.n * g.ho * g.wo + TILE_M - 1) / TILE_M;
     if (bits8 && g.c_out % 16 == 0) {
-        t.bn = choose_bn_staged(g.c_out, false, t.kb);
+        t.bn = narrow_bn(choose_bn_staged(g.c_out, false, t.kb), m_tiles, g, 148);
     } else if (g.c_out % 16 == 0 && (big || pointwise)) {
         t.bn = g.c_out > 32 ? 64 : 32;
     } else {
@@ -1196,7 +1213,7 @@ F8TcTiles f8_tc_tiles(const F8ConvGeom &g, bool bits8) {
 
 cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant &q, const F8TcTensorView &xv,
                             const int8_t *w, const int32_t *bias, const void *res, void *y, int *status_word,
-                            const char **why, const F8Sibling *sib) {
+                            const char **why, const F8Sibling *sib, bool in_network) {
     *why = "";
     if (!load_driver_entry_points()) {
         *why = "cuTensorMapEncode entry points not available";
@@ -1258,6 +1275,16 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
     const bool staged = p.epi != EPI_GENERIC;
     p.bn = wide ? (g.c_out > 32 ? 64 : 32) : staged ? (k_heavy_res ? 256 : choose_bn_staged(g.c_out, q.has_res != 0, p.kb)) : choose_bn(g.c_out);
     p.m_tiles = (p.M + TILE_M - 1) / TILE_M;
+    // (single-layer calls keep the tiles that CTA pairs need)
+    const bool pair_shape = g.c % 128 == 0 && g.c_out % 256 == 0 && g.kh * g.kw * (g.c / 128) >= 8 && big_x && p.m_tiles >= 2;
+    if (staged && !wide && (in_network || !pair_shape)) {
+        const int bn = narrow_bn(p.bn, p.m_tiles, g, sm_count_here());
+        if (bn < p.bn) {
+            p.bn = bn;
+            p.kb = choose_kb(g.c);           // (64-byte chunks make room for the ring of 256-wide tiles)
+            p.c_chunks = (g.c + p.kb - 1) / p.kb;
+        }
+    }
     if (wide && g.c_out >= 128) {
         // 64-wide tiles leave room for three (two) buffers of the ring; where 128-wide ones give every SM one tile at most, a single
         // buffer will do and the activations are read half as often (3x3 256 -> 256 at 14 x 14, batch 33: 22.5 -> 18.5 us)

@@ -87,7 +87,7 @@ size_t f8_tc_plan_size();
 // Encodes tensor maps and tile schedule; returns cudaSuccess or an error (no launch).
 cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant &q, const F8TcTensorView &xv,
                             const int8_t *w /* [c_out][kh][kw][g.c] */, const int32_t *bias, const void *res,
-                            void *y, int *status_word, const char **why, const F8Sibling *sib = nullptr);
+                            void *y, int *status_word, const char **why, const F8Sibling *sib = nullptr, bool in_network = false);
 // Label reported (with the wait's site) when a bounded wait of this launch gives up; 0 = none.
 void f8_tc_plan_set_tag(F8TcPlan *plan, int tag);
 // overlap_previous: the grid may start before the preceding work of the stream has finished; only its weight
@@ -142,12 +142,16 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
 
 // ---- small layers (f8_small_tc.cu): implicit GEMM on mma.sync for layers bound by latency; every output kind, shortcut and
 // sibling; c a multiple of 16, c_out of 4, weights, bias, shortcut and outputs 16-byte aligned.  `wanted`: the rule by which a
-// network (`alone`: a single-layer call) prefers it to the other kernels; bits8: one 8-bit output, shortcut of 8 bits or none.
-bool f8_small_tc_supported(const F8ConvGeom &g);
+// network prefers it to the other kernels; bits8: one 8-bit output, shortcut of 8 bits or none.
 bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8);
-bool f8_small_tc_wanted_alone(const F8ConvGeom &g, bool bits8);
-cudaError_t f8_launch_small_tc(const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
-                               const void *res, void *y, cudaStream_t st, bool overlap_previous, const F8Sibling *sib = nullptr);
+struct F8SmallPlan;
+size_t f8_small_plan_size();
+cudaError_t f8_small_plan_init(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
+                               const void *res, void *y, const F8Sibling *sib, int tag);
+cudaError_t f8_small_launch(const F8SmallPlan *plan, bool overlap_previous, cudaStream_t st);
+// A single-layer call: launches where this kernel is the better one, else cudaErrorNotSupported.
+cudaError_t f8_launch_small_alone(const F8ConvGeom &g, const F8Requant &q, bool bits8, const void *x, const int8_t *w, const int32_t *bias,
+                                  const void *res, void *y, cudaStream_t st, const F8Sibling *sib = nullptr);
 
 // Device status word (0 = fine); allocated once per device on first use, together with a host-visible copy of its
 // first word that kernels write through (f8_status_host_code reads it without synchronising).

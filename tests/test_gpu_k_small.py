@@ -123,3 +123,44 @@ def test_current_stream_without_the_raw_handle(ref, monkeypatch):
     assert a._stream(side) == handle
     side.synchronize()
     assert_equal_arrays(out.cpu().numpy(), ref.run_layer(layer, x))
+
+
+# (h, w, c, c_out, k, stride, pad, n, x_signed, y_dtype, with_res): edges of the windows and of the panels
+WINDOWS = [
+    (2, 2, 1008, 32, 5, 1, 2, 1, False, synth.U8, False),       # weights of 25200 bytes a channel: several panels, the last one shorter
+    (3, 5, 16, 16, 3, 1, 1, 7, False, synth.U8, True),          # one unit per tap, windows that cross images
+    (9, 9, 48, 24, 3, 2, 1, 5, True, synth.S8, False),          # three units per tap, stride 2, columns past the last channel
+    (13, 13, 112, 36, 3, 1, 1, 2, False, synth.S32, False),     # seven units per tap; an odd number of them in all
+    (6, 11, 64, 260, 1, 2, 0, 3, False, synth.U8, False),       # skipped pixels
+    (1, 7, 32, 20, 1, 1, 0, 2, True, synth.U8, True),           # fewer pixels than rows of a tile
+    (12, 12, 32, 64, 3, 1, 0, 2, False, synth.U8, False),       # no padding: rows between two images that no filter starts at
+    (11, 11, 64, 64, 2, 2, 0, 3, False, synth.U8, False),       # ... and that no filter reaches
+    (8, 8, 128, 128, 7, 1, 3, 1, False, synth.U8, False),       # 49 taps
+]
+
+
+@pytest.mark.parametrize("case", range(len(WINDOWS)))
+def test_windows_and_panels(ref, case):
+    h, w, c, c_out, k, stride, pad, n, xs, y_dtype, with_res = WINDOWS[case]
+    rng = np.random.default_rng(2600 + case)
+    layer = random_conv_layer(rng, h=h, w=w, c=c, c_out=c_out, k=k, stride=stride, pad=pad, x_signed=xs, y_dtype=y_dtype, with_res=with_res)
+    layers = [layer]
+    if with_res:
+        short = random_conv_layer(rng, h=h, w=w, c=c, c_out=c_out, k=k, stride=stride, pad=pad, x_signed=xs, y_dtype=layer.r_dtype,
+                                  with_res=False, fl_x=layer.fl_x)
+        short.fl_y = layer.fl_r
+        layer.res = 1
+        layers = [short, layer]
+    a = api()
+    x = random_input(rng, n, layers[0])
+    want = ref.net_forward(layers, x)
+    net = a.Net(layers, n)
+    out = Guarded((n, layer.ho, layer.wo, c_out), a.torch_dtype(y_dtype))
+    before = a.f8_tc_launch_count()
+    net.forward(a.to_device(x), out=out.t)
+    torch.cuda.synchronize()
+    a.f8_device_status()
+    assert a.f8_tc_launch_count() - before == len(layers) and not a.f8_debug_last_plan()["m_tiles"], "another kernel took the layer"
+    assert out.intact()
+    assert_equal_arrays(out.t.cpu().numpy().reshape(want[-1].shape), want[-1])
+    net.close()
