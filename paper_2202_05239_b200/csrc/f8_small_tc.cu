@@ -537,7 +537,9 @@ bool pick_split(const F8ConvGeom &g, Split *best) {
                 const float fetch = at_once * px * g.c / 45, fetch_w = at_once * bn * k / 45;
                 // (a block's own instructions, about 500 a warp, where an SM runs several)
                 const float issue = 700.f * std::max(0.f, (float)tiles / 148 - 1);
-                const float cycles = 700 + issue + fetch + mul + finish + (panels - 1) * 300.f + std::max(0, panels - 2) * fetch_w / panels +
+                // (no room for the next layer's block: its start is not hidden)
+                const float alone = occ == 1 ? 600.f : 0.f;
+                const float cycles = 700 + alone + issue + fetch + mul + finish + (panels - 1) * 300.f + std::max(0, panels - 2) * fetch_w / panels +
                                      (rounds - 1) * (1500 + fetch + fetch_w + mul + finish);
                 if (cycles < best->cycles) *best = {t, 1 << wm_shift, 1 << wn_shift, wk, at16, panels, window, weights, smem, tiles, cycles};
             }
@@ -597,10 +599,9 @@ static double tcgen05_us(const F8ConvGeom &g, bool bits8) {
     // a chunk of K: 256-wide tiles at the tensor rate, narrow ones at the rate their activations come in
     const double chunk = t.bn > 128 ? 0.30 * width : (t.bn <= 32 ? 0.11 : (t.row_tiles ? 0.14 : 0.17)) * (t.bn > 64 ? width : 1.0);
     const double finish = 0.25 * std::max(1.0, t.bn / 64.0), rounds = std::ceil((double)t.tiles / 148);
-    // (c_out that 16 does not divide, 32-bit or second outputs of small tensors: direct stores)
-    const bool direct = g.c_out % 16 != 0 || (!bits8 && t.row_tiles);
-    return 2.7 + rounds * std::max(t.chunks * chunk, finish) + finish + (out * (bits8 ? 1 : 4) + (double)g.n * g.h * g.w * g.c) / 6e6 +
-           (direct ? out * (bits8 ? 18e-6 : 24e-6) : 0.0);
+    // (8-bit outputs of a c_out that 16 does not divide, 32-bit or second outputs of small tensors: direct stores)
+    const double direct = bits8 ? (g.c_out % 16 != 0 ? 18e-6 * out : 0.0) : (t.row_tiles ? 1.5 : 0.0);
+    return 2.7 + rounds * std::max(t.chunks * chunk, finish) + finish + (out * (bits8 ? 1 : 4) + (double)g.n * g.h * g.w * g.c) / 6e6 + direct;
 }
 // (only the tap inside the image counts there: one pixel, 3 x 3 x 800 to 24 channels 2.4 us)
 static double cuda_core_us(const F8ConvGeom &g) {
@@ -611,7 +612,7 @@ bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8) {
     Split s;
     if (!shape_ok(g) || !pick_split(g, &s)) return false;
     if (!f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c)) return small_us(s) < cuda_core_us(g);
-    return s.panels == 1 && small_us(s) < 0.93 * tcgen05_us(g, bits8);
+    return s.panels == 1 && small_us(s) < 0.97 * tcgen05_us(g, bits8);
 }
 
 struct F8SmallPlan {
