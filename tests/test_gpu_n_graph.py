@@ -1,0 +1,65 @@
+"""GPU parity of repeated forward passes over the same buffers, which go out as one CUDA graph from the second pass on."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2202_05239_b200 import synth
+from gpu_util import api, assert_equal_arrays
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("name,batch,image", [("resnet18", 3, 64), ("resnet50", 1, 96), ("mobilenetv2", 2, 64), ("resnet18_siblings", 2, 64)])
+def test_repeated_passes(ref, name, batch, image):
+    a = api()
+    layers = synth.make_net(name, 0, image=image)
+    hosts = [synth.draw_image(batch, s, image, image) for s in (1, 2)]
+    wants = [ref.net_forward(layers, h, keep_all=False)[-1] for h in hosts]
+    net = a.Net(layers, batch)
+    x = a.to_device(hosts[0])
+    out = torch.empty((batch,) + net.out_shape, dtype=net.out_dtype, device="cuda")
+    ws = torch.empty(net.workspace_bytes(batch), dtype=torch.uint8, device="cuda")
+    other = torch.empty_like(out)
+    side = torch.cuda.Stream()
+    counts = []
+
+    def check(which, **kw):
+        x.copy_(torch.from_numpy(hosts[which]))
+        o = kw.pop("out", out)
+        o.zero_()
+        torch.cuda.synchronize()
+        before = a.f8_tc_launch_count()
+        net.forward(x, out=o, workspace=ws, **kw)
+        torch.cuda.synchronize()
+        a.f8_device_status()
+        if "dump" not in kw:
+            counts.append((net.last_launch_count, a.f8_tc_launch_count() - before))
+        assert_equal_arrays(o.cpu().numpy(), wants[which])
+
+    for i in range(4):                       # the second and later passes are the graph's; the input changes in place
+        check(i & 1)
+    check(1, stream=side)                    # on another stream
+    check(0, out=other)                      # another output: a plan of its own, then a graph of its own
+    check(1, out=other)
+    check(0, dump=[net.layer_output(i, batch) for i in range(len(layers))])
+    check(1)
+    check(0)
+    try:                                     # kernels carry the bound of their waits: a new one means new launches
+        a.f8_debug_set_wait_limit_ms(1500.0)
+        check(1)
+        check(0)
+    finally:
+        a.f8_debug_set_wait_limit_ms(0.0)
+    assert len(set(counts)) == 1
+    # inside a caller's capture the launches become the caller's
+    g = torch.cuda.CUDAGraph()
+    check(1)
+    with torch.cuda.graph(g, stream=side):
+        net.forward(x, out=out, workspace=ws, stream=torch.cuda.current_stream())
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert_equal_arrays(out.cpu().numpy(), wants[1])
+    del g
+    check(0)
+    net.close()
