@@ -210,7 +210,8 @@ f8_status run_dense(const F8ConvGeom &g, const F8Requant &q, const void *x, cons
         const char *why = "";
         cudaError_t e = f8_tc_plan_init(plan.get(), g, q, dense_view(x, g), w, bias, res, y, f8_status_word(), &why, sib);
         if (e == cudaSuccess) {
-            e = f8_tc_launch(plan.get(), false, st);   // the caller's weights may come from earlier work in the stream
+            // only the start of the blocks overlaps earlier work in the stream, which may write the caller's weights
+            e = f8_tc_launch(plan.get(), true, st);
             if (e != cudaSuccess) return cuda_fail(e, "tensor-core conv launch");
             ++g_tc_launches;
             return F8_OK;
@@ -1295,7 +1296,7 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                         v.stride_n = (uint64_t)L.pack_wp * cb * L.pack_hp;
                         PlanPtr plan = alloc_plan();
                         if (plan && f8_tc_plan_init(plan.get(), pg, L.q, v, L.w_packed, L.b, stp.res, stp.y,
-                                                    f8_status_word(), &why) == cudaSuccess) {
+                                                    f8_status_word(), &why, nullptr, true) == cudaSuccess) {
                             Step pre;
                             pre.kind = -1;
                             pre.layer = i;

@@ -115,6 +115,8 @@ __device__ __forceinline__ void block_sum(double &s1, double &s2) {
 template <bool VEC>
 __global__ void __launch_bounds__(FOLD_THREADS) fold_stats_kernel(const FoldParams p) {
     __shared__ double sc[FOLD_MAX_ROWS];
+    // (in this order: the launch behind reads the inputs before its own wait)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     double s1 = 0.0, s2 = 0.0;
     for (long long e0 = (long long)blockIdx.x * FOLD_CHUNK; e0 < p.n; e0 += (long long)gridDim.x * FOLD_CHUNK) {
@@ -161,6 +163,7 @@ __global__ void __launch_bounds__(FOLD_THREADS) fold_quant_kernel(const FoldPara
     int row0;
     bool table = stage_scales(p, e0, sc, &row0);
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     double s1 = 0.0, s2 = 0.0;
     for (int b = threadIdx.x; b < p.blocks; b += FOLD_THREADS) {
         s1 += p.partial[2 * b];
@@ -217,7 +220,7 @@ __global__ void __launch_bounds__(FOLD_THREADS) fold_bias_kernel(const FoldParam
 
 template <bool VEC>
 cudaError_t launch_fold(const FoldParams &p, cudaStream_t st) {
-    fold_stats_kernel<VEC><<<p.blocks, FOLD_THREADS, 0, st>>>(p);
+    // both launches may start while what is before them in the stream drains
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)p.blocks);
     cfg.blockDim = dim3(FOLD_THREADS);
@@ -227,7 +230,8 @@ cudaError_t launch_fold(const FoldParams &p, cudaStream_t st) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, fold_quant_kernel<VEC>, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fold_stats_kernel<VEC>, p);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, fold_quant_kernel<VEC>, p);
     if (e == cudaSuccess && p.bias_last) fold_bias_kernel<<<(p.c_out + FOLD_THREADS - 1) / FOLD_THREADS, FOLD_THREADS, 0, st>>>(p);
     return e;
 }

@@ -82,6 +82,7 @@ struct FastDiv {
 __device__ __forceinline__ int fast_div(int n, FastDiv d) { return (int)(((uint64_t)(uint32_t)n * d.mul) >> d.shift); }
 
 struct TcParams {
+    int wait_all;                   // everything behind the barriers waits for the grids before this one (not only activations and outputs)
     int M;                    // total output pixels
     int ho, wo;
     int c_out;
@@ -404,6 +405,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     const uint32_t tmem_base = uniform(tmem_base_slot);
     // the next grid in the stream may be scheduled from here on: its CTAs take over an SM when this grid's
     // CTA there has exited, and run their prologue while the rest of this grid finishes
+    if (p.wait_all) grid_dependency_wait();      // a call of its own: the weights may come from earlier work in the stream as well
     grid_launch_dependents();
 
     // per worker: 128-row tiles, 256-row tiles of a pair, or groups of p.sup M tiles
@@ -1224,6 +1226,7 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
     }
     memset(plan, 0, sizeof(*plan));
     TcParams &p = plan->p;
+    p.wait_all = in_network ? 0 : 1;
     p.epi_groups = 4;
     p.M = g.n * g.ho * g.wo;
     p.ho = g.ho;

@@ -55,6 +55,8 @@ __device__ __forceinline__ uint4 requant16(const int (&u)[8], const int (&v)[8],
 // acc 32-byte, y1 / y2 16-byte aligned; the last thread takes the ragged tail.
 __global__ void __launch_bounds__(256) requant_dual_kernel(const int32_t *__restrict__ acc, long long n, F8Requant q1, F8Requant q2,
                                                             uint8_t *__restrict__ y1, uint8_t *__restrict__ y2) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const long long i = ((long long)blockIdx.x * 256 + threadIdx.x) * 16;
     if (i + 16 <= n) {
         int u[8], v[8];
@@ -76,6 +78,8 @@ __global__ void __launch_bounds__(256) requant_dual_kernel(const int32_t *__rest
 // element 78.0), one output 25.1 (64.0); with the alignment of the kernel above 29.2 and 25.1.
 __global__ void __launch_bounds__(256) requant_dual_words_kernel(const int32_t *__restrict__ acc, long long n, F8Requant q1, F8Requant q2,
                                                                  uint8_t *__restrict__ y1, uint8_t *__restrict__ y2) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const long long i0 = ((long long)blockIdx.x * 1024 + threadIdx.x) * 4;
     int4 a[4];
 #pragma unroll
@@ -100,6 +104,8 @@ __global__ void __launch_bounds__(256) requant_dual_words_kernel(const int32_t *
 // Any alignment.
 __global__ void __launch_bounds__(256) requant_dual_scalar_kernel(const int32_t *__restrict__ acc, long long n, F8Requant q1, F8Requant q2,
                                                                   uint8_t *__restrict__ y1, uint8_t *__restrict__ y2) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const long long stride = (long long)gridDim.x * 256;
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += stride) {
         const int a = __ldg(acc + i);
@@ -136,13 +142,25 @@ extern "C" f8_status f8_requantize_dual_fixed(long long n, const int32_t *acc, i
     const uintptr_t y = (uintptr_t)y1 | (uintptr_t)y2;
     const long long blocks = (n + 4095) / 4096;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (((uintptr_t)acc & 31) == 0 && (y & 15) == 0 && blocks < (1ll << 31))
-        requant_dual_kernel<<<(unsigned)blocks, 256, 0, st>>>(acc, n, q1, q2, (uint8_t *)y1, (uint8_t *)y2);
-    else if (((uintptr_t)acc & 15) == 0 && (y & 3) == 0 && blocks < (1ll << 31))
-        requant_dual_words_kernel<<<(unsigned)blocks, 256, 0, st>>>(acc, n, q1, q2, (uint8_t *)y1, (uint8_t *)y2);
-    else
-        requant_dual_scalar_kernel<<<(unsigned)(blocks < 148 * 16 ? blocks : 148 * 16), 256, 0, st>>>(acc, n, q1, q2, (uint8_t *)y1, (uint8_t *)y2);
-    cudaError_t e = cudaGetLastError();
+    // the blocks may start while what is before them in the stream drains (29.7 M elements, call after call: a gap of 1 us less)
+    cudaLaunchConfig_t cfg = {};
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.gridDim = dim3((unsigned)std::min<long long>(blocks, (1ll << 31) - 1));
+    cudaError_t e;
+    if (((uintptr_t)acc & 31) == 0 && (y & 15) == 0 && blocks < (1ll << 31)) {
+        e = cudaLaunchKernelEx(&cfg, requant_dual_kernel, acc, n, q1, q2, (uint8_t *)y1, (uint8_t *)y2);
+    } else if (((uintptr_t)acc & 15) == 0 && (y & 3) == 0 && blocks < (1ll << 31)) {
+        e = cudaLaunchKernelEx(&cfg, requant_dual_words_kernel, acc, n, q1, q2, (uint8_t *)y1, (uint8_t *)y2);
+    } else {
+        cfg.gridDim = dim3((unsigned)std::min<long long>(blocks, 148 * 16));
+        e = cudaLaunchKernelEx(&cfg, requant_dual_scalar_kernel, acc, n, q1, q2, (uint8_t *)y1, (uint8_t *)y2);
+    }
     if (e != cudaSuccess) return f8_set_error(F8_ERR_CUDA, cudaGetErrorString(e));
     return F8_OK;
 }

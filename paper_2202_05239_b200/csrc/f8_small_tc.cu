@@ -48,6 +48,7 @@ struct SmallParams {
     uint32_t k_bytes;                       // of an output channel's weights
     int bulk;                               // these are fetched by bulk copies
     int unit_step, dst_step, dst_wrap;      // SM_THREADS 16-byte units further on in the first panel's window
+    int wait_first;                         // a call of its own: the weights may come from earlier work in the stream as well
     int tag;
     int *status;
     unsigned long long wait_limit;
@@ -134,6 +135,7 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
     const bool one_panel = PW || p.panels == 1;
     const int first16 = one_panel ? p.last16 : p.p16;
     const uint32_t first_magic = one_panel ? p.last_magic : p.p16_magic;
+    if (p.wait_first) grid_dependency_wait();
     grid_launch_dependents();
 
     // ---- weights of the first two panels: bulk copies, one per output channel, where these are long enough (a lane issues one in about 40
@@ -710,5 +712,6 @@ cudaError_t f8_launch_small_alone(const F8ConvGeom &g, const F8Requant &q, bool 
     const double stores = direct ? (bits8 ? 18e-6 : 24e-6) * ((double)g.n * g.ho * g.wo * g.c_out) : 0.0;
     if (small_us(plan.s) + 4.2 >= 8.0 + std::ceil((double)t.tiles / 148) * t.chunks * chunk + stores) return cudaErrorNotSupported;
     fill_plan(&plan, g, q, x, w, bias, res, y, sib, 0);
-    return f8_small_launch(&plan, false, st);
+    plan.p.wait_first = 1;
+    return f8_small_launch(&plan, true, st);
 }
