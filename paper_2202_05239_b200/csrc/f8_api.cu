@@ -568,6 +568,8 @@ struct f8_net {
     std::vector<int> t_cp;                       // per tensor: channels as stored (intermediate 8-bit tensors are padded
                                                  // to a multiple of 16 so that every dense layer can use the TMA path)
     int max_batch = 0;
+    int need_batch = -1, need_micro = 0;         // workspace bytes of the last batch asked for
+    size_t need = 0;
     // cached execution plan
     int plan_batch = -1;
     const void *plan_x = nullptr;
@@ -581,6 +583,8 @@ struct f8_net {
     int last_launches = 0;
     // The launches of the cached plan as a graph, from its second pass on (f8_net_forward)
     cudaGraphExec_t graph = nullptr;
+    cudaGraph_t graph_src = nullptr;             // what it was made from; its nodes, one per step, name those of `graph`
+    std::vector<cudaGraphNode_t> graph_nodes;
     int graph_passes = 0;                        // passes since the plan was made; -1: no graph for this network
     long long graph_tc = 0;                      // tensor-core launches in it
     unsigned long long graph_wait_limit = 0;     // bound of in-kernel waits that its kernels carry
@@ -802,9 +806,33 @@ void drop_graph(f8_net *net) {
     if (net->graph) {
         RelaxedCapture relaxed;
         cudaGraphExecDestroy(net->graph);
+        cudaGraphDestroy(net->graph_src);
     }
+    net->graph_src = nullptr;
+    net->graph_nodes.clear();
     net->graph = nullptr;
     if (net->graph_passes > 0) net->graph_passes = 0;
+}
+
+// The nodes of the plan's graph in the order of its steps (left empty should the graph be anything but a chain of that many kernels).
+void list_nodes(f8_net *net) {
+    cudaGraphNode_t node;
+    size_t n = 1;
+    if (cudaGraphGetRootNodes(net->graph_src, &node, &n) != cudaSuccess || n != 1) return;
+    for (size_t k = 0; k < net->steps.size(); ++k) {
+        cudaGraphNodeType type;
+        if (cudaGraphNodeGetType(node, &type) != cudaSuccess || type != cudaGraphNodeTypeKernel) break;
+        net->graph_nodes.push_back(node);
+        cudaGraphNode_t next;
+        cudaGraphEdgeData edge;
+        n = 1;
+        if (cudaGraphNodeGetDependentNodes_v2(node, nullptr, nullptr, &n) != cudaSuccess || n != (k + 1 < net->steps.size() ? 1u : 0u)) break;
+        if (n && cudaGraphNodeGetDependentNodes_v2(node, &next, &edge, &n) != cudaSuccess) break;
+        node = next;
+        if (!n) return;
+    }
+    (void)cudaGetLastError();
+    net->graph_nodes.clear();
 }
 
 void free_layers(f8_net *net) {
@@ -818,7 +846,36 @@ void free_layers(f8_net *net) {
 
 }   // namespace
 
-namespace { f8_status launch_steps(f8_net *net, cudaStream_t st, void *const *layer_dump); }
+namespace {
+f8_status launch_steps(f8_net *net, cudaStream_t st, void *const *layer_dump, size_t from = 0, size_t to = (size_t)-1);
+}
+
+namespace {
+
+// Gives the graph's nodes of these steps the parameters of the steps as they are now.
+bool rebind_graph(f8_net *net, const std::vector<size_t> &steps) {
+    if (net->graph_nodes.size() != net->steps.size()) return false;
+    RelaxedCapture relaxed;
+    const long long before = g_tc_launches;
+    bool ok = true;
+    for (size_t k : steps) {
+        cudaGraph_t g = nullptr;
+        if (!ok || cudaStreamBeginCapture(net->lane_stream, cudaStreamCaptureModeRelaxed) != cudaSuccess) { ok = false; break; }
+        const f8_status s = launch_steps(net, net->lane_stream, nullptr, k, k + 1);
+        cudaGraphNode_t node;
+        size_t n = 1;
+        cudaKernelNodeParams params = {};
+        ok = cudaStreamEndCapture(net->lane_stream, &g) == cudaSuccess && s == F8_OK && cudaGraphGetRootNodes(g, &node, &n) == cudaSuccess && n == 1 &&
+             cudaGraphKernelNodeGetParams(node, &params) == cudaSuccess &&
+             cudaGraphExecKernelNodeSetParams(net->graph, net->graph_nodes[k], &params) == cudaSuccess;
+        if (g) cudaGraphDestroy(g);
+    }
+    g_tc_launches = before;
+    if (!ok) (void)cudaGetLastError();
+    return ok;
+}
+
+}   // namespace
 
 extern "C" {
 
@@ -1164,7 +1221,12 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
     if (batch == 0) { net->last_launches = 0; return F8_OK; }
     if (!x || !y) return fail(F8_ERR_NULL, "x and y must not be NULL");
     if (!aligned16(x) || !aligned16(y) || !aligned16(workspace)) return fail(F8_ERR_ALIGN, "device pointers must be 16-byte aligned");
-    const size_t need = f8_net_workspace_bytes(net, batch);
+    if (net->need_batch != batch || net->need_micro != g_micro_batch) {
+        net->need = f8_net_workspace_bytes(net, batch);
+        net->need_batch = batch;
+        net->need_micro = g_micro_batch;
+    }
+    const size_t need = net->need;
     if (need > 256 && (!workspace || workspace_bytes < need))
         return fail(F8_ERR_WORKSPACE, "workspace of %zu bytes needed, %zu given", need, workspace_bytes);
     cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -1178,18 +1240,18 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
     if (layer_dump)
         for (int i = 0; i < nl; ++i)
             if (net->layers[i].w_core && layer_dump[i]) dump_fusable = true;
-    const bool replan = net->plan_batch != batch || net->plan_x != x || net->plan_y != y || net->plan_ws != workspace ||
-                        net->plan_force_direct != g_force_direct || net->plan_dump_first != dump_fusable ||
-                        net->plan_dumping != (layer_dump != nullptr) ||
-                        net->plan_options != g_plan_off || net->plan_micro != g_micro_batch || net->plan_lanes != g_lanes ||
-                        net->plan_profiling != net->profiling;
+    const bool other_plan = net->plan_batch != batch || net->plan_ws != workspace || net->plan_force_direct != g_force_direct ||
+                            net->plan_dump_first != dump_fusable || net->plan_dumping != (layer_dump != nullptr) || net->plan_options != g_plan_off ||
+                            net->plan_micro != g_micro_batch || net->plan_lanes != g_lanes || net->plan_profiling != net->profiling;
+    const bool replan = other_plan || net->plan_x != x || net->plan_y != y;
+    // only the caller's tensors have moved: the steps that touch them are planned again, the others stay
+    bool rebind = replan && !other_plan && net->last_lanes == 1 && net->last_regions == 0 && !net->steps.empty();
+    std::vector<size_t> rebound;
     net->overlap_layers = !(g_plan_off & F8_PLAN_OFF_LAYER_OVERLAP);
     net->sync_layers = (g_plan_off & F8_PLAN_SYNC_LAYERS) != 0;
-    if (replan || net->graph_wait_limit != g_wait_limit_cycles) drop_graph(net);
-    net->graph_wait_limit = g_wait_limit_cycles;
     if (replan) {
         std::fill(g_last_plan, g_last_plan + 10, 0);
-        net->steps.clear();
+        if (!rebind) net->steps.clear();
         net->plan_batch = -1;
         const int lanes = lanes_for(net, batch);
         net->last_lanes = lanes;
@@ -1393,7 +1455,32 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
             }
             ln.steps.push_back(std::move(stp));
         };
-        for (int k = 0; k < lanes; ++k) {
+        for (size_t k = 0; rebind && k < net->steps.size(); ++k) {
+            const Step &old = net->steps[k];
+            const int last_layer = old.fused_pool || old.kind == -3 || old.kind == -4 ? old.layer + 1 : old.layer;
+            bool touches = last_layer + 1 == nl || (old.has_sib && last_layer + 2 == nl);
+            for (int l = old.layer; l <= last_layer; ++l)
+                touches = touches || net->layers[l].d.src == 0 || (net->layers[l].q.has_res && net->layers[l].d.res == 0);
+            if (!touches) continue;
+            Lane &ln = lane_list[0];
+            ln.steps.clear();
+            ln.skip_layer = -1;
+            plan_layer(ln, 0, old.layer, ln.n, 0, false);
+            if (old.kind == -1 || ln.steps.size() != 1 || ln.steps[0].kind != old.kind) {      // (a first layer in two launches)
+                rebind = false;
+            } else {
+                net->steps[k] = std::move(ln.steps[0]);
+                rebound.push_back(k);
+            }
+        }
+        if (!rebind) {
+            net->steps.clear();
+            for (Lane &ln : lane_list) {
+                ln.steps.clear();
+                ln.skip_layer = -1;
+            }
+        }
+        for (int k = 0; !rebind && k < lanes; ++k) {
             Lane &ln = lane_list[k];
             for (int i = 0; i < nl;) {
                 const int r = ln.layer_region[i];
@@ -1413,7 +1500,7 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
             }
         }
         // launch order: the lanes take turns, one launch each
-        {
+        if (!rebind) {
             size_t longest = 0;
             for (const Lane &ln : lane_list) longest = std::max(longest, ln.steps.size());
             for (size_t j = 0; j < longest; ++j)
@@ -1433,9 +1520,12 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
         net->plan_profiling = net->profiling;
     }
 
-    // From the second pass over the same buffers on the launches go out as one graph: the host issues it in about 10 us instead of 2.7 us
+    // From the second pass of a plan on the launches go out as one graph: the host issues it in about 10 us instead of 2.7 us
     // a launch, and the hand-overs inside it are shorter (ResNet-50 at batch 1 211 -> 189 us a pass, at batch 19, 160 x 160, 350 -> 320).
-    // The first pass does not pay for a graph that may never run again.  A caller's own capture takes the launches one by one.
+    // The first pass does not pay for a graph that may never run again.  Where only the caller's tensors have moved, the nodes that
+    // touch them get their new parameters.  A caller's own capture takes the launches one by one.
+    if ((replan && !rebind) || net->graph_wait_limit != g_wait_limit_cycles || (net->graph && !rebound.empty() && !rebind_graph(net, rebound))) drop_graph(net);
+    net->graph_wait_limit = g_wait_limit_cycles;
     const bool graph_ok = net->graph_passes >= 0 && net->last_lanes == 1 && !layer_dump && !net->profiling && !net->sync_layers && net->steps.size() >= 4;
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (graph_ok && net->graph_passes >= 1 && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
@@ -1449,7 +1539,12 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                 s = launch_steps(net, net->lane_stream, nullptr);
                 if (cudaStreamEndCapture(net->lane_stream, &g) != cudaSuccess || s != F8_OK || cudaGraphInstantiate(&net->graph, g, 0) != cudaSuccess)
                     net->graph = nullptr;
-                if (g) cudaGraphDestroy(g);
+                if (net->graph) {
+                    net->graph_src = g;
+                    list_nodes(net);
+                } else if (g) {
+                    cudaGraphDestroy(g);
+                }
             }
             net->graph_tc = g_tc_launches - before;
             g_tc_launches = before;
@@ -1474,7 +1569,7 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
 namespace {
 
 // Enqueues the cached plan's launches (and the copies of the layers' outputs that are asked for).
-f8_status launch_steps(f8_net *net, cudaStream_t st, void *const *layer_dump) {
+f8_status launch_steps(f8_net *net, cudaStream_t st, void *const *layer_dump, size_t from, size_t to) {
     int launches = 0;
     const bool prof = net->profiling;
     if (prof) {
@@ -1494,7 +1589,8 @@ f8_status launch_steps(f8_net *net, cudaStream_t st, void *const *layer_dump) {
         if (e == cudaSuccess) e = cudaStreamWaitEvent(net->lane_stream, net->ev_fork, 0);
         if (e != cudaSuccess) return cuda_fail(e, "second lane fork");
     }
-    for (Step &stp : net->steps) {
+    for (size_t k = from; k < std::min(to, net->steps.size()); ++k) {
+        Step &stp = net->steps[k];
         NetLayer &L = net->layers[stp.layer];
         cudaError_t e = cudaSuccess;
         st = stp.lane == 1 ? net->lane_stream : caller_stream;
@@ -1577,7 +1673,7 @@ f8_status launch_steps(f8_net *net, cudaStream_t st, void *const *layer_dump) {
         if (e == cudaSuccess) e = cudaStreamWaitEvent(caller_stream, net->ev_join, 0);
         if (e != cudaSuccess) return cuda_fail(e, "second lane join");
     }
-    net->last_launches = launches;
+    if (from == 0 && to >= net->steps.size()) net->last_launches = launches;
     return F8_OK;
 }
 

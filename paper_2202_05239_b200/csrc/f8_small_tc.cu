@@ -602,7 +602,7 @@ static double tcgen05_us(const F8ConvGeom &g, bool bits8) {
     const double chunk = t.bn > 128 ? 0.30 * width : (t.bn <= 32 ? 0.11 : (t.row_tiles ? 0.14 : 0.17)) * (t.bn > 64 ? width : 1.0);
     const double finish = 0.25 * std::max(1.0, t.bn / 64.0), rounds = std::ceil((double)t.tiles / 148);
     // (8-bit outputs of a c_out that 16 does not divide, 32-bit or second outputs of small tensors: direct stores)
-    const double direct = bits8 ? (g.c_out % 16 != 0 ? 18e-6 * out : 0.0) : (t.row_tiles ? 1.5 : 0.0);
+    const double direct = bits8 ? (g.c_out % 16 != 0 ? 18e-6 * out : 0.0) : (g.c_out % 16 != 0 ? 16e-6 * out : (t.row_tiles ? 1.5 : 0.0));
     return 2.7 + rounds * std::max(t.chunks * chunk, finish) + finish + (out * (bits8 ? 1 : 4) + (double)g.n * g.h * g.w * g.c) / 6e6 + direct;
 }
 // (only the tap inside the image counts there: one pixel, 3 x 3 x 800 to 24 channels 2.4 us)

@@ -1,4 +1,4 @@
-"""GPU parity of repeated forward passes over the same buffers, which go out as one CUDA graph from the second pass on."""
+"""GPU parity of repeated forward passes, which go out as one CUDA graph from the second pass on."""
 import numpy as np
 import pytest
 import torch
@@ -39,8 +39,13 @@ def test_repeated_passes(ref, name, batch, image):
     for i in range(4):                       # the second and later passes are the graph's; the input changes in place
         check(i & 1)
     check(1, stream=side)                    # on another stream
-    check(0, out=other)                      # another output: a plan of its own, then a graph of its own
+    check(0, out=other)                      # another output, then the first one: the same graph with other parameters
+    check(1)
     check(1, out=other)
+    first, x = x, torch.empty_like(x)        # ... and another input
+    check(0)
+    check(1, out=other)
+    x = first
     check(0, dump=[net.layer_output(i, batch) for i in range(len(layers))])
     check(1)
     check(0)
