@@ -194,8 +194,7 @@ f8_status run_dense(const F8ConvGeom &g, const F8Requant &q, const void *x, cons
     std::fill(g_last_plan, g_last_plan + 10, 0);      // (no plan unless the tcgen05 kernel makes one below)
     const size_t x_bytes = (size_t)g.n * g.h * g.w * g.c;
     // Inputs of a few tiles: the kernel for small layers, which needs no tensor maps (encoding four of them takes the host longer
-    // than the layer takes the GPU).  16 x 16 x 16, 3 x 3: 6.8 -> 5.1 us on the host.  Not with thousands of output channels or
-    // products per output (31 x 31 x 16, 3 x 3 to 4096 channels 28.9 us, on the tcgen05 kernel 15.7).
+    // than the layer takes the GPU).  Not where its estimate is the larger one: thousands of output channels, several panels of K.
     if (!g_force_direct && !(g_plan_off & F8_PLAN_OFF_SMALL_KERNEL)) {
         const cudaError_t e = f8_launch_small_alone(g, q, is_bits8(q, sib), x, w, bias, res, y, st, sib);
         if (e == cudaSuccess) {

@@ -10,7 +10,8 @@
 // Behind the wait there is one fetch of the window, one pass over K with all warps on slices of their own (mma.sync m16n8k32, no block
 // barrier inside), and the sums of the slices meet in shared memory (integers: any order gives the same result) for bias, shortcut,
 // rounding shift, clip and a second consumer, for every output kind the library has.  The form before it walked K in 128-byte chunks
-// with a barrier each and gathered every tap: K = 2304 took 3.5 us behind the wait, K = 4608 7.5 - 10 us.
+// with a barrier each and gathered every tap: K = 2304 took 3.5 us behind the wait, K = 4608 7.5 - 10 us, now 1.3 - 1.5 us.  Inside a
+// network 14 x 14, 3 x 3 256 -> 256 of one image adds 3.5 us, 1 x 1 64 -> 384 1.8 us, of which 1.15 us are the hand-over itself.
 // Layers whose window and weights do not fit go over the channels in panels, two in flight.
 // mma.sync cannot reach the rate of tcgen05.mma (2045 multiply-adds a clock and SM, measured), which is why layers with more work
 // stay with the other kernel (f8_small_tc_wanted has the rule and what was measured on both sides of it).
@@ -684,16 +685,19 @@ cudaError_t f8_small_plan_init(F8SmallPlan *plan, const F8ConvGeom &g, const F8R
     return cudaSuccess;
 }
 
+static cudaError_t launch_plan(const SmallParams &p, const Split &s, bool xs, cudaStream_t st, bool overlap_previous) {
+    if (p.pointwise && !p.strided && p.panels == 1) {
+        if (s.t == 32) return xs ? launch_small<2, 4, true, true>(p, s, st, overlap_previous) : launch_small<2, 4, false, true>(p, s, st, overlap_previous);
+        return xs ? launch_small<1, 2, true, true>(p, s, st, overlap_previous) : launch_small<1, 2, false, true>(p, s, st, overlap_previous);
+    }
+    if (s.t == 32) return xs ? launch_small<2, 4, true, false>(p, s, st, overlap_previous) : launch_small<2, 4, false, false>(p, s, st, overlap_previous);
+    return xs ? launch_small<1, 2, true, false>(p, s, st, overlap_previous) : launch_small<1, 2, false, false>(p, s, st, overlap_previous);
+}
+
 cudaError_t f8_small_launch(const F8SmallPlan *plan, bool overlap_previous, cudaStream_t st) {
     SmallParams p = plan->p;
     p.wait_limit = f8_wait_limit_cycles();
-    const Split &s = plan->s;
-    if (p.pointwise && !p.strided && p.panels == 1) {
-        if (s.t == 32) return plan->x_signed ? launch_small<2, 4, true, true>(p, s, st, overlap_previous) : launch_small<2, 4, false, true>(p, s, st, overlap_previous);
-        return plan->x_signed ? launch_small<1, 2, true, true>(p, s, st, overlap_previous) : launch_small<1, 2, false, true>(p, s, st, overlap_previous);
-    }
-    if (s.t == 32) return plan->x_signed ? launch_small<2, 4, true, false>(p, s, st, overlap_previous) : launch_small<2, 4, false, false>(p, s, st, overlap_previous);
-    return plan->x_signed ? launch_small<1, 2, true, false>(p, s, st, overlap_previous) : launch_small<1, 2, false, false>(p, s, st, overlap_previous);
+    return launch_plan(p, plan->s, plan->x_signed != 0, st, overlap_previous);
 }
 
 // A call of its own, inputs below 16 KiB: launches and returns success, or cudaErrorNotSupported where another kernel is the better one.
@@ -713,5 +717,6 @@ cudaError_t f8_launch_small_alone(const F8ConvGeom &g, const F8Requant &q, bool 
     if (small_us(plan.s) + 4.2 >= 8.0 + std::ceil((double)t.tiles / 148) * t.chunks * chunk + stores) return cudaErrorNotSupported;
     fill_plan(&plan, g, q, x, w, bias, res, y, sib, 0);
     plan.p.wait_first = 1;
-    return f8_small_launch(&plan, true, st);
+    plan.p.wait_limit = f8_wait_limit_cycles();
+    return launch_plan(plan.p, plan.s, plan.x_signed != 0, st, true);
 }

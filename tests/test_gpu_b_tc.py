@@ -249,3 +249,35 @@ def test_fully_connected_layers_with_many_outputs(ref, c, c_out, n):
     layer = random_conv_layer(np.random.default_rng(c_out), h=1, w=1, c=c, c_out=c_out, k=1, stride=1, pad=0, x_signed=False, y_dtype=synth.S32,
                               with_res=False)
     check_layer(ref, layer, random_input(np.random.default_rng(1), n, layer), expect_tc=True)
+
+
+# Layers of a network whose tiles leave SMs idle get narrower ones; a call of its own keeps the tiles that CTA pairs need
+# (h, w, c, c_out, k, n, x_signed, columns of a tile in a network)
+NARROW_CASES = [
+    (14, 14, 256, 256, 3, 16, False, 64),        # 25 M tiles: 100 tiles of 64 columns
+    (14, 14, 256, 256, 3, 33, False, 128),       # 51: 102 of 128, 204 of 64
+    (7, 7, 512, 480, 3, 40, True, 64),           # 16: 128 of 64, the last of a row half empty
+    (28, 28, 128, 128, 3, 8, False, 128),        # a single tile of columns: its windows stay
+    (14, 14, 96, 576, 1, 8, False, 256),         # less than one 128-byte chunk of K
+    (14, 14, 256, 1024, 1, 40, False, 256),      # 62: two tiles of 256 columns for every SM
+]
+
+
+@pytest.mark.parametrize("case", range(len(NARROW_CASES)))
+def test_narrow_tiles_in_a_network(ref, case):
+    from paper_2202_05239_b200 import api as a
+    h, w, c, c_out, k, n, xs, bn = NARROW_CASES[case]
+    rng = np.random.default_rng(1700 + case)
+    layer = random_conv_layer(rng, h=h, w=w, c=c, c_out=c_out, k=k, stride=1, pad=k // 2, x_signed=xs, y_dtype=synth.U8, with_res=False)
+    x = random_input(rng, n, layer)
+    a.f8_debug_plan_options(a.PLAN_OFF_SMALL_KERNEL)
+    try:
+        net = a.Net([layer], n)
+        out = net.forward(a.to_device(x))
+        torch.cuda.synchronize()
+        plan = a.f8_debug_last_plan()
+    finally:
+        a.f8_debug_plan_options(0)
+    assert plan["bn"] == bn, plan
+    assert np.array_equal(out.cpu().numpy(), ref.run_layer(layer, x))
+    net.close()
