@@ -613,9 +613,14 @@ static double cuda_core_us(const F8ConvGeom &g) {
 
 bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8) {
     Split s;
-    if (!shape_ok(g) || !pick_split(g, &s)) return false;
-    if (!f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c)) return small_us(s) < cuda_core_us(g);
-    return s.panels == 1 && small_us(s) < 0.97 * tcgen05_us(g, bits8);
+    if (!shape_ok(g)) return false;
+    if (!f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c)) return pick_split(g, &s) && small_us(s) < cuda_core_us(g);
+    // what every split takes at least (products at the rate of mma.sync, blocks of at most 8192 outputs): spares large layers the search
+    const double out = (double)g.n * g.ho * g.wo * g.c_out, other = 0.97 * tcgen05_us(g, bits8);
+    s.panels = 1;
+    s.cycles = (float)(700 + out * g.kh * g.kw * g.c / (148 * 1800.0) + 700 * std::max(0.0, out / (8192 * 148.0) - 1));
+    if (small_us(s) >= other) return false;
+    return pick_split(g, &s) && s.panels == 1 && small_us(s) < other;
 }
 
 struct F8SmallPlan {
