@@ -55,8 +55,8 @@ struct SmallParams {
     unsigned long long wait_limit;
     uint32_t pa, pb;                        // bytes from pixel to pixel of a window, from channel to channel of the weights
     uint32_t b_off, stage;                  // weights behind the window; bytes of a stage
-    int plain8;                             // one 8-bit output, shift 1 .. 24: multiply-add, shift, saturating pack
-    int mul_acc, mul_res, round;
+    int plain8;                             // one 8-bit output, shift 2 .. 24: multiply-add, shifts, saturating pack
+    int mul_acc, mul_res;
     const uint8_t *x;
     const int8_t *wgt;                      // [c_out][taps * c]
     const int32_t *bias;
@@ -105,12 +105,13 @@ __device__ __forceinline__ void store4(void *y, int y_kind, int s, int lo, int h
     else *(uint32_t *)((uint8_t *)y + o) = f8_pack4(t[0], t[1], t[2], t[3]);
 }
 
-// Four sums to four bytes: rounding shift (the constant is in v already) and clip.
+// Four sums to four bytes: rounding shift by s >= 2 and clip.  Half the constant is added behind most of the shift: v + 2^(s-1) would
+// leave 32 bits for sums that do fit (a 32-bit shortcut takes them up to 2^31 - 1).
 __device__ __forceinline__ uint32_t pack_plain8(const int (&v)[4], int s, bool is_signed) {
     int t[4];
     uint32_t hi, o;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) t[j] = v[j] >> s;
+    for (int j = 0; j < 4; ++j) t[j] = ((v[j] >> (s - 1)) + 1) >> 1;
     if (is_signed) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) t[j] = max(t[j], -127);
@@ -318,8 +319,8 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
     PIN(bulk);
     PIN(put); PIN(pitch_bytes); PIN(slice_bytes); PIN(get); PIN(get_step); PIN(my_slices);
     if (!PW) PIN(n_panels);
-    int mul_acc = p.mul_acc, mul_res = p.mul_res, round = p.round, shift = p.q.s, plain8 = p.plain8, out_signed = p.q.y_kind == F8_S8, r_signed = p.q.r_signed;
-    PIN(mul_acc); PIN(mul_res); PIN(round); PIN(shift); PIN(plain8); PIN(out_signed); PIN(r_signed);
+    int mul_acc = p.mul_acc, mul_res = p.mul_res, shift = p.q.s, plain8 = p.plain8, out_signed = p.q.y_kind == F8_S8, r_signed = p.q.r_signed;
+    PIN(mul_acc); PIN(mul_res); PIN(shift); PIN(plain8); PIN(out_signed); PIN(r_signed);
     uint8_t *y8 = (uint8_t *)p.y + out0;
     PIN64(y8);
 
@@ -461,8 +462,6 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
                 for (int e = 0; e < 4; ++e) v[e] = v[e] * mul_acc + rr[e] * mul_res;
             }
             if (plain8) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] += round;
                 *(uint32_t *)(y8 + skip) = pack_plain8(v, shift, out_signed);
             } else {
                 store4(p.y, p.q.y_kind, p.q.s, p.q.lo, p.q.hi, v, out0 + skip);
@@ -674,10 +673,9 @@ static void fill_plan(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q
     p.tag = tag;
     p.b_off = (uint32_t)s.window;
     p.stage = (uint32_t)(s.window + s.weights);
-    p.plain8 = (q.y_kind == F8_U8 || q.y_kind == F8_S8) && q.s >= 1 && q.s <= 24 && !(sib && sib->y2);
+    p.plain8 = (q.y_kind == F8_U8 || q.y_kind == F8_S8) && q.s >= 2 && q.s <= 24 && !(sib && sib->y2);
     p.mul_acc = 1 << q.sh_acc;
     p.mul_res = 1 << q.sh_res;
-    p.round = p.plain8 ? 1 << (q.s - 1) : 0;
     p.x = (const uint8_t *)x; p.wgt = w; p.bias = bias; p.res = res; p.y = y;
     p.q = q;
     if (sib) p.sib = *sib;

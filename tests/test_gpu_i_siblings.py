@@ -87,6 +87,36 @@ def test_sibling_outputs_and_32_bit_shortcuts(ref, case):
         assert torch.equal(single, y1.t)
 
 
+# (h, c, n, kernel): 16 KiB and less take the kernel for small layers, the others the tcgen05 kernel
+@pytest.mark.parametrize("h,c,n,small", [(16, 16, 1, True), (7, 48, 2, True), (28, 64, 6, False)])
+@pytest.mark.parametrize("kind", [U8, S8])
+@pytest.mark.parametrize("s", [1, 2, 8, 24, 25, 31])
+def test_sums_at_the_ends_of_32_bits(ref, h, c, n, small, kind, s):
+    """One 8-bit output of a sum with a 32-bit shortcut: the sum has to fit int32, the sum plus the rounding constant has not."""
+    a = api()
+    fl_y = 0 if s == 31 else 7 if s < 25 else 6
+    fa = s + fl_y
+    fl_x = min(fa, 7)
+    layer = random_conv_layer(np.random.default_rng(s), h=h, w=h, c=c, c_out=c, k=3, stride=1, pad=1, x_signed=False, y_dtype=kind, with_res=False,
+                              fl_x=fl_x, fl_w=fa - fl_x, fl_y=fl_y)
+    layer.weight[:] = 0
+    x = np.zeros((n, h, h, c), dtype=np.uint8)
+    top, half = (1 << 31) - 1, 1 << (s - 1)
+    sums = np.array([top, top + 1 - half, top - half, top - 2 * half, -top - 1, -top - 1 + half, 0, half, half - 1, -half, -half - 1, 3 * half], dtype=np.int64)
+    layer.bias[:] = 0
+    res = np.resize(np.clip(sums, -top - 1, top), (n, h, h, c)).astype(np.int32)
+    want, _ = ref.conv2d_siblings(x, layer.weight, layer.bias, stride=1, pad=1, fl_x=fl_x, fl_w=fa - fl_x, y1_kind=kind, fl_y1=fl_y, residual=res, fl_r=fa)
+    desc = a.conv_desc(layer, n)
+    desc.r_dtype, desc.fl_r = S32, fa
+    y = Guarded((n, h, h, c), a.torch_dtype(kind))
+    a.f8_conv2d_siblings_fixed(desc, 0, 0, a.to_device(x), a.to_device(layer.weight), a.to_device(layer.bias), a.to_device(res), y.t, None)
+    torch.cuda.synchronize()
+    a.f8_device_status()
+    assert bool(a.f8_debug_last_plan()["m_tiles"]) != small
+    assert y.intact()
+    assert_equal_arrays(y.t.cpu().numpy(), want)
+
+
 def test_sibling_validation():
     a = api()
     rng = np.random.default_rng(1)
