@@ -48,8 +48,9 @@ struct FoldParams {
     bool bias_last;                       // the biases overwrite gamma or sigma: in a launch behind the last use of the row scales
 };
 
+// (no read-only loads in this file: the first launch's blocks already wait while the grid before them may write these tensors)
 __device__ __forceinline__ double row_scale(const FoldParams &p, int row) {
-    return __dmul_rn(__ddiv_rn((double)__ldg(p.gamma + row), (double)__ldg(p.sigma + row)), p.ratio);
+    return __dmul_rn(__ddiv_rn((double)p.gamma[row], (double)p.sigma[row]), p.ratio);
 }
 
 // Scales of the rows the chunk at e0 touches, once per chunk (false: too many rows for the table).
@@ -76,14 +77,14 @@ __device__ __forceinline__ void load_weights(const FoldParams &p, long long e0, 
 #pragma unroll
         for (int g = 0; g < FOLD_PER_THREAD / 4; ++g) {
             const long long e = fold_index<true>(e0, 4 * g);
-            const float4 t = e < p.n ? __ldg((const float4 *)(p.w + e)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 t = e < p.n ? *(const float4 *)(p.w + e) : make_float4(0.f, 0.f, 0.f, 0.f);
             f[4 * g] = t.x; f[4 * g + 1] = t.y; f[4 * g + 2] = t.z; f[4 * g + 3] = t.w;
         }
     } else {
 #pragma unroll
         for (int j = 0; j < FOLD_PER_THREAD; ++j) {
             const long long e = fold_index<false>(e0, j);
-            f[j] = e < p.n ? __ldg(p.w + e) : 0.f;
+            f[j] = e < p.n ? p.w[e] : 0.f;
         }
     }
 }
@@ -144,8 +145,8 @@ __global__ void __launch_bounds__(FOLD_THREADS) fold_stats_kernel(const FoldPara
 __device__ __forceinline__ void write_biases(const FoldParams &p, int fl) {
     const int fa = p.fl_x + fl;
     for (int i = (int)(blockIdx.x * FOLD_THREADS + threadIdx.x); i < p.c_out; i += (int)gridDim.x * FOLD_THREADS) {
-        const double gs = __ddiv_rn((double)__ldg(p.gamma + i), (double)__ldg(p.sigma + i));
-        const double be = __ddiv_rn(__dsub_rn((double)__ldg(p.beta + i), __dmul_rn(gs, (double)__ldg(p.mu + i))), p.eta_out);
+        const double gs = __ddiv_rn((double)p.gamma[i], (double)p.sigma[i]);
+        const double be = __ddiv_rn(__dsub_rn((double)p.beta[i], __dmul_rn(gs, (double)p.mu[i])), p.eta_out);
         double t = floor(__dadd_rn(scalbn(be, fa), 0.5));
         t = fmin(fmax(t, -2147483648.0), 2147483647.0);
         p.b_q[i] = (int32_t)t;

@@ -235,7 +235,7 @@ __device__ __forceinline__ void epilogue_chunk(const TcParams &p, const int (&ac
     }
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
-        const int b = (j < nvalid && p.bias) ? __ldg(p.bias + co0 + j) : 0;
+        const int b = (j < nvalid && p.bias) ? p.bias[co0 + j] : 0;
         v[j] = f8_align_add(acc[j] + b, r[j], p.q);
     }
     if (!row_valid) return;
@@ -880,6 +880,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         bool ok = true;
         if (STAGED) {
             {
+                // (a plain load: in a call of its own the grid before this one may write the biases)
                 // bias' = (bias << sh_acc) + 2^(s-1) for every (padded) output column, once per CTA.  Only these warps
                 // read the table, so they build it -- behind a barrier of their own -- while the producers and the MMA
                 // issuers are already at work: the prologue of a CTA starts when the previous layer's CTA has left the SM,
@@ -887,7 +888,7 @@ f8_conv_gemm_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
                 int *bias_all = (int *)(smem + p.bias_off);
                 const int rnd = WIDE ? 0 : 1 << (p.q.s - 1);      // (two outputs round at different places)
                 for (int i = (int)threadIdx.x - FIRST_EPI_WARP * 32; i < p.n_tiles * p.bn; i += NUM_EPI_WARPS * 32)
-                    bias_all[i] = ((i < p.c_out && p.bias) ? (__ldg(p.bias + i) << p.q.sh_acc) : 0) + rnd;
+                    bias_all[i] = ((i < p.c_out && p.bias) ? (p.bias[i] << p.q.sh_acc) : 0) + rnd;
                 asm volatile("bar.sync 1, %0;" ::"n"(NUM_EPI_WARPS * 32) : "memory");
             }
             const int tile_row = quarter * 32 + lane;

@@ -13,10 +13,12 @@
 
 namespace {
 
+// (no read-only loads in this file: what is read may be written by the grid before this one while the blocks here already wait)
 __device__ __forceinline__ void load32(const int32_t *p, int (&v)[8]) {
-    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "l"(p));
+                 : "l"(p)
+                 : "memory");
 }
 
 // Four rounded, clipped and packed codes.  SHIFT: 1 <= s <= 31; else the general form (s <= 0: a left shift).
@@ -53,7 +55,7 @@ __device__ __forceinline__ uint4 requant16(const int (&u)[8], const int (&v)[8],
 }
 
 // acc 32-byte, y1 / y2 16-byte aligned; the last thread takes the ragged tail.
-__global__ void __launch_bounds__(256) requant_dual_kernel(const int32_t *__restrict__ acc, long long n, F8Requant q1, F8Requant q2,
+__global__ void __launch_bounds__(256) requant_dual_kernel(const int32_t *acc, long long n, F8Requant q1, F8Requant q2,
                                                             uint8_t *__restrict__ y1, uint8_t *__restrict__ y2) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -66,7 +68,7 @@ __global__ void __launch_bounds__(256) requant_dual_kernel(const int32_t *__rest
         if (y2) *(uint4 *)(y2 + i) = requant16(u, v, q2);
     } else {
         for (long long j = i; j < n; ++j) {
-            const int a = __ldg(acc + j);
+            const int a = acc[j];
             y1[j] = (uint8_t)(f8_requant(a, 0, q1) & 0xff);
             if (y2) y2[j] = (uint8_t)(f8_requant(a, 0, q2) & 0xff);
         }
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(256) requant_dual_kernel(const int32_t *__rest
 // acc 16-byte, y1 / y2 4-byte aligned (views that start at a multiple of four elements): four 16-byte loads in flight per thread,
 // neighbouring threads on neighbouring words.  29.7 M elements, two outputs: 30.4 us (element by
 // element 78.0), one output 25.1 (64.0); with the alignment of the kernel above 29.2 and 25.1.
-__global__ void __launch_bounds__(256) requant_dual_words_kernel(const int32_t *__restrict__ acc, long long n, F8Requant q1, F8Requant q2,
+__global__ void __launch_bounds__(256) requant_dual_words_kernel(const int32_t *acc, long long n, F8Requant q1, F8Requant q2,
                                                                  uint8_t *__restrict__ y1, uint8_t *__restrict__ y2) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -84,7 +86,7 @@ __global__ void __launch_bounds__(256) requant_dual_words_kernel(const int32_t *
     int4 a[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-        if (i0 + 1024 * u + 4 <= n) a[u] = __ldg((const int4 *)(acc + i0 + 1024 * u));
+        if (i0 + 1024 * u + 4 <= n) a[u] = *(const int4 *)(acc + i0 + 1024 * u);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const long long i = i0 + 1024 * u;
@@ -93,7 +95,7 @@ __global__ void __launch_bounds__(256) requant_dual_words_kernel(const int32_t *
             if (y2) *(uint32_t *)(y2 + i) = requant4(a[u], q2);
         } else {
             for (long long j = i; j < n; ++j) {
-                const int v = __ldg(acc + j);
+                const int v = acc[j];
                 y1[j] = (uint8_t)(f8_requant(v, 0, q1) & 0xff);
                 if (y2) y2[j] = (uint8_t)(f8_requant(v, 0, q2) & 0xff);
             }
@@ -102,13 +104,13 @@ __global__ void __launch_bounds__(256) requant_dual_words_kernel(const int32_t *
 }
 
 // Any alignment.
-__global__ void __launch_bounds__(256) requant_dual_scalar_kernel(const int32_t *__restrict__ acc, long long n, F8Requant q1, F8Requant q2,
+__global__ void __launch_bounds__(256) requant_dual_scalar_kernel(const int32_t *acc, long long n, F8Requant q1, F8Requant q2,
                                                                   uint8_t *__restrict__ y1, uint8_t *__restrict__ y2) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const long long stride = (long long)gridDim.x * 256;
     for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < n; i += stride) {
-        const int a = __ldg(acc + i);
+        const int a = acc[i];
         y1[i] = (uint8_t)(f8_requant(a, 0, q1) & 0xff);
         if (y2) y2[i] = (uint8_t)(f8_requant(a, 0, q2) & 0xff);
     }

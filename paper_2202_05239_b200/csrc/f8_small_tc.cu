@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
     const int f_row = it >> gs, f_col = (it & ((1 << gs) - 1)) * 4, co = n0 + f_col;
     const int m_end = it < groups && co < p.c_out ? min(p.M, m0 + p.bm) : 0;
     int4 bias = make_int4(0, 0, 0, 0);               // (one of the threads that share a group)
-    if (p.bias && m_end && part == 0) bias = __ldg((const int4 *)(p.bias + co));
+    if (p.bias && m_end && part == 0) bias = *(const int4 *)(p.bias + co);      // (no read-only load: the wait above is inside this kernel)
 
     // ---- the copies of this thread: the first ones as finished addresses, the loop for what is left, further panels, skipped pixels
     const int n_first = !PW && (p.strided || !one_panel) ? 0 : count * first16;
