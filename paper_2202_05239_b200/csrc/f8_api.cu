@@ -1556,6 +1556,7 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
             const cudaError_t e = cudaGraphLaunch(net->graph, st);
             if (e != cudaSuccess) return cuda_fail(e, "launch of the pass");
             g_tc_launches += net->graph_tc;
+            net->last_launches = (int)net->steps.size();       // (a pass of no images in between has set it to 0)
             return F8_OK;
         }
     }

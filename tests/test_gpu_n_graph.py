@@ -68,3 +68,22 @@ def test_repeated_passes(ref, name, batch, image):
     del g
     check(0)
     net.close()
+
+
+def test_launch_count_behind_a_pass_of_no_images():
+    a = api()
+    layers = synth.make_net("resnet18", 0, image=64)
+    net = a.Net(layers, 2)
+    x = a.to_device(synth.draw_image(2, 1, 64, 64))
+    out = torch.empty((2,) + net.out_shape, dtype=net.out_dtype, device="cuda")
+    ws = torch.empty(net.workspace_bytes(2), dtype=torch.uint8, device="cuda")
+    for _ in range(12):
+        net.forward(x, out=out, workspace=ws)
+    launches = net.last_launch_count
+    assert launches > 4
+    net.forward(x[:0], out=out[:0], workspace=ws)
+    assert net.last_launch_count == 0
+    net.forward(x, out=out, workspace=ws)
+    assert net.last_launch_count == launches
+    torch.cuda.synchronize()
+    net.close()
