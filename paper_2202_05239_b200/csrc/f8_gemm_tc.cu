@@ -1196,6 +1196,13 @@ bool f8_tc_supported(const F8ConvGeom &g, size_t x_bytes) {
     return true;
 }
 
+// Tiles of output pixels: inputs below 128 KiB of layers that are not pointwise take whole output rows of one image per tile (`rows`).
+static long long m_tile_count(const F8ConvGeom &g, bool rows) {
+    if (!rows || g.wo > TILE_M) return ((long long)g.n * g.ho * g.wo + TILE_M - 1) / TILE_M;
+    const int per = std::min(TILE_M / g.wo, g.ho);
+    return (long long)g.n * ((g.ho + per - 1) / per);
+}
+
 F8TcTiles f8_tc_tiles(const F8ConvGeom &g, bool bits8) {
     F8TcTiles t;
     t.kb = choose_kb(g.c);
@@ -1203,8 +1210,7 @@ F8TcTiles f8_tc_tiles(const F8ConvGeom &g, bool bits8) {
     const bool pointwise = g.kh == 1 && g.kw == 1 && g.stride_h == 1 && g.stride_w == 1 && g.pad_h == 0 && g.pad_w == 0;
     const bool big = (size_t)g.n * g.h * g.w * g.c >= 128 * 1024;
     t.row_tiles = !big && !pointwise && g.wo <= TILE_M;
-    const int rows = t.row_tiles ? std::min(TILE_M / g.wo, g.ho) : 1;
-    const long long m_tiles = t.row_tiles ? (long long)g.n * ((g.ho + rows - 1) / rows) : ((long long)g.n * g.ho * g.wo + TILE_M - 1) / TILE_M;
+    const long long m_tiles = m_tile_count(g, t.row_tiles);
     if (bits8 && g.c_out % 16 == 0) {
         t.bn = narrow_bn(choose_bn_staged(g.c_out, false, t.kb), m_tiles, g, 148);
     } else if (g.c_out % 16 == 0 && (big || pointwise)) {
@@ -1285,7 +1291,8 @@ cudaError_t f8_tc_plan_init(F8TcPlan *plan, const F8ConvGeom &g, const F8Requant
     // (single-layer calls keep the tiles that CTA pairs need)
     const bool pair_shape = g.c % 128 == 0 && g.c_out % 256 == 0 && g.kh * g.kw * (g.c / 128) >= 8 && big_x && p.m_tiles >= 2;
     if (staged && !wide && (in_network || !pair_shape)) {
-        const int bn = narrow_bn(p.bn, p.m_tiles, g, sm_count_here());
+        // (by the tiles that the layer will have: 7 x 7, 3 x 3 64 -> 512 of 40 images has 40 of whole rows, not 16)
+        const int bn = narrow_bn(p.bn, m_tile_count(g, !big_x && !pointwise1), g, sm_count_here());
         if (bn < p.bn) {
             p.bn = bn;
             p.kb = choose_kb(g.c);           // (64-byte chunks make room for the ring of 256-wide tiles)

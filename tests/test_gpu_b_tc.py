@@ -260,6 +260,10 @@ NARROW_CASES = [
     (28, 28, 128, 128, 3, 8, False, 128),        # a single tile of columns: its windows stay
     (14, 14, 96, 576, 1, 8, False, 256),         # less than one 128-byte chunk of K
     (14, 14, 256, 1024, 1, 40, False, 256),      # 62: two tiles of 256 columns for every SM
+    # below 128 KiB: tiles of whole rows, one image each
+    (7, 7, 64, 512, 3, 40, False, 256),          # 40 tiles, 16 by pixels: 160 of 128 columns would be two rounds
+    (7, 7, 256, 1024, 3, 10, True, 128),         # 10 tiles: 80 of 128, 160 of 64
+    (7, 7, 64, 512, 3, 18, False, 64),           # 18: 144 of 64
 ]
 
 
@@ -279,5 +283,7 @@ def test_narrow_tiles_in_a_network(ref, case):
     finally:
         a.f8_debug_plan_options(0)
     assert plan["bn"] == bn, plan
+    if bn < 128 or (bn == 128 and c_out > 128):          # made narrower: one tile at most for every SM
+        assert plan["m_tiles"] * plan["n_tiles"] <= torch.cuda.get_device_properties(0).multi_processor_count, plan
     assert np.array_equal(out.cpu().numpy(), ref.run_layer(layer, x))
     net.close()
