@@ -55,8 +55,9 @@ struct SmallParams {
     unsigned long long wait_limit;
     uint32_t pa, pb;                        // bytes from pixel to pixel of a window, from channel to channel of the weights
     uint32_t b_off, stage;                  // weights behind the window; bytes of a stage
-    int plain8;                             // one 8-bit output, shift 2 .. 24: multiply-add, shifts, saturating pack
-    int mul_acc, mul_res;
+    int plain8;                             // one 8-bit output, shift 1 .. 24, sums that fit 32 bits with the rounding constant: multiply-add,
+                                            // shift, saturating pack
+    int mul_acc, mul_res, round;
     const uint8_t *x;
     const int8_t *wgt;                      // [c_out][taps * c]
     const int32_t *bias;
@@ -105,13 +106,12 @@ __device__ __forceinline__ void store4(void *y, int y_kind, int s, int lo, int h
     else *(uint32_t *)((uint8_t *)y + o) = f8_pack4(t[0], t[1], t[2], t[3]);
 }
 
-// Four sums to four bytes: rounding shift by s >= 2 and clip.  Half the constant is added behind most of the shift: v + 2^(s-1) would
-// leave 32 bits for sums that do fit (a 32-bit shortcut takes them up to 2^31 - 1).
+// Four sums to four bytes: rounding shift (the constant is in v already) and clip.
 __device__ __forceinline__ uint32_t pack_plain8(const int (&v)[4], int s, bool is_signed) {
     int t[4];
     uint32_t hi, o;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) t[j] = ((v[j] >> (s - 1)) + 1) >> 1;
+    for (int j = 0; j < 4; ++j) t[j] = v[j] >> s;
     if (is_signed) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) t[j] = max(t[j], -127);
@@ -319,8 +319,8 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
     PIN(bulk);
     PIN(put); PIN(pitch_bytes); PIN(slice_bytes); PIN(get); PIN(get_step); PIN(my_slices);
     if (!PW) PIN(n_panels);
-    int mul_acc = p.mul_acc, mul_res = p.mul_res, shift = p.q.s, plain8 = p.plain8, out_signed = p.q.y_kind == F8_S8, r_signed = p.q.r_signed;
-    PIN(mul_acc); PIN(mul_res); PIN(shift); PIN(plain8); PIN(out_signed); PIN(r_signed);
+    int mul_acc = p.mul_acc, mul_res = p.mul_res, round = p.round, shift = p.q.s, plain8 = p.plain8, out_signed = p.q.y_kind == F8_S8, r_signed = p.q.r_signed;
+    PIN(mul_acc); PIN(mul_res); PIN(round); PIN(shift); PIN(plain8); PIN(out_signed); PIN(r_signed);
     uint8_t *y8 = (uint8_t *)p.y + out0;
     PIN64(y8);
 
@@ -462,6 +462,8 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
                 for (int e = 0; e < 4; ++e) v[e] = v[e] * mul_acc + rr[e] * mul_res;
             }
             if (plain8) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] += round;
                 *(uint32_t *)(y8 + skip) = pack_plain8(v, shift, out_signed);
             } else {
                 store4(p.y, p.q.y_kind, p.q.s, p.q.lo, p.q.hi, v, out0 + skip);
@@ -631,7 +633,7 @@ struct F8SmallPlan {
 size_t f8_small_plan_size() { return sizeof(F8SmallPlan); }
 
 static void fill_plan(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
-                      const void *res, void *y, const F8Sibling *sib, int tag) {
+                      const void *res, void *y, const F8Sibling *sib, int tag, bool alone) {
     const Split &s = plan->s;
     plan->x_signed = g.x_signed;
     SmallParams &p = plan->p;
@@ -673,9 +675,12 @@ static void fill_plan(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q
     p.tag = tag;
     p.b_off = (uint32_t)s.window;
     p.stage = (uint32_t)(s.window + s.weights);
-    p.plain8 = (q.y_kind == F8_U8 || q.y_kind == F8_S8) && q.s >= 2 && q.s <= 24 && !(sib && sib->y2);
+    // A network has checked that its sums fit 32 bits together with the constant 2^(s-1).  Of a single-layer call with a 32-bit shortcut
+    // only the sums themselves do: they are rounded by the general path.
+    p.plain8 = (q.y_kind == F8_U8 || q.y_kind == F8_S8) && q.s >= 1 && q.s <= 24 && !(sib && sib->y2) && !(alone && q.r_s32);
     p.mul_acc = 1 << q.sh_acc;
     p.mul_res = 1 << q.sh_res;
+    p.round = p.plain8 ? 1 << (q.s - 1) : 0;
     p.x = (const uint8_t *)x; p.wgt = w; p.bias = bias; p.res = res; p.y = y;
     p.q = q;
     if (sib) p.sib = *sib;
@@ -684,7 +689,7 @@ static void fill_plan(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q
 cudaError_t f8_small_plan_init(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
                                const void *res, void *y, const F8Sibling *sib, int tag) {
     if (!shape_ok(g) || !pick_split(g, &plan->s)) return cudaErrorNotSupported;
-    fill_plan(plan, g, q, x, w, bias, res, y, sib, tag);
+    fill_plan(plan, g, q, x, w, bias, res, y, sib, tag, false);
     return cudaSuccess;
 }
 
@@ -718,7 +723,7 @@ cudaError_t f8_launch_small_alone(const F8ConvGeom &g, const F8Requant &q, bool 
     const double chunk = t.bn <= 16 ? 0.14 : (t.bn <= 32 ? (pointwise ? 0.18 : 0.12) : (t.bn <= 64 ? 0.13 : (t.bn <= 128 ? 0.25 : 0.5)));
     const double stores = direct ? (bits8 ? 18e-6 : 24e-6) * ((double)g.n * g.ho * g.wo * g.c_out) : 0.0;
     if (small_us(plan.s) + 4.2 >= 8.0 + std::ceil((double)t.tiles / 148) * t.chunks * chunk + stores) return cudaErrorNotSupported;
-    fill_plan(&plan, g, q, x, w, bias, res, y, sib, 0);
+    fill_plan(&plan, g, q, x, w, bias, res, y, sib, 0, true);
     plan.p.wait_first = 1;
     plan.p.wait_limit = f8_wait_limit_cycles();
     return launch_plan(plan.p, plan.s, plan.x_signed != 0, st, true);
