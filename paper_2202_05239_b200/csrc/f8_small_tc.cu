@@ -12,7 +12,8 @@
 // rounding shift, clip and a second consumer, for every output kind the library has.  The form before it walked K in 128-byte chunks
 // with a barrier each and gathered every tap: K = 2304 took 3.5 us behind the wait, K = 4608 7.5 - 10 us, now 1.3 - 1.5 us.  Inside a
 // network 14 x 14, 3 x 3 256 -> 256 of one image adds 3.5 us, 1 x 1 64 -> 384 1.8 us, of which 1.15 us are the hand-over itself.
-// Layers whose window and weights do not fit go over the channels in panels, two in flight.
+// Layers whose window and weights do not fit go over the channels in panels, two in flight (one where two of the smallest panels do
+// not fit either: filters of 21 x 21 and more).
 // mma.sync cannot reach the rate of tcgen05.mma (2045 multiply-adds a clock and SM, measured), which is why layers with more work
 // stay with the other kernel (f8_small_tc_wanted has the rule and what was measured on both sides of it).
 #include <math.h>
@@ -45,6 +46,7 @@ struct SmallParams {
     int ho, wo, kh, kw, taps, stride, pad;
     int pointwise, strided;                 // 1x1 without padding; 1x1 that skips pixels
     int panels, p16, last16;                // panels of channels: 16-byte units per pixel in one, in the last one
+    int ahead;                              // panels in flight: 2 or 1
     uint32_t wo_magic, ho_magic, kw_magic, p16_magic, last_magic, row_magic, last_row_magic;
     uint32_t k_bytes;                       // of an output channel's weights
     int bulk;                               // these are fetched by bulk copies
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
         __syncwarp();
     }
     load_weights(0);
-    if (!one_panel) load_weights(1);
+    if (!one_panel && p.ahead == 2) load_weights(1);
 
     // ---- the window: the input pixels of this tile, contiguous in memory (rows of the batch, one below the other)
     int first = m0, count;
@@ -195,8 +197,9 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
     } else {
         const int r0 = quick_div(m0, p.wo_magic), r1 = quick_div(m1, p.wo_magic);
         const int i0 = quick_div(r0, p.ho_magic), i1 = quick_div(r1, p.ho_magic);
-        const int y0 = i0 * p.h + max((r0 - i0 * p.ho) * p.stride - p.pad, 0);
-        const int y1 = i1 * p.h + min((r1 - i1 * p.ho) * p.stride - p.pad + p.kh - 1, p.h - 1);
+        // (both inside an image: with padding as large as the filter, rows of outputs may read nothing but padding)
+        const int y0 = i0 * p.h + min(max((r0 - i0 * p.ho) * p.stride - p.pad, 0), p.h - 1);
+        const int y1 = i1 * p.h + max(min((r1 - i1 * p.ho) * p.stride - p.pad + p.kh - 1, p.h - 1), 0);
         first = y0 * p.w;
         count = (y1 - y0 + 1) * p.w;
         ih = p.h;
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
         if (j < win_n) cp_async16(win_dst[j], win_src + j * SM_THREADS * 16);
     if (more_window) load_window(0, window_left);
     cp_async_commit();
-    if (n_panels > 1) load_window(1, tid);
+    if (n_panels > 1 && p.ahead == 2) load_window(1, tid);
     cp_async_commit();
 #pragma unroll
     for (int j = 0; j < FINISH_AHEAD; ++j) {
@@ -407,11 +410,14 @@ __global__ void __launch_bounds__(SM_THREADS, MT == 1 ? 3 : 2) f8_conv_small_tc_
             if (steps_left) mma(0);
         }
         __syncthreads();                             // everybody has read the stage
-        if (panel + 2 < n_panels) {
-            load_weights(panel + 2);
-            load_window(panel + 2, tid);
+        if (!PW && n_panels > 1) {
+            if (panel + p.ahead < n_panels) {
+                load_weights(panel + p.ahead);
+                load_window(panel + p.ahead, tid);
+            }
+            cp_async_commit();
+            if (p.ahead == 1) cp_async_commit();     // (the wait above leaves one group in flight: an empty one)
         }
-        cp_async_commit();
     }
 
     // ---- the slices of K meet in shared memory
@@ -483,7 +489,7 @@ int log2_of(int v) {
 
 // How a layer is cut: warp tile edge, warps along rows, columns and K, channels per panel, shared memory, estimated cycles.
 struct Split {
-    int t, wm, wn, wk_shift, p16, panels;
+    int t, wm, wn, wk_shift, p16, panels, ahead;
     size_t window, weights, smem;           // one stage's window and weights, whole block
     long long tiles;
     float cycles;
@@ -517,10 +523,10 @@ bool pick_split(const F8ConvGeom &g, Split *best) {
                 const int wk = 3 - wm_shift - wn_shift, bn = t << wn_shift;
                 if (wn_shift && bn / 2 >= c_out) break;
                 const size_t red = ((size_t)bm << wk) * (bn + 8) * 4;
-                int at16 = 0;
+                int at16 = 0, ahead = 2;
                 size_t window = 0, weights = 0, smem = 0;
-                // one panel where it fits, else two stages in half of the shared memory
-                for (int p16 = c16; p16 >= 1; p16 = p16 == c16 ? (c16 + 1) / 2 : p16 - std::max(1, p16 / 8)) {
+                // one panel where it fits, else two stages in half of the shared memory; the smallest panel may take all of it
+                for (int p16 = c16;; p16 = p16 == c16 ? (c16 + 1) / 2 : p16 - std::max(1, p16 / 8)) {
                     window = ((size_t)px * ((p16 | 1) * 16) + 127) / 128 * 128;
                     weights = ((size_t)bn * (((size_t)taps * p16 | 1) * 16) + 16 + 127) / 128 * 128;
                     smem = SM_ZERO + std::max((window + weights) * (p16 == c16 ? 1 : 2), red);
@@ -528,7 +534,11 @@ bool pick_split(const F8ConvGeom &g, Split *best) {
                         at16 = p16;
                         break;
                     }
-                    if (c16 == 1) break;
+                    if (p16 == 1 && c16 > 1 && SM_ZERO + std::max(window + weights, red) <= (size_t)SM_SMEM) {
+                        smem = SM_ZERO + std::max(window + weights, red);
+                        at16 = ahead = 1;
+                    }
+                    if (p16 == 1) break;
                 }
                 if (!at16) continue;
                 const int panels = (c16 + at16 - 1) / at16;
@@ -543,9 +553,9 @@ bool pick_split(const F8ConvGeom &g, Split *best) {
                 const float issue = 700.f * std::max(0.f, (float)tiles / 148 - 1);
                 // (no room for the next layer's block: its start is not hidden)
                 const float alone = occ == 1 ? 600.f : 0.f;
-                const float cycles = 700 + alone + issue + fetch + mul + finish + (panels - 1) * 300.f + std::max(0, panels - 2) * fetch_w / panels +
+                const float cycles = 700 + alone + issue + fetch + mul + finish + (panels - 1) * 300.f + std::max(0, panels - ahead) * (ahead == 2 ? fetch_w : 2 * (fetch + fetch_w)) / panels +
                                      (rounds - 1) * (1500 + fetch + fetch_w + mul + finish);
-                if (cycles < best->cycles) *best = {t, 1 << wm_shift, 1 << wn_shift, wk, at16, panels, window, weights, smem, tiles, cycles};
+                if (cycles < best->cycles) *best = {t, 1 << wm_shift, 1 << wn_shift, wk, at16, panels, ahead, window, weights, smem, tiles, cycles};
             }
         }
     return best->cycles < 1e29f;
@@ -580,7 +590,6 @@ cudaError_t launch_small(const SmallParams &p, const Split &s, cudaStream_t st, 
 
 static bool shape_ok(const F8ConvGeom &g) {
     if (g.c % 16 != 0 || g.c_out % 4 != 0 || g.pad_h_end >= 0 || g.stride_h != g.stride_w || g.pad_h != g.pad_w) return false;
-    if (g.pad_h >= g.kh || g.pad_w >= g.kw) return false;                // (a window starts and ends inside an image)
     const long long m = (long long)g.n * g.ho * g.wo, k = (long long)g.kh * g.kw * g.c;
     if (m <= 0 || m >= (1ll << 24) || k >= (1ll << 24) || g.kh >= 256 || g.kw >= 256) return false;
     // 32-bit offsets, and quotients by multiplication (n * d < 2^32)
@@ -607,15 +616,17 @@ static double tcgen05_us(const F8ConvGeom &g, bool bits8) {
     const double direct = bits8 ? (g.c_out % 16 != 0 ? 18e-6 * out : 0.0) : (g.c_out % 16 != 0 ? 16e-6 * out : (t.row_tiles ? 1.5 : 0.0));
     return 2.7 + rounds * std::max(t.chunks * chunk, finish) + finish + (out * (bits8 ? 1 : 4) + (double)g.n * g.h * g.w * g.c) / 6e6 + direct;
 }
-// (only the tap inside the image counts there: one pixel, 3 x 3 x 800 to 24 channels 2.4 us)
-static double cuda_core_us(const F8ConvGeom &g) {
-    return g.h == 1 && g.w == 1 ? 2.0 + 0.0095 * g.c * std::max(1.0, (double)g.n * g.ho * g.wo * g.c_out / 256) : 1e9;
+// (only the taps inside the image count there: one pixel, 3 x 3 x 800 to 24 channels 2.4 us.  Of more pixels it has no estimate but for
+// filters that take a panel at a time here: 25 x 25 over 11 x 11 x 32 to 64 channels 70.6 us, here 20.0; over 3 x 3 x 48 to 40 14.4, here 29.4)
+static double cuda_core_us(const F8ConvGeom &g, const Split &s) {
+    if (g.h == 1 && g.w == 1) return 2.0 + 0.0095 * g.c * std::max(1.0, (double)g.n * g.ho * g.wo * g.c_out / 256);
+    return s.ahead == 1 ? 2.0 + 0.0177 * g.c * std::min(g.kh, g.h) * std::min(g.kw, g.w) : 1e9;
 }
 
 bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8) {
     Split s;
     if (!shape_ok(g)) return false;
-    if (!f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c)) return pick_split(g, &s) && small_us(s) < cuda_core_us(g);
+    if (!f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c)) return pick_split(g, &s) && small_us(s) < cuda_core_us(g, s);
     // what every split takes at least (products at the rate of mma.sync, blocks of at most 8192 outputs): spares large layers the search
     const double out = (double)g.n * g.ho * g.wo * g.c_out, other = 0.97 * tcgen05_us(g, bits8);
     s.panels = 1;
@@ -655,6 +666,7 @@ static void fill_plan(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q
     p.strided = p.pointwise && g.stride_h > 1;
     p.panels = s.panels;
     p.p16 = s.p16;
+    p.ahead = s.ahead;
     p.last16 = g.c / 16 - (s.panels - 1) * s.p16;
     p.wo_magic = magic_of(g.wo);
     p.ho_magic = magic_of(g.ho);
@@ -674,7 +686,7 @@ static void fill_plan(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q
     p.status = f8_status_word();
     p.tag = tag;
     p.b_off = (uint32_t)s.window;
-    p.stage = (uint32_t)(s.window + s.weights);
+    p.stage = s.ahead == 2 ? (uint32_t)(s.window + s.weights) : 0u;
     // A network has checked that its sums fit 32 bits together with the constant 2^(s-1).  Of a single-layer call with a 32-bit shortcut
     // only the sums themselves do: they are rounded by the general path.
     p.plain8 = (q.y_kind == F8_U8 || q.y_kind == F8_S8) && q.s >= 1 && q.s <= 24 && !(sib && sib->y2) && !(alone && q.r_s32);

@@ -136,6 +136,18 @@ WINDOWS = [
     (12, 12, 32, 64, 3, 1, 0, 2, False, synth.U8, False),       # no padding: rows between two images that no filter starts at
     (11, 11, 64, 64, 2, 2, 0, 3, False, synth.U8, False),       # ... and that no filter reaches
     (8, 8, 128, 128, 7, 1, 3, 1, False, synth.U8, False),       # 49 taps
+    # padding as large as the filter and larger: outputs, and whole rows of them, that read nothing but padding
+    (8, 8, 32, 32, 3, 1, 3, 1, False, synth.U8, True),
+    (12, 12, 64, 64, 1, 1, 1, 2, True, synth.S8, False),
+    (9, 9, 16, 24, 2, 2, 2, 3, False, synth.U8, False),
+    (5, 6, 48, 20, 1, 3, 2, 2, False, synth.S32, False),
+    (7, 7, 32, 48, 3, 2, 5, 4, True, synth.U8, False),
+    (1, 1, 2048, 64, 1, 1, 1, 1, False, synth.U8, False),
+    (4, 4, 64, 72, 5, 1, 7, 2, False, synth.U8, False),
+    # filters so large that only one of the smallest panels fits: two and three of them
+    (11, 11, 32, 64, 25, 1, 12, 1, False, synth.U8, False),
+    (8, 8, 32, 40, 29, 1, 14, 1, True, synth.U8, False),
+    (9, 9, 48, 16, 25, 1, 12, 1, False, synth.S8, True),
 ]
 
 
