@@ -580,6 +580,7 @@ struct f8_net {
     std::vector<size_t> t_off;                   // workspace offset per tensor
     size_t pack_off = 0;
     int last_launches = 0;
+    int last_plan[10] = {0};                     // what f8_debug_last_plan reports of the cached plan
     // The launches of the cached plan as a graph, from its second pass on (f8_net_forward)
     cudaGraphExec_t graph = nullptr;
     cudaGraph_t graph_src = nullptr;             // what it was made from; its nodes, one per step, name those of `graph`
@@ -1517,6 +1518,9 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
         net->plan_micro = g_micro_batch;
         net->plan_lanes = g_lanes;
         net->plan_profiling = net->profiling;
+        // (steps that were planned again are what they were; the report is of the whole plan)
+        if (rebind) std::copy(net->last_plan, net->last_plan + 10, g_last_plan);
+        else std::copy(g_last_plan, g_last_plan + 10, net->last_plan);
     }
 
     // From the second pass of a plan on the launches go out as one graph: the host issues it in about 10 us instead of 2.7 us

@@ -87,3 +87,22 @@ def test_launch_count_behind_a_pass_of_no_images():
     assert net.last_launch_count == launches
     torch.cuda.synchronize()
     net.close()
+
+
+def test_last_plan_of_a_pass_with_other_buffers():
+    """f8_debug_last_plan reports the pass's plan, also when only the steps at the caller's tensors were planned again."""
+    a = api()
+    layers = synth.make_net("resnet50", 0, image=96)
+    net = a.Net(layers, 8)
+    x = a.to_device(synth.draw_image(8, 1, 96, 96))
+    ws = torch.empty(net.workspace_bytes(8), dtype=torch.uint8, device="cuda")
+    outs = [torch.empty((8,) + net.out_shape, dtype=net.out_dtype, device="cuda") for _ in range(2)]
+    net.forward(x, out=outs[0], workspace=ws)
+    plan = a.f8_debug_last_plan()
+    assert plan["m_tiles"] > 0
+    net.forward(x, out=outs[1], workspace=ws)
+    assert a.f8_debug_last_plan() == plan
+    net.forward(x.clone(), out=outs[0], workspace=ws)
+    assert a.f8_debug_last_plan() == plan
+    torch.cuda.synchronize()
+    net.close()
