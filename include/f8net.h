@@ -394,6 +394,13 @@ int f8_net_micro_batching(const f8_net *net, int *images);
 void f8_debug_set_lanes(int lanes);
 int f8_net_lanes(const f8_net *net);
 
+/* How the passes of this object went out (n <= 4 ints are written, the count is returned): [0] 1 when the last f8_net_forward sent
+ * its launches as the kept graph, [1] graphs made so far, [2] launches of kept graphs that got new parameters because the caller's
+ * tensors had moved, [3] attempts to make or launch a graph that failed (the launches then go out one by one; the next plan, or the
+ * same one about a hundred passes later, tries again).  f8_debug_fail_graphs: test hook, the next `count` attempts of this process fail. */
+int f8_net_graph_info(const f8_net *net, int *info, int n);
+void f8_debug_fail_graphs(int count);
+
 /* What the most recent tcgen05 plan of this process decided (n <= 10 ints are written, the count is returned; all zero when the
  * last single-layer call, or the last network planned, made none):
  * [0] flags below, [1] epilogue variant (0 generic, 1 u8, 2 u8 + residual, 3 s8, 4 s8 + residual, 5 with a 32-bit

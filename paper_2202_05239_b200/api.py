@@ -283,11 +283,19 @@ _lib.f8_debug_set_lanes.argtypes = [_ci]
 _lib.f8_debug_set_lanes.restype = None
 _lib.f8_net_lanes.argtypes = [_vp]
 _lib.f8_net_fused_pairs.argtypes = [_vp]
+_lib.f8_net_graph_info.argtypes = [_vp, ctypes.POINTER(_ci), _ci]
+_lib.f8_debug_fail_graphs.argtypes = [_ci]
+_lib.f8_debug_fail_graphs.restype = None
 
 
 def f8_debug_set_lanes(lanes: int):
     """Concurrent lanes of f8_net_forward: 0 the library's rule, 1 or 2 that many."""
     _lib.f8_debug_set_lanes(lanes)
+
+
+def f8_debug_fail_graphs(count: int):
+    """The next `count` attempts of a network to keep its launches as a graph fail (on the host)."""
+    _lib.f8_debug_fail_graphs(count)
 
 
 def f8_debug_last_plan() -> dict:
@@ -439,6 +447,13 @@ class Net:
     def fused_pairs(self) -> int:
         """Launches of the last forward pass that ran two layers at once."""
         return int(_lib.f8_net_fused_pairs(self._h))
+
+    @property
+    def graph_info(self) -> dict:
+        """Whether the last forward pass went out as the kept graph; graphs made, launches updated and failures so far."""
+        v = (_ci * 4)()
+        _lib.f8_net_graph_info(self._h, v, 4)
+        return dict(zip(("last", "made", "updates", "failed"), [int(x) for x in v]))
 
     def micro_batching(self):
         """(number of runs of layers the last forward pass executed depth-first over micro-batches, smallest micro-batch)."""

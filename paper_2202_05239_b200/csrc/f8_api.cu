@@ -23,6 +23,8 @@ unsigned long long g_wait_limit_cycles = 0;   // 0: the kernels' default
 int g_last_plan[10] = {0};
 int g_micro_batch = 0;                        // 0: no micro-batching; > 0: this micro-batch in every eligible run; -1: the L2 rule
 int g_lanes = 0;                              // 0: automatic; 1 / 2: that many concurrent lanes in f8_net_forward
+int g_fail_graphs = 0;                        // so many graphs of networks fail to be made (test hook)
+constexpr int GRAPH_RETRY = 100;              // passes after a failure until a graph is tried again
 
 f8_status fail(f8_status s, const char *fmt, ...) {
     va_list ap;
@@ -306,6 +308,8 @@ void f8_debug_plan_options(unsigned off_mask) { g_plan_off = off_mask; }
 
 void f8_debug_set_micro_batch(int images) { g_micro_batch = images > 0 ? images : (images < 0 ? -1 : 0); }
 
+void f8_debug_fail_graphs(int count) { g_fail_graphs = count > 0 ? count : 0; }
+
 void f8_debug_set_lanes(int lanes) { g_lanes = lanes == 1 || lanes == 2 ? lanes : 0; }
 
 int f8_debug_last_plan(int *info, int n) {
@@ -585,7 +589,8 @@ struct f8_net {
     cudaGraphExec_t graph = nullptr;
     cudaGraph_t graph_src = nullptr;             // what it was made from; its nodes, one per step, name those of `graph`
     std::vector<cudaGraphNode_t> graph_nodes;
-    int graph_passes = 0;                        // passes since the plan was made; -1: no graph for this network
+    int graph_passes = 0;                        // passes since the plan was made; below 0: so many until a graph is tried again
+    int graph_stats[4] = {0};                    // f8_net_graph_info
     long long graph_tc = 0;                      // tensor-core launches in it
     unsigned long long graph_wait_limit = 0;     // bound of in-kernel waits that its kernels carry
     // optional per-layer timing
@@ -811,7 +816,7 @@ void drop_graph(f8_net *net) {
     net->graph_src = nullptr;
     net->graph_nodes.clear();
     net->graph = nullptr;
-    if (net->graph_passes > 0) net->graph_passes = 0;
+    net->graph_passes = 0;
 }
 
 // The nodes of the plan's graph in the order of its steps (left empty should the graph be anything but a chain of that many kernels).
@@ -871,7 +876,8 @@ bool rebind_graph(f8_net *net, const std::vector<size_t> &steps) {
         if (g) cudaGraphDestroy(g);
     }
     g_tc_launches = before;
-    if (!ok) (void)cudaGetLastError();
+    if (ok) net->graph_stats[2] += (int)steps.size();
+    else (void)cudaGetLastError();
     return ok;
 }
 
@@ -1160,6 +1166,13 @@ size_t f8_net_workspace_bytes(const f8_net *net, int batch) {
 }
 
 int f8_net_last_launch_count(const f8_net *net) { return net ? net->last_launches : 0; }
+
+int f8_net_graph_info(const f8_net *net, int *info, int n) {
+    if (!net || !info || n <= 0) return 0;
+    const int m = n < 4 ? n : 4;
+    for (int i = 0; i < m; ++i) info[i] = net->graph_stats[i];
+    return m;
+}
 
 int f8_net_lanes(const f8_net *net) { return net ? net->last_lanes : 0; }
 
@@ -1529,7 +1542,8 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
     // touch them get their new parameters.  A caller's own capture takes the launches one by one.
     if ((replan && !rebind) || net->graph_wait_limit != g_wait_limit_cycles || (net->graph && !rebound.empty() && !rebind_graph(net, rebound))) drop_graph(net);
     net->graph_wait_limit = g_wait_limit_cycles;
-    const bool graph_ok = net->graph_passes >= 0 && net->last_lanes == 1 && !layer_dump && !net->profiling && !net->sync_layers && net->steps.size() >= 4;
+    net->graph_stats[0] = 0;
+    const bool graph_ok = net->last_lanes == 1 && !layer_dump && !net->profiling && !net->sync_layers && net->steps.size() >= 4;
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (graph_ok && net->graph_passes >= 1 && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
         if (!net->graph) {
@@ -1540,8 +1554,10 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
             f8_status s = F8_ERR_CUDA;
             if (cudaStreamBeginCapture(net->lane_stream, cudaStreamCaptureModeRelaxed) == cudaSuccess) {
                 s = launch_steps(net, net->lane_stream, nullptr);
-                if (cudaStreamEndCapture(net->lane_stream, &g) != cudaSuccess || s != F8_OK || cudaGraphInstantiate(&net->graph, g, 0) != cudaSuccess)
+                if (cudaStreamEndCapture(net->lane_stream, &g) != cudaSuccess || s != F8_OK || g_fail_graphs > 0 ||
+                    cudaGraphInstantiate(&net->graph, g, 0) != cudaSuccess)
                     net->graph = nullptr;
+                if (g_fail_graphs > 0) --g_fail_graphs;
                 if (net->graph) {
                     net->graph_src = g;
                     list_nodes(net);
@@ -1551,20 +1567,27 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
             }
             net->graph_tc = g_tc_launches - before;
             g_tc_launches = before;
+            // (a moment without memory, for instance: this plan tries again later, another plan as if nothing had happened)
             if (!net->graph) {
                 (void)cudaGetLastError();
-                net->graph_passes = -1;
+                net->graph_passes = -GRAPH_RETRY;
             }
+            ++net->graph_stats[net->graph ? 1 : 3];
         }
         if (net->graph) {
-            const cudaError_t e = cudaGraphLaunch(net->graph, st);
-            if (e != cudaSuccess) return cuda_fail(e, "launch of the pass");
-            g_tc_launches += net->graph_tc;
-            net->last_launches = (int)net->steps.size();       // (a pass of no images in between has set it to 0)
-            return F8_OK;
+            if (cudaGraphLaunch(net->graph, st) == cudaSuccess) {
+                g_tc_launches += net->graph_tc;
+                net->last_launches = (int)net->steps.size();       // (a pass of no images in between has set it to 0)
+                net->graph_stats[0] = 1;
+                return F8_OK;
+            }
+            (void)cudaGetLastError();            // its first launch needs memory too; nothing of it has been enqueued
+            drop_graph(net);
+            net->graph_passes = -GRAPH_RETRY;
+            ++net->graph_stats[3];
         }
     }
-    if (net->graph_passes == 0) net->graph_passes = 1;
+    if (net->graph_passes < 1) ++net->graph_passes;
     return launch_steps(net, st, layer_dump);
 }
 

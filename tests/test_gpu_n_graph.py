@@ -106,3 +106,38 @@ def test_last_plan_of_a_pass_with_other_buffers():
     assert a.f8_debug_last_plan() == plan
     torch.cuda.synchronize()
     net.close()
+
+
+def test_a_graph_that_cannot_be_made_is_tried_again(ref):
+    """The failure is made on the host.  The passes go out launch by launch meanwhile; another plan tries at once, the same one later."""
+    a = api()
+    layers = synth.make_net("resnet18", 0, image=64)
+    host = synth.draw_image(2, 1, 64, 64)
+    want = ref.net_forward(layers, host, keep_all=False)[-1]
+    net = a.Net(layers, 2)
+    x = a.to_device(host)
+    out = torch.empty((2,) + net.out_shape, dtype=net.out_dtype, device="cuda")
+    spaces = [torch.empty(net.workspace_bytes(2), dtype=torch.uint8, device="cuda") for _ in range(2)]
+
+    def passes(n, ws):
+        for _ in range(n):
+            out.zero_()
+            net.forward(x, out=out, workspace=ws)
+        torch.cuda.synchronize()
+        assert_equal_arrays(out.cpu().numpy(), want)
+        return net.graph_info
+    try:
+        a.f8_debug_fail_graphs(2)
+        assert passes(40, spaces[0]) == {"last": 0, "made": 0, "updates": 0, "failed": 1}
+        info = passes(40, spaces[1])                     # another plan: its first attempt fails too
+        assert (info["made"], info["failed"]) == (0, 2)
+        info = passes(40, spaces[0])
+        assert (info["last"], info["made"], info["failed"]) == (1, 1, 2)
+        a.f8_debug_fail_graphs(1)
+        info = passes(40, spaces[1])
+        assert (info["last"], info["made"], info["failed"]) == (0, 1, 3)
+        info = passes(100, spaces[1])                    # the same plan
+        assert (info["last"], info["made"], info["failed"]) == (1, 2, 3)
+    finally:
+        a.f8_debug_fail_graphs(0)
+    net.close()
