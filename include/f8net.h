@@ -216,9 +216,10 @@ size_t f8_net_workspace_bytes(const f8_net *net, int batch);
  * input; y: the last layer's output ([batch, out] int32 logits for a net ending in a linear
  * layer).  layer_dump: NULL, or an array of n_layers device pointers; a non-NULL entry i
  * receives a copy of layer i's output (for parity checks).
- * Schedule: layers run one after the other over the whole batch on cuda_stream.  From the second pass with the same batch and workspace
- * on they go out as one CUDA graph that the object keeps (and drops when these or a debug setting change); inside a
- * capture of the caller's, with layer_dump and with profiling they are always launched one by one.  Two alternatives exist, both off
+ * Schedule: layers run one after the other over the whole batch on cuda_stream.  After sixteen passes with the same batch and workspace
+ * they go out as one CUDA graph that the object keeps (and drops when these or a debug setting change; the driver takes some memory for
+ * it, and where there is none the launches stay single ones); inside a capture of the caller's, with layer_dump and with profiling they
+ * are always launched one by one.  Two alternatives exist, both off
  * by default because they measured slower on this GPU (every extra launch costs about 5 us of drained SMs):
  * f8_debug_set_lanes(2) cuts the batch into two halves that run as two independent passes, one on cuda_stream and
  * one on a stream the network owns, launched alternately (the call returns with cuda_stream waiting for both);

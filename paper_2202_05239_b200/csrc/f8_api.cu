@@ -24,6 +24,13 @@ int g_last_plan[10] = {0};
 int g_micro_batch = 0;                        // 0: no micro-batching; > 0: this micro-batch in every eligible run; -1: the L2 rule
 int g_lanes = 0;                              // 0: automatic; 1 / 2: that many concurrent lanes in f8_net_forward
 int g_fail_graphs = 0;                        // so many graphs of networks fail to be made (test hook)
+// Passes of a plan that go out launch by launch before its launches are kept as a graph.  Making one costs the calling thread about 280 us
+// for the 52 - 54 launches of ResNet-50 or MobileNet V2 (capture, instantiation, first upload; 200 for the 22 of ResNet-18) and saves 15 - 30
+// us a pass that the caller waits for, so it is paid back after 10 to 20 passes.  A plan that is left sooner, as by a server whose batch
+// changes, never pays.  Batch 1 and 19 in turns (ResNet-18: 8), n passes each, waited for, us a pass, graph from the second pass / after
+// sixteen: ResNet-50 n = 2 444 / 300, n = 8 305 / 287, n = 16 281 / 284, n = 32 268 / 280, n = 64 261 / 267;
+// MobileNet V2 n = 2 384 / 237, n = 8 250 / 227, n = 64 210 / 214; ResNet-18 n = 2 241 / 145, n = 8 156 / 139, n = 64 130 / 133.
+constexpr int GRAPH_AFTER = 16;
 constexpr int GRAPH_RETRY = 100;              // passes after a failure until a graph is tried again
 
 f8_status fail(f8_status s, const char *fmt, ...) {
@@ -585,7 +592,7 @@ struct f8_net {
     size_t pack_off = 0;
     int last_launches = 0;
     int last_plan[10] = {0};                     // what f8_debug_last_plan reports of the cached plan
-    // The launches of the cached plan as a graph, from its second pass on (f8_net_forward)
+    // The launches of the cached plan as a graph, once it has been used GRAPH_AFTER times (f8_net_forward)
     cudaGraphExec_t graph = nullptr;
     cudaGraph_t graph_src = nullptr;             // what it was made from; its nodes, one per step, name those of `graph`
     std::vector<cudaGraphNode_t> graph_nodes;
@@ -1536,16 +1543,15 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
         else std::copy(g_last_plan, g_last_plan + 10, net->last_plan);
     }
 
-    // From the second pass of a plan on the launches go out as one graph: the host issues it in about 10 us instead of 2.7 us
-    // a launch, and the hand-overs inside it are shorter (ResNet-50 at batch 1 211 -> 189 us a pass, at batch 19, 160 x 160, 350 -> 320).
-    // The first pass does not pay for a graph that may never run again.  Where only the caller's tensors have moved, the nodes that
-    // touch them get their new parameters.  A caller's own capture takes the launches one by one.
+    // The launches of a plan that stays in use go out as one graph: the host issues it in 13 - 25 us instead of 2.7 us a launch, and the
+    // hand-overs inside it are shorter (ResNet-50 at batch 1 211 -> 189 us a pass, at batch 19, 160 x 160, 350 -> 320).  Where only the
+    // caller's tensors have moved, the nodes that touch them get their new parameters.  A caller's own capture takes the launches one by one.
     if ((replan && !rebind) || net->graph_wait_limit != g_wait_limit_cycles || (net->graph && !rebound.empty() && !rebind_graph(net, rebound))) drop_graph(net);
     net->graph_wait_limit = g_wait_limit_cycles;
     net->graph_stats[0] = 0;
     const bool graph_ok = net->last_lanes == 1 && !layer_dump && !net->profiling && !net->sync_layers && net->steps.size() >= 4;
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (graph_ok && net->graph_passes >= 1 && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
+    if (graph_ok && net->graph_passes >= GRAPH_AFTER && cudaStreamIsCapturing(st, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
         if (!net->graph) {
             // captured on the network's own stream; nothing but launches happens in between
             const long long before = g_tc_launches;
@@ -1587,7 +1593,7 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
             ++net->graph_stats[3];
         }
     }
-    if (net->graph_passes < 1) ++net->graph_passes;
+    if (net->graph_passes < GRAPH_AFTER) ++net->graph_passes;
     return launch_steps(net, st, layer_dump);
 }
 

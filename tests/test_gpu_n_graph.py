@@ -1,4 +1,4 @@
-"""GPU parity of repeated forward passes, which go out as one CUDA graph from the second pass on."""
+"""GPU parity of repeated forward passes, which go out as one CUDA graph once a plan has been used often enough."""
 import numpy as np
 import pytest
 import torch
@@ -7,6 +7,8 @@ from paper_2202_05239_b200 import synth
 from gpu_util import api, assert_equal_arrays
 
 pytestmark = pytest.mark.gpu
+
+AFTER = 16         # passes of a plan before its launches are kept as a graph
 
 
 @pytest.mark.parametrize("name,batch,image", [("resnet18", 3, 64), ("resnet50", 1, 96), ("mobilenetv2", 2, 64), ("resnet18_siblings", 2, 64)])
@@ -36,37 +38,82 @@ def test_repeated_passes(ref, name, batch, image):
             counts.append((net.last_launch_count, a.f8_tc_launch_count() - before))
         assert_equal_arrays(o.cpu().numpy(), wants[which])
 
-    for i in range(4):                       # the second and later passes are the graph's; the input changes in place
+    for i in range(AFTER + 3):               # the input changes in place
         check(i & 1)
+        assert net.graph_info["last"] == (i >= AFTER)
+    assert net.graph_info["made"] == 1
     check(1, stream=side)                    # on another stream
+    assert net.graph_info == {"last": 1, "made": 1, "updates": 0, "failed": 0}
     check(0, out=other)                      # another output, then the first one: the same graph with other parameters
+    last = net.graph_info["updates"]         # launches that read the input or write the output
+    assert last > 0
     check(1)
     check(1, out=other)
+    assert net.graph_info == {"last": 1, "made": 1, "updates": 3 * last, "failed": 0}
     first, x = x, torch.empty_like(x)        # ... and another input
     check(0)
+    assert net.graph_info == {"last": 1, "made": 1, "updates": 4 * last, "failed": 0}
     check(1, out=other)
     x = first
-    check(0, dump=[net.layer_output(i, batch) for i in range(len(layers))])
-    check(1)
     check(0)
+    assert net.graph_info["last"] == 1 and net.graph_info["made"] == 1
+    check(0, dump=[net.layer_output(i, batch) for i in range(len(layers))])
+    assert net.graph_info["last"] == 0
+    for i in range(AFTER + 1):               # another plan now
+        check(i & 1)
+    assert net.graph_info["last"] == 1 and net.graph_info["made"] == 2
+    net.set_profiling(True)
+    check(0)
+    assert net.graph_info["last"] == 0
+    net.set_profiling(False)
+    for i in range(AFTER + 1):
+        check(i & 1)
+    assert net.graph_info["last"] == 1 and net.graph_info["made"] == 3
     try:                                     # kernels carry the bound of their waits: a new one means new launches
         a.f8_debug_set_wait_limit_ms(1500.0)
         check(1)
-        check(0)
+        assert net.graph_info["last"] == 0
+        for i in range(AFTER):
+            check(i & 1)
+        assert net.graph_info["last"] == 1 and net.graph_info["made"] == 4
     finally:
         a.f8_debug_set_wait_limit_ms(0.0)
+    for i in range(AFTER + 1):
+        check(i & 1)
+    assert net.graph_info["last"] == 1 and net.graph_info["failed"] == 0
     assert len(set(counts)) == 1
     # inside a caller's capture the launches become the caller's
     g = torch.cuda.CUDAGraph()
     check(1)
     with torch.cuda.graph(g, stream=side):
         net.forward(x, out=out, workspace=ws, stream=torch.cuda.current_stream())
+        assert net.graph_info["last"] == 0
     out.zero_()
     g.replay()
     torch.cuda.synchronize()
     assert_equal_arrays(out.cpu().numpy(), wants[1])
     del g
     check(0)
+    assert net.graph_info["last"] == 1
+    net.close()
+
+
+def test_batches_in_turns_make_no_graph(ref):
+    """A plan that is left before its graph would pay costs what its launches cost."""
+    a = api()
+    layers = synth.make_net("resnet18", 0, image=64)
+    host = synth.draw_image(3, 1, 64, 64)
+    want = ref.net_forward(layers, host, keep_all=False)[-1]
+    net = a.Net(layers, 3)
+    x = a.to_device(host)
+    ws = torch.empty(net.workspace_bytes(3), dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        for n in (1, 3):
+            for _ in range(AFTER):
+                out = net.forward(x[:n], workspace=ws)
+            torch.cuda.synchronize()
+            assert_equal_arrays(out.cpu().numpy(), want[:n])
+    assert net.graph_info["made"] == 0
     net.close()
 
 
@@ -77,8 +124,9 @@ def test_launch_count_behind_a_pass_of_no_images():
     x = a.to_device(synth.draw_image(2, 1, 64, 64))
     out = torch.empty((2,) + net.out_shape, dtype=net.out_dtype, device="cuda")
     ws = torch.empty(net.workspace_bytes(2), dtype=torch.uint8, device="cuda")
-    for _ in range(12):
+    for _ in range(AFTER + 2):
         net.forward(x, out=out, workspace=ws)
+    assert net.graph_info["last"] == 1
     launches = net.last_launch_count
     assert launches > 4
     net.forward(x[:0], out=out[:0], workspace=ws)
