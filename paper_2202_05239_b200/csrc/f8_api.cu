@@ -1308,6 +1308,8 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
         const size_t x_image_bytes = (size_t)net->t_h[0] * net->t_w[0] * net->t_c[0];
         const size_t y_image_bytes = (size_t)net->t_h[nl] * net->t_w[nl] * net->t_c[nl] * net->t_elem[nl];
 
+        SmallPlanPtr next_small;        // for the next layer that takes the kernel for small layers
+
         // Plans layer i for images [img0, img0 + n) of the batch.  Inside a micro-batched run (in_run) tensors that live
         // entirely in the run hold one micro-batch and always start at their base address; all other tensors are
         // addressed at the slice of these images.
@@ -1423,10 +1425,12 @@ f8_status f8_net_forward(f8_net *net, int batch, const void *x, void *y, void *w
                     // planned above
                 } else if ([&]() -> bool {
                                const F8Sibling *sib = stp.has_sib ? &stp.sib : nullptr;
-                               if ((g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) || !f8_small_tc_wanted(stp.g, is_bits8(L.q, sib))) return false;
-                               SmallPlanPtr sp = alloc_small_plan();
-                               if (!sp || f8_small_plan_init(sp.get(), stp.g, L.q, stp.x, L.w, L.b, stp.res, stp.y, sib, i + 1) != cudaSuccess) return false;
-                               stp.splan = std::move(sp);
+                               if (g_plan_off & F8_PLAN_OFF_SMALL_KERNEL) return false;
+                               if (!next_small) next_small = alloc_small_plan();
+                               if (!next_small || f8_small_plan_init(next_small.get(), stp.g, L.q, is_bits8(L.q, sib), stp.x, L.w, L.b, stp.res, stp.y,
+                                                                     sib, i + 1) != cudaSuccess)
+                                   return false;
+                               stp.splan = std::move(next_small);
                                return true;
                            }()) {
                     stp.use_tc = true;

@@ -146,8 +146,9 @@ cudaError_t f8_launch_stem_tc(const F8ConvGeom &g, const F8Requant &q, int kh2, 
 bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8);
 struct F8SmallPlan;
 size_t f8_small_plan_size();
-cudaError_t f8_small_plan_init(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
-                               const void *res, void *y, const F8Sibling *sib, int tag);
+// A layer of a network: plans where it is wanted, else cudaErrorNotSupported.
+cudaError_t f8_small_plan_init(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q, bool bits8, const void *x, const int8_t *w,
+                               const int32_t *bias, const void *res, void *y, const F8Sibling *sib, int tag);
 cudaError_t f8_small_launch(const F8SmallPlan *plan, bool overlap_previous, cudaStream_t st);
 // A single-layer call: launches where this kernel is the better one, else cudaErrorNotSupported.
 cudaError_t f8_launch_small_alone(const F8ConvGeom &g, const F8Requant &q, bool bits8, const void *x, const int8_t *w, const int32_t *bias,

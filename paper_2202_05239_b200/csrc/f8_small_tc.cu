@@ -496,33 +496,53 @@ struct Split {
 };
 
 // Input pixels that a tile of bm output pixels reads at most.
-long long window_pixels(const F8ConvGeom &g, int bm) {
+int window_pixels(const F8ConvGeom &g, int bm) {
     if (g.kh == 1 && g.kw == 1 && g.pad_h == 0) return bm;                // (rows past the last pixel are read, and their sums dropped)
     // output rows it touches, then input rows: the rows between two images count where a filter does not reach the last ones
-    long long rows = bm % g.wo == 0 ? bm / g.wo : (g.wo % bm == 0 ? 1 : (bm + g.wo - 2) / g.wo + 1);
-    rows = std::min(rows, (long long)g.n * g.ho);
-    const long long seams = (rows + g.ho - 2) / g.ho, skipped = std::max(0, g.h - g.ho * g.stride_h);
-    return std::min((rows - 1) * g.stride_h + g.kh + seams * skipped, (long long)g.n * g.h) * g.w;
+    const int span = (bm - 1) / g.wo;
+    int rows = bm == (span + 1) * g.wo ? span + 1 : (bm < g.wo && g.wo % bm == 0 ? 1 : (bm + g.wo - 2) / g.wo + 1);
+    rows = std::min(rows, g.n * g.ho);
+    const int skipped = g.h - g.ho * g.stride_h, seams = skipped > 0 ? (rows + g.ho - 2) / g.ho * skipped : 0;
+    return std::min((rows - 1) * g.stride_h + g.kh + seams, g.n * g.h) * g.w;
 }
 
 // Cuts a layer so that it is done soonest after its input is (an estimate in cycles, fitted to the layers of the networks at batches 1 - 32).
-// A call of its own pays for this search: single precision, and no warp tiles of 32 x 32 where 16 x 16 ones leave SMs idle.
-bool pick_split(const F8ConvGeom &g, Split *best) {
-    const long long M = (long long)g.n * g.ho * g.wo;
+// Every plan of a layer and every call of its own pays for this search: single precision, no warp tiles of 32 x 32 where 16 x 16 ones
+// leave SMs idle, and no search for panels in a split whose least time, with all SMs to itself, is above the best one's or the limit.
+bool pick_split(const F8ConvGeom &g, Split *best, float limit = 1e30f) {
+    const int M = g.n * g.ho * g.wo;                                      // (below 2^24)
     const int c16 = g.c / 16, taps = g.kh * g.kw, c_out = g.c_out;
     const float k = (float)taps * g.c;
     const int k_steps = (taps * c16 + 1) / 2;
-    const int t_end = (M + 15) / 16 * ((c_out + 15) / 16) < 148 ? 16 : 32;
-    best->cycles = 1e30f;
+    const int t_end = (long long)((M + 15) / 16) * ((c_out + 15) / 16) < 148 ? 16 : 32;
+    best->cycles = limit;
+    best->tiles = 0;
     for (int t = 16; t <= t_end; t += 16)
         for (int wm_shift = 0; wm_shift <= 3; ++wm_shift) {
-            const int bm = t << wm_shift;
+            const int t_shift = t == 16 ? 4 : 5, bm = t << wm_shift;
             if (wm_shift && bm / 2 >= M) break;
-            const long long px = window_pixels(g, bm), m_tiles = (M + bm - 1) / bm;
+            const int px = window_pixels(g, bm), m_tiles = (M + bm - 1) >> (t_shift + wm_shift);
             for (int wn_shift = 0; wn_shift + wm_shift <= 3; ++wn_shift) {
                 const int wk = 3 - wm_shift - wn_shift, bn = t << wn_shift;
                 if (wn_shift && bn / 2 >= c_out) break;
                 const size_t red = ((size_t)bm << wk) * (bn + 8) * 4;
+                const long long tiles = (long long)m_tiles * ((c_out + bn - 1) >> (t_shift + wn_shift));
+                const float steps = (float)((k_steps + (1 << wk) - 1) >> wk);
+                // (a block's own instructions, about 500 a warp, where an SM runs several)
+                const float issue = 700.f * std::max(0.f, (float)tiles / 148 - 1);
+                struct Parts { float fetch, fetch_w, mul, finish; };
+                auto parts = [&](float at_once) {
+                    Parts e;
+                    e.mul = std::max(steps * (t == 16 ? 45.f : 75.f), at_once * bm * bn * k * (t == 16 ? 1 / 900.f : 1 / 1800.f));
+                    e.finish = 350 + 100 * ((bm * bn + 1023) / 1024) + at_once * red / 64;
+                    e.fetch = at_once * px * g.c / 45;
+                    e.fetch_w = at_once * bn * k / 45;
+                    return e;
+                };
+                {
+                    const Parts e = parts(1.f);
+                    if (700 + 0.f + issue + e.fetch + e.mul + e.finish >= best->cycles) continue;
+                }
                 int at16 = 0, ahead = 2;
                 size_t window = 0, weights = 0, smem = 0;
                 // one panel where it fits, else two stages in half of the shared memory; the smallest panel may take all of it
@@ -542,23 +562,18 @@ bool pick_split(const F8ConvGeom &g, Split *best) {
                 }
                 if (!at16) continue;
                 const int panels = (c16 + at16 - 1) / at16;
-                const long long tiles = m_tiles * ((c_out + bn - 1) / bn);
                 const int occ = std::min(t == 16 ? 3 : 2, (int)(SM_SMEM / smem));
                 const float at_once = (float)std::min<long long>(occ, (tiles + 147) / 148), rounds = (float)((tiles + 148 * occ - 1) / (148 * occ));
-                const float steps = (float)((k_steps + (1 << wk) - 1) >> wk);
-                const float mul = std::max(steps * (t == 16 ? 45.f : 75.f), at_once * bm * bn * k * (t == 16 ? 1 / 900.f : 1 / 1800.f));
-                const float finish = 350 + 100 * ((bm * bn + 1023) / 1024) + at_once * red / 64;
-                const float fetch = at_once * px * g.c / 45, fetch_w = at_once * bn * k / 45;
-                // (a block's own instructions, about 500 a warp, where an SM runs several)
-                const float issue = 700.f * std::max(0.f, (float)tiles / 148 - 1);
+                const Parts e = parts(at_once);
                 // (no room for the next layer's block: its start is not hidden)
                 const float alone = occ == 1 ? 600.f : 0.f;
-                const float cycles = 700 + alone + issue + fetch + mul + finish + (panels - 1) * 300.f + std::max(0, panels - ahead) * (ahead == 2 ? fetch_w : 2 * (fetch + fetch_w)) / panels +
-                                     (rounds - 1) * (1500 + fetch + fetch_w + mul + finish);
+                const float cycles = 700 + alone + issue + e.fetch + e.mul + e.finish + (panels - 1) * 300.f +
+                                     std::max(0, panels - ahead) * (ahead == 2 ? e.fetch_w : 2 * (e.fetch + e.fetch_w)) / panels +
+                                     (rounds - 1) * (1500 + e.fetch + e.fetch_w + e.mul + e.finish);
                 if (cycles < best->cycles) *best = {t, 1 << wm_shift, 1 << wn_shift, wk, at16, panels, ahead, window, weights, smem, tiles, cycles};
             }
         }
-    return best->cycles < 1e29f;
+    return best->tiles > 0;
 }
 
 template <int MT, int NT, bool XS, bool PW>
@@ -623,16 +638,20 @@ static double cuda_core_us(const F8ConvGeom &g, const Split &s) {
     return s.ahead == 1 ? 2.0 + 0.0177 * g.c * std::min(g.kh, g.h) * std::min(g.kw, g.w) : 1e9;
 }
 
-bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8) {
-    Split s;
+// Whether a network takes this kernel for the layer, and how it is cut then.
+static bool wanted(const F8ConvGeom &g, bool bits8, Split *s) {
     if (!shape_ok(g)) return false;
-    if (!f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c)) return pick_split(g, &s) && small_us(s) < cuda_core_us(g, s);
+    if (!f8_tc_supported(g, (size_t)g.n * g.h * g.w * g.c)) return pick_split(g, s) && small_us(*s) < cuda_core_us(g, *s);
     // what every split takes at least (products at the rate of mma.sync, blocks of at most 8192 outputs): spares large layers the search
     const double out = (double)g.n * g.ho * g.wo * g.c_out, other = 0.97 * tcgen05_us(g, bits8);
-    s.panels = 1;
-    s.cycles = (float)(700 + out * g.kh * g.kw * g.c / (148 * 1800.0) + 700 * std::max(0.0, out / (8192 * 148.0) - 1));
-    if (small_us(s) >= other) return false;
-    return pick_split(g, &s) && s.panels == 1 && small_us(s) < other;
+    const double least = 700 + out * g.kh * g.kw * g.c / (148 * 1800.0) + 700 * std::max(0.0, out / (8192 * 148.0) - 1), limit = (other - 0.9) * (1900 / 1.75);
+    if (least >= limit) return false;
+    return pick_split(g, s, (float)limit * 1.0001f) && s->panels == 1 && small_us(*s) < other;
+}
+
+bool f8_small_tc_wanted(const F8ConvGeom &g, bool bits8) {
+    Split s;
+    return wanted(g, bits8, &s);
 }
 
 struct F8SmallPlan {
@@ -698,9 +717,9 @@ static void fill_plan(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q
     if (sib) p.sib = *sib;
 }
 
-cudaError_t f8_small_plan_init(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q, const void *x, const int8_t *w, const int32_t *bias,
-                               const void *res, void *y, const F8Sibling *sib, int tag) {
-    if (!shape_ok(g) || !pick_split(g, &plan->s)) return cudaErrorNotSupported;
+cudaError_t f8_small_plan_init(F8SmallPlan *plan, const F8ConvGeom &g, const F8Requant &q, bool bits8, const void *x, const int8_t *w,
+                               const int32_t *bias, const void *res, void *y, const F8Sibling *sib, int tag) {
+    if (!wanted(g, bits8, &plan->s)) return cudaErrorNotSupported;
     fill_plan(plan, g, q, x, w, bias, res, y, sib, tag, false);
     return cudaSuccess;
 }
