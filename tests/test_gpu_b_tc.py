@@ -287,3 +287,40 @@ def test_narrow_tiles_in_a_network(ref, case):
         assert plan["m_tiles"] * plan["n_tiles"] <= torch.cuda.get_device_properties(0).multi_processor_count, plan
     assert np.array_equal(out.cpu().numpy(), ref.run_layer(layer, x))
     net.close()
+
+
+# The same with a shortcut of 8 bits, whose ring makes 64-byte chunks of K and 256-wide tiles the usual form of pointwise layers
+# (h, c, c_out, k, n, x_signed, y_dtype, columns of a tile, bytes of a chunk)
+NARROW_RESIDUAL_CASES = [
+    (14, 128, 512, 1, 8, False, synth.U8, 64, 128),      # 13 M tiles: 104 of 64 columns, back to whole chunks
+    (14, 192, 256, 1, 20, True, synth.S8, 64, 128),      # 31: 124 of 64
+    (14, 256, 512, 1, 24, False, synth.S8, 128, 128),    # 37: 148 of 128, one for every SM
+    (14, 256, 1024, 1, 24, False, synth.U8, 256, 64),    # 37: 148 of 256 already
+    (14, 96, 192, 1, 10, False, synth.U8, 256, 64),      # less than one 128-byte chunk of K
+    (14, 256, 256, 3, 16, False, synth.U8, 64, 128),     # 25 tiles of a layer that has 256-wide tiles and CTA pairs elsewhere
+    (14, 256, 256, 3, 33, True, synth.S8, 128, 128),
+    (7, 64, 512, 3, 18, False, synth.U8, 64, 64),        # whole rows of one image per tile
+]
+
+
+@pytest.mark.parametrize("case", range(len(NARROW_RESIDUAL_CASES)))
+def test_narrow_tiles_with_a_shortcut_in_a_network(ref, case):
+    from paper_2202_05239_b200 import api as a
+    h, c, c_out, k, n, xs, y_dtype, bn, kb = NARROW_RESIDUAL_CASES[case]
+    rng = np.random.default_rng(1800 + case)
+    layer = random_conv_layer(rng, h=h, w=h, c=c, c_out=c_out, k=k, stride=1, pad=k // 2, x_signed=xs, y_dtype=y_dtype, with_res=True)
+    short = random_conv_layer(rng, h=h, w=h, c=c, c_out=c_out, k=k, stride=1, pad=k // 2, x_signed=xs, y_dtype=layer.r_dtype, with_res=False,
+                              fl_x=layer.fl_x)
+    short.fl_y = layer.fl_r
+    x = random_input(rng, n, layer)
+    a.f8_debug_plan_options(a.PLAN_OFF_SMALL_KERNEL)
+    try:
+        net = a.Net([short, layer], n)
+        out = net.forward(a.to_device(x))
+        torch.cuda.synchronize()
+        plan = a.f8_debug_last_plan()
+    finally:
+        a.f8_debug_plan_options(0)
+    assert (plan["bn"], plan["kb"]) == (bn, kb), plan
+    assert np.array_equal(out.cpu().numpy(), ref.net_forward([short, layer], x)[-1])
+    net.close()
